@@ -41,6 +41,7 @@ struct la_ctx {
   double* d_sigma[LA_MAX_LEVELS] = {};
   // complex64 path: the Galerkin stencils rounded to float once, as its kernels use them
   float* d_sigma32[LA_MAX_LEVELS] = {};
+  double* d_gtab[2] = {};           // 1D Galerkin tables of two successive levels (la_set_hamiltonian)
   double* d_partials = nullptr;
   double* d_N = nullptr;
   int* d_status = nullptr;
@@ -402,6 +403,8 @@ extern "C" la_status la_init(const la_config* cfg, void* stream, la_ctx** out) {
       if (k.precision == 1) ALLOC(c->d_sigma32[l], sizeof(float) * (size_t)G.np * LA_NPAIR * box5_count(k.dim));
     }
   }
+  if (c->L > 1)
+    for (int j = 0; j < 2; ++j) ALLOC(c->d_gtab[j], sizeof(double) * (size_t)galerkin_table_doubles(c->geo[1].n));
   c->nparts = norm_blocks(c->np0);
   ALLOC(c->d_partials, sizeof(double) * c->nparts);
   ALLOC(c->d_N, sizeof(double) * 2);
@@ -586,11 +589,8 @@ extern "C" la_status la_set_hamiltonian(la_ctx* c, const double* V0, const la_pu
   LA_TRY(load_any(c, c->d_V0, V0, sizeof(double) * c->np0));
   LA_CUDA(c, cudaMemcpyAsync(c->d_tm, &c->htm, sizeof(TimeMats), cudaMemcpyHostToDevice, c->stream));
   // Galerkin spatial factors of every coarse level (static)
-  for (int l = 1; l < c->L; ++l) {
-    if (l == 1) launch_galerkin_from_fine(c->fine, c->geo[1], c->d_sigma[1], c->stream);
-    else launch_galerkin_coarse(c->geo[l - 1], c->d_sigma[l - 1], c->geo[l], c->d_sigma[l], c->stream);
-    LA_CHECK_LAUNCH(c);
-  }
+  launch_galerkin(c->fine, c->geo, c->L, c->d_sigma, c->d_gtab[0], c->d_gtab[1], c->stream);
+  LA_CHECK_LAUNCH(c);
   // the complex64 kernels read the stencils as float: round them once here, which halves the bytes
   // every Galerkin-level sweep, residual and factorisation streams and changes no result
   if (c->cfg.precision == 1) {

@@ -384,9 +384,10 @@ void launch_loop_cond(LoopState* st, const double* Nnew, double tol, int max_cyc
                       cudaGraphConditionalHandle h, cudaStream_t s);
 void launch_loop_record(const LoopState* st, LoopRecord* rec, cudaStream_t s);
 // Galerkin coarse stencils
-void launch_galerkin_from_fine(const FineOp& g, const LevelGeom& coarse, double* sigma_c, cudaStream_t s);
-void launch_galerkin_coarse(const LevelGeom& fine, const double* sigma_f, const LevelGeom& coarse, double* sigma_c,
-                            cudaStream_t s);
+// builds sigma[1] .. sigma[levels - 1]; tab0, tab1: scratch of galerkin_table_doubles(geo[1].n) doubles each
+long long galerkin_table_doubles(const int n[3]);
+void launch_galerkin(const FineOp& g, const LevelGeom* geo, int levels, double* const* sigma, double* tab0,
+                     double* tab1, cudaStream_t s);
 // subvolume factorisation and sweeps (dispatch over the padded subvolume size)
 template <typename R>
 cudaError_t launch_factor(const LevelGeom& L, const FineOp* fine, const R* sigma, const TimeMats* tm,
