@@ -979,6 +979,44 @@ __device__ __forceinline__ void wide_column_step(int J, int band, int n, const F
   __syncthreads();
 }
 
+// Fills the shared-memory tables of the wide assembly for the subvolume with origin o and extent e; all
+// threads of the CTA, synchronised on return.
+template <typename R>
+__device__ __forceinline__ void wide_tables(const LevelGeom& L, const FineOp& g, const TimeMats* __restrict__ tm,
+                                            const int o[3], const int e[3], R* sP, R* sPd, R* sD, R* sX, R* sN,
+                                            int* sXYZ, typename C2<R>::T* sHH) {
+  typedef typename C2<R>::T CT;
+  const int tid = threadIdx.x, nthr = blockDim.x, K = tm->K, KK = K * K, npts = e[0] * e[1] * e[2];
+  for (int i = tid; i < LA_NPAIR * KK; i += nthr) sP[i] = (R)tm->P[i / KK][i % KK];
+  const R wx = (R)(0.5 * g.ih2[0]), wy = (R)(0.5 * g.ih2[1]), wz = (R)(0.5 * g.ih2[2]);
+  for (int i = tid; i < npts; i += nthr) {
+    int lx, ly, lz;
+    local_coords(i, e, lx, ly, lz);
+    const int px = o[0] + lx, py = o[1] + ly, pz = o[2] + lz;
+    sD[i] = (R)(g.dsum + g.V0[(pz * g.n[1] + py) * g.n[0] + px]);
+    sX[i] = (R)fine_x(g, px, py, pz);
+    // unused axes have n = 1 and w = 0
+    const int cx = (px > 0 ? 1 : 0) + (px + 1 < g.n[0] ? 1 : 0), cy = (py > 0 ? 1 : 0) + (py + 1 < g.n[1] ? 1 : 0),
+              cz = (pz > 0 ? 1 : 0) + (pz + 1 < g.n[2] ? 1 : 0);
+    sN[i] = wx * wx * (R)cx + wy * wy * (R)cy + wz * wz * (R)cz;
+    sXYZ[i] = lx | (ly << 8) | (lz << 16);
+  }
+  __syncthreads();
+  for (int p = tid; p < npts * npts; p += nthr) {
+    const int i = p / npts, j = p - i * npts;
+    const int pi = sXYZ[i], pj = sXYZ[j];
+    const int dx = (pj & 255) - (pi & 255), dy = ((pj >> 8) & 255) - ((pi >> 8) & 255), dz = (pj >> 16) - (pi >> 16);
+    R H, H2;
+    wide_h_h2<R>(dx, dy, dz, sD[i], sD[j], sN[i], wx, wy, wz, H, H2);
+    sHH[i * kHHStride + j] = mkc<CT>(H, H2);
+  }
+  for (int i = tid; i < KK; i += nthr) {
+    sPd[i] = sP[1 * KK + i] - sP[3 * KK + i];
+    sPd[KK + i] = sP[2 * KK + i] - sP[6 * KK + i];
+  }
+  __syncthreads();
+}
+
 template <typename R, int NPAD>
 __global__ void __launch_bounds__(kFactorThreads, sizeof(R) == 4 ? 2 : 1)
 k_factor_wide(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C2<R>::T* __restrict__ factors,
@@ -1007,34 +1045,7 @@ k_factor_wide(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C
   subvol_box(L, b, o, e);
   const int npts = e[0] * e[1] * e[2], n = npts * K;
   CT* F = factors + (size_t)b * L.fsize;
-  for (int i = tid; i < LA_NPAIR * KK; i += kFactorThreads) S.sP[i] = (R)tm->P[i / KK][i % KK];
-  const R wx = (R)(0.5 * g.ih2[0]), wy = (R)(0.5 * g.ih2[1]), wz = (R)(0.5 * g.ih2[2]);
-  for (int i = tid; i < npts; i += kFactorThreads) {
-    int lx, ly, lz;
-    local_coords(i, e, lx, ly, lz);
-    const int px = o[0] + lx, py = o[1] + ly, pz = o[2] + lz;
-    S.sD[i] = (R)(g.dsum + g.V0[(pz * g.n[1] + py) * g.n[0] + px]);
-    S.sX[i] = (R)fine_x(g, px, py, pz);
-    // unused axes have n = 1 and w = 0
-    const int cx = (px > 0 ? 1 : 0) + (px + 1 < g.n[0] ? 1 : 0), cy = (py > 0 ? 1 : 0) + (py + 1 < g.n[1] ? 1 : 0),
-              cz = (pz > 0 ? 1 : 0) + (pz + 1 < g.n[2] ? 1 : 0);
-    S.sN[i] = wx * wx * (R)cx + wy * wy * (R)cy + wz * wz * (R)cz;
-    S.sXYZ[i] = lx | (ly << 8) | (lz << 16);
-  }
-  __syncthreads();
-  for (int p = tid; p < npts * npts; p += kFactorThreads) {
-    const int i = p / npts, j = p - i * npts;
-    const int pi = S.sXYZ[i], pj = S.sXYZ[j];
-    const int dx = (pj & 255) - (pi & 255), dy = ((pj >> 8) & 255) - ((pi >> 8) & 255), dz = (pj >> 16) - (pi >> 16);
-    R H, H2;
-    wide_h_h2<R>(dx, dy, dz, S.sD[i], S.sD[j], S.sN[i], wx, wy, wz, H, H2);
-    S.sHH[i * kHHStride + j] = mkc<CT>(H, H2);
-  }
-  for (int i = tid; i < KK; i += kFactorThreads) {
-    S.sPd[i] = S.sP[1 * KK + i] - S.sP[3 * KK + i];
-    S.sPd[KK + i] = S.sP[2 * KK + i] - S.sP[6 * KK + i];
-  }
-  __syncthreads();
+  wide_tables<R>(L, g, tm, o, e, S.sP, S.sPd, S.sD, S.sX, S.sN, S.sXYZ, S.sHH);
   const FastDiv dK = L.fd_K;
   const WideTables<R> T = S.tables();
   // block column 0: assembled only, one row per thread
@@ -1058,6 +1069,267 @@ k_factor_wide(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C
       case 4: wide_column_step<R, NPAD, 4>(J, L.band, n, dK, K, F, S, status); break;
       default: wide_column_step<R, NPAD, 2>(J, L.band, n, dK, K, F, S, status); break;
     }
+  }
+}
+
+// ------------------------------------------------------------------------ banded, window in registers
+// Wide complex64 factors whose block band is at most W: blocked right-looking Cholesky with the active
+// window in registers.  While block column J is eliminated, the trailing blocks (J + i, J + j),
+// 1 <= j <= i <= W, are the only ones that change (no fill outside the envelope), so thread (ti, tk) keeps
+// its entry (ti, tk) of each of them in registers and the window moves one block along the diagonal per
+// column; a new block row is assembled as it enters.  Per column, three barriers:
+//   panel   L_i = A_i inv(L_JJ)^dagger for the W blocks below the diagonal, to the factor store and,
+//           k-major, to shared memory;
+//   column  the blocks (i, 1) take the rank-16 update first and go to shared memory as the next column;
+//   rest    a ninth warp factorises and inverts the next diagonal block (lookahead) while the others apply
+//           the rank-16 update to the remaining blocks and assemble the row that enters.
+// The factor is written once and never read back.
+// 96^3, K = 4, 4x4x4 subvolumes (13,824 factors of 256 unknowns, W = 8): 6.88 ms = 25 TFLOP/s of banded flops,
+// bound by instruction issue (67% of the slots, 46% of the FMA pipe); 11.1 ms with the left-looking
+// factorisation below, which waits on its own earlier blocks in L2 and on a diagonal step three times
+// as long.  A diagonal step by one of the eight warps instead of a ninth: 9.6 ms.
+template <int W> struct BandSmem {
+  // the panel and the inverse hold two columns k, k + 1 of a row next to each other, one 16-byte load for
+  // both; rows of a panel pair: one more than the window, so that the transposed stores spread over the banks
+  static constexpr int kPanStride = 2 * (LA_BLK * W + 1);
+  // complex entries: column blocks, inverse, two row buffers of the diagonal step, panel, the blocks (i, 1)
+  static constexpr int kComplex = (W + 1) * LA_BLK * kRowStride + 256 + 32 + LA_BLK / 2 * kPanStride + 256 * W;
+};
+template <typename R, int W>
+__host__ __device__ constexpr size_t band_factor_smem() {
+  return 2 * sizeof(R) * ((size_t)BandSmem<W>::kComplex + (size_t)kWidePtsMax * kHHStride) +
+         sizeof(R) * (LA_NPAIR * LA_KMAX * LA_KMAX + 3 * kWidePtsMax + 2 * LA_KMAX * LA_KMAX) +
+         sizeof(int) * kWidePtsMax;
+}
+
+// Cholesky factor and inverse of the 16 x 16 block D (row stride kRowStride) by one warp, in place: step j
+// scales column j to L and frees it, and the inverse X of L fills the freed columns, so lane (r, h) =
+// (lane % 16, lane / 16) holds one value per column of parity h of row r, A[r][c] for c > j and X[r][c] for
+// c <= j, and every step updates the rows r > j by v[c] -= L_rj w[c] with the row w[c] = conj(L_cj) for
+// c > j, X[j][c] for c <= j (passed through shared memory, read as 16-byte pairs).  Ends with X = inv(L).
+template <typename CT>
+__device__ __forceinline__ void band_diag(const CT* D, CT* sInvT, CT* buf, CT* Fdiag, int* status) {
+  typedef typename Re<CT>::T R;
+  const int lane = threadIdx.x & 31, r = lane & 15, h = lane >> 4;
+  CT v[LA_BLK / 2];   // column 2 u + h
+#pragma unroll
+  for (int u = 0; u < LA_BLK / 2; ++u) v[u] = D[r * kRowStride + 2 * u + h];
+#pragma unroll
+  for (int j = 0; j < LA_BLK; ++j) {
+    const int uj = j >> 1, hj = j & 1;
+    CT l;
+    l.x = __shfl_sync(0xffffffffu, v[uj].x, r + 16 * hj);
+    l.y = __shfl_sync(0xffffffffu, v[uj].y, r + 16 * hj);
+    R d2 = __shfl_sync(0xffffffffu, v[uj].x, j + 16 * hj);
+    if (!(d2 > (R)0)) {
+      if (lane == 0) atomicOr(status, 1);
+      d2 = (R)1;
+    }
+    const R inv = rsq(d2);
+    l = r > j ? mkc<CT>(l.x * inv, l.y * inv) : mkc<CT>((R)0, (R)0);
+    if (h == hj) v[uj] = mkc<CT>((R)(r == j ? 1 : 0), (R)0);   // column j now belongs to X
+    CT* b = buf + (j & 1) * 16;   // [parity][8] columns
+    if (r > j && h == 0) b[(r & 1) * 8 + (r >> 1)] = mkc<CT>(l.x, -l.y);
+    if (r == j) {
+#pragma unroll
+      for (int u = 0; 2 * u <= j; ++u) {
+        if (2 * u + h > j) continue;
+        v[u] = mkc<CT>(v[u].x * inv, v[u].y * inv);
+        b[h * 8 + u] = v[u];
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < LA_BLK / 2; u += 2) {
+      const CPair<CT> p = lds_pair(b + h * 8 + u);
+      const CT w0 = p.a(), w1 = p.b();
+      CT &t0 = v[u], &t1 = v[u + 1];
+      t0.x = fma(-l.x, w0.x, t0.x); t0.x = fma(l.y, w0.y, t0.x);
+      t0.y = fma(-l.x, w0.y, t0.y); t0.y = fma(-l.y, w0.x, t0.y);
+      t1.x = fma(-l.x, w1.x, t1.x); t1.x = fma(l.y, w1.y, t1.x);
+      t1.y = fma(-l.x, w1.y, t1.y); t1.y = fma(-l.y, w1.x, t1.y);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < LA_BLK / 2; ++u) {
+    const int c = 2 * u + h;
+    if (c > r) v[u] = mkc<CT>((R)0, (R)0);
+    Fdiag[r * LA_BLK + c] = v[u];
+    sInvT[(c >> 1) * 32 + 2 * r + (c & 1)] = mkc<CT>(v[u].x, -v[u].y);
+  }
+}
+
+// v -= x conj(y)
+template <typename CT>
+__device__ __forceinline__ void band_fma(CT& v, const CT x, const CT y) {
+  v.x = fma(-x.x, y.x, v.x); v.x = fma(-x.y, y.y, v.x);
+  v.y = fma(-x.y, y.x, v.y); v.y = fma(x.x, y.y, v.y);
+}
+// Rank-16 update of the window blocks (i, j), I0 <= i <= I1, 2 <= j <= i: a(i, j) -= L_i L_j^dagger.
+// a(i, j) is at (i - 2) (i - 1) / 2 + j - 2.
+template <typename CT, int W, int I0, int I1>
+__device__ __forceinline__ void band_update(CT (&a)[W * (W - 1) / 2], const CT* pan, int ti, int tk) {
+#pragma unroll 1
+  for (int k2 = 0; k2 < LA_BLK / 2; ++k2) {
+    const CT* p = pan + k2 * BandSmem<W>::kPanStride;
+    CPair<CT> x[I1 - I0 + 1];
+#pragma unroll
+    for (int i = I0; i <= I1; ++i) x[i - I0] = lds_pair(p + 2 * (LA_BLK * (i - 1) + ti));
+#pragma unroll
+    for (int j = 2; j <= I1; ++j) {
+      const CPair<CT> y = lds_pair(p + 2 * (LA_BLK * (j - 1) + tk));
+#pragma unroll
+      for (int i = I0; i <= I1; ++i)
+        if (j <= i) {
+          CT& v = a[(i - 2) * (i - 1) / 2 + j - 2];
+          band_fma(v, x[i - I0].a(), y.a());
+          band_fma(v, x[i - I0].b(), y.b());
+        }
+    }
+  }
+}
+
+constexpr int kBandThreads = kFactorThreads + 32;
+__device__ __forceinline__ void band_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
+template <typename R, int NPAD, int W>
+__global__ void __launch_bounds__(kBandThreads, 2)
+k_factor_band(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C2<R>::T* __restrict__ factors,
+              int* __restrict__ status) {
+  typedef typename C2<R>::T CT;
+  static_assert(W % 4 == 0, "window rows are updated in groups of four");
+  constexpr int NB = NPAD / LA_BLK, S = BandSmem<W>::kPanStride;
+  extern __shared__ __align__(16) unsigned char smem[];
+  CT* sA = reinterpret_cast<CT*>(smem);              // [(W + 1) * 16][18] the column's blocks, diagonal first
+  CT* sInvT = sA + (W + 1) * LA_BLK * kRowStride;   // inv(L_JJ)^dagger, [k / 2][c][k % 2]
+  CT* sBuf = sInvT + 256;                            // [2][16] rows of the diagonal step
+  CT* sPan = sBuf + 32;                              // [8][S] the panel, [k / 2][row][k % 2]
+  CT* sB = sPan + LA_BLK / 2 * S;                        // [W][256] the blocks (i, 1), each thread its own entries
+  CT* sHH = sB + 256 * W;                            // [64][65] (H, H^2) of the point pairs
+  R* sP = reinterpret_cast<R*>(sHH + kWidePtsMax * kHHStride);
+  R* sPd = sP + LA_NPAIR * LA_KMAX * LA_KMAX;
+  R* sD = sPd + 2 * LA_KMAX * LA_KMAX;
+  R* sX = sD + kWidePtsMax;
+  R* sN = sX + kWidePtsMax;
+  int* sXYZ = reinterpret_cast<int*>(sN + kWidePtsMax);
+
+  const int tid = threadIdx.x, ti = tid >> 4, tk = tid & 15;
+  const int K = tm->K, KK = K * K, band = L.band;
+  int o[3], e[3];
+  subvol_box(L, blockIdx.x, o, e);
+  const int npts = e[0] * e[1] * e[2], n = npts * K;
+  CT* F = factors + (size_t)blockIdx.x * L.fsize;
+  wide_tables<R>(L, g, tm, o, e, sP, sPd, sD, sX, sN, sXYZ, sHH);
+  const FastDiv dK = L.fd_K;
+  const WideTables<R> T{sHH, sP, sPd, sX};
+  // entry (ti, tk) of block (I, J) of G_UU; where K divides 16 its time functions do not depend on the block
+  const bool kdiv = (LA_BLK % K) == 0;
+  const int ppb = LA_BLK / K, pr = fdiv(ti, dK), pc = fdiv(tk, dK), mn = (ti - pr * K) * K + (tk - pc * K);
+  auto entry = [&](int I, int J) {
+    if (!kdiv) return wide_entry<R>(wide_row<R>(LA_BLK * I + ti, dK, K, sX), LA_BLK * J + tk, n, dK, K, T);
+    const int i = I * ppb + pr, j = J * ppb + pc;
+    if (i >= npts || j >= npts) return mkc<CT>((R)(I == J && ti == tk ? 1 : 0), (R)0);
+    const CT hh = sHH[i * kHHStride + j];
+    const R xp = sX[i], xq = sX[j];
+    R re = hh.y * sP[4 * KK + mn] + hh.x * (xq * sP[5 * KK + mn] + xp * sP[7 * KK + mn]);
+    R im = hh.x * sPd[mn];
+    if (i == j) {
+      re += sP[mn] + xp * xp * sP[8 * KK + mn];
+      im += xp * sPd[KK + mn];
+    }
+    return mkc<CT>(re, im);
+  };
+  if (tid >= kFactorThreads) {   // the diagonal warp
+    for (int J = 0; J < NB; ++J) {
+      __syncthreads();   // column J is in sA
+      band_diag<CT>(sA, sInvT, sBuf, F + (size_t)tri_index(J, J) * 256, status);
+      __syncthreads();
+    }
+    return;
+  }
+#pragma unroll 1
+  for (int i = 0; i <= W && i < NB; ++i) sA[(LA_BLK * i + ti) * kRowStride + tk] = entry(i, 0);
+  __syncthreads();
+#pragma unroll 1
+  for (int i = 1; i <= W && i < NB; ++i) sB[(i - 1) * 256 + tid] = entry(i, 1);
+  CT a[W * (W - 1) / 2];   // a(i, j) = block (J + i, J + j), 2 <= j <= i
+#pragma unroll
+  for (int i = 2; i <= W; ++i)
+#pragma unroll
+    for (int j = 2; j <= i; ++j) a[(i - 2) * (i - 1) / 2 + j - 2] = entry(i, j);
+  __syncthreads();
+#pragma unroll 1
+  for (int J = 0; J < NB; ++J) {
+    const int we = NB - 1 - J < W ? NB - 1 - J : W;   // blocks below the diagonal
+    // panel, four blocks at a time
+#pragma unroll 1
+    for (int i0 = 1; i0 <= we; i0 += 4) {
+      CT l[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) l[u] = mkc<CT>(0, 0);
+      const CT* ar = sA + (LA_BLK * i0 + ti) * kRowStride;
+#pragma unroll 2
+      for (int k = 0; k < LA_BLK; k += 2) {
+        const CPair<CT> iv = lds_pair(sInvT + k * LA_BLK + 2 * tk);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const CPair<CT> ap = lds_pair(ar + u * LA_BLK * kRowStride + k);
+          cfma(l[u], ap.a(), iv.a());
+          cfma(l[u], ap.b(), iv.b());
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u;
+        if (i > we) break;
+        sPan[(tk >> 1) * S + 2 * (LA_BLK * (i - 1) + ti) + (tk & 1)] = l[u];
+        if (i <= band) F[(size_t)tri_index(J + i, J) * 256 + tid] = l[u];
+      }
+    }
+    if (we == 0) break;
+    band_bar();
+    // next column: the blocks (i, 1), updated first, and the block that enters the band
+#pragma unroll 1
+    for (int i0 = 1; i0 <= we; i0 += 4) {
+      CT v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = sB[(i0 - 1 + u) * 256 + tid];
+#pragma unroll 2
+      for (int k2 = 0; k2 < LA_BLK / 2; ++k2) {
+        const CT* p = sPan + k2 * S;
+        const CPair<CT> y = lds_pair(p + 2 * tk);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const CPair<CT> x = lds_pair(p + 2 * (LA_BLK * (i0 - 1 + u) + ti));
+          band_fma(v[u], x.a(), y.a());
+          band_fma(v[u], x.b(), y.b());
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sA[(LA_BLK * (i0 - 1 + u) + ti) * kRowStride + tk] = v[u];
+    }
+    if (J + 1 + W < NB) sA[(LA_BLK * W + ti) * kRowStride + tk] = entry(J + 1 + W, J + 1);
+    __syncthreads();
+    if (we > 1) {
+      band_update<CT, W, 2, 4>(a, sPan, ti, tk);
+      if constexpr (W > 4) {
+        if (we > 6) band_update<CT, W, 5, W>(a, sPan, ti, tk);
+        else if (we > 4) band_update<CT, W, 5, 6>(a, sPan, ti, tk);
+      }
+    }
+    // move the window one block along the diagonal
+#pragma unroll
+    for (int i = 2; i <= W; ++i) sB[(i - 2) * 256 + tid] = a[(i - 2) * (i - 1) / 2];
+#pragma unroll
+    for (int i = 2; i < W; ++i)
+#pragma unroll
+      for (int j = 2; j <= i; ++j) a[(i - 2) * (i - 1) / 2 + j - 2] = a[(i - 1) * i / 2 + j - 1];
+    if (J + 1 + W < NB) {
+      sB[(W - 1) * 256 + tid] = entry(J + 1 + W, J + 2);
+#pragma unroll
+      for (int j = 2; j <= W; ++j) a[(W - 2) * (W - 1) / 2 + j - 2] = entry(J + 1 + W, J + 1 + j);
+    }
+    __syncthreads();
   }
 }
 
@@ -1818,6 +2090,22 @@ cudaError_t launch_factor_wide_n(const LevelGeom& L, const FineOp* fine, const T
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   kern<<<L.nsub, kFactorThreads, smem, s>>>(L, *fine, tm, factors, status);
+  return cudaGetLastError();
+}
+
+template <typename R, int NPAD, int W>
+cudaError_t launch_factor_band_n(const LevelGeom& L, const FineOp* fine, const TimeMats* tm,
+                                 typename C2<R>::T* factors, int* status, cudaStream_t s) {
+  if (!fine) return cudaErrorInvalidValue;
+  constexpr size_t smem = band_factor_smem<R, W>();
+  auto kern = k_factor_band<R, NPAD, W>;
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    attr_set = true;
+  }
+  kern<<<L.nsub, kBandThreads, smem, s>>>(L, *fine, tm, factors, status);
   return cudaGetLastError();
 }
 

@@ -6,7 +6,10 @@ cudaError_t launch_factor<float>(const LevelGeom& L, const FineOp* fine, const f
                                   float2* factors, int* status, cudaStream_t s) {
 #define LA_CALL(N) launch_factor_blk_n<float, N>(L, fine, sigma, tm, factors, status, s)
   {
-#define LA_WCALL(N) launch_factor_wide_n<float, N>(L, fine, tm, factors, status, s)
+#define LA_WCALL(N)                                                                          \
+  (L.band <= 4 ? launch_factor_band_n<float, N, 4>(L, fine, tm, factors, status, s)          \
+   : L.band <= 8 ? launch_factor_band_n<float, N, 8>(L, fine, tm, factors, status, s)        \
+                 : launch_factor_wide_n<float, N>(L, fine, tm, factors, status, s))
     LA_NPAD_DISPATCH_WIDE(L.npad, LA_WCALL)
 #undef LA_WCALL
   }
