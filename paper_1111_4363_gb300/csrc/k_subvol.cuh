@@ -34,6 +34,7 @@ template <typename CT> __device__ __forceinline__ void cfma_conj(CT& acc, const 
 
 constexpr int kFactorThreads = 256;
 constexpr int kSweepThreads = 128;
+constexpr int kSuperThreads = 256;   // sweeps with superblock factors
 
 __device__ __forceinline__ void local_coords(int i, const int e[3], int& x, int& y, int& z) {
   x = i % e[0];
@@ -648,6 +649,12 @@ __device__ __forceinline__ void cp_async_elem_zf(double2* sdst, const double2* g
                "l"(gsrc), "r"(valid ? 16 : 0)
                : "memory");
 }
+// 16 bytes, both addresses 16-byte aligned
+__device__ __forceinline__ void cp_async16_zf(void* sdst, const void* gsrc, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(sdst)),
+               "l"(gsrc), "r"(valid ? 16 : 0)
+               : "memory");
+}
 // one real value
 __device__ __forceinline__ void cp_async_real(float* sdst, const float* gsrc) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(sdst)), "l"(gsrc)
@@ -1084,16 +1091,25 @@ k_factor_wide(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C
 //   rest    a ninth warp factorises and inverts the next diagonal block (lookahead) while the others apply
 //           the rank-16 update to the remaining blocks and assemble the row that enters.
 // The factor is written once and never read back.
-// 96^3, K = 4, 4x4x4 subvolumes (13,824 factors of 256 unknowns, W = 8): 6.88 ms = 25 TFLOP/s of banded flops,
-// bound by instruction issue (67% of the slots, 46% of the FMA pipe); 11.1 ms with the left-looking
+// Its diagonal superblocks of kSuper block rows hold the inverse of L's superblock instead of L, so that the
+// triangular solves take NB / 4 steps of larger mat-vecs instead of NB (factor_is_super).  The inverse X is
+// built along with the elimination: the blocks Z_IC = sum_{C <= k < I} L_Ik X_kC grow by one term per column,
+// and X_IC = -inv(L_II) Z_IC when the diagonal block I is inverted; 16 block products per superblock, 11%
+// more multiplications.
+// 96^3, K = 4, 4x4x4 subvolumes (13,824 factors of 256 unknowns, W = 8): 8.24 ms = 21 TFLOP/s of banded flops,
+// bound by instruction issue (6.88 ms without the superblocks' inverses, 67% of the issue slots and 46% of
+// the FMA pipe busy); 11.1 ms with the left-looking
 // factorisation below, which waits on its own earlier blocks in L2 and on a diagonal step three times
 // as long.  A diagonal step by one of the eight warps instead of a ninth: 9.6 ms.
+constexpr int kSuper = 4;
 template <int W> struct BandSmem {
   // the panel and the inverse hold two columns k, k + 1 of a row next to each other, one 16-byte load for
   // both; rows of a panel pair: one more than the window, so that the transposed stores spread over the banks
   static constexpr int kPanStride = 2 * (LA_BLK * W + 1);
-  // complex entries: column blocks, inverse, two row buffers of the diagonal step, panel, the blocks (i, 1)
-  static constexpr int kComplex = (W + 1) * LA_BLK * kRowStride + 256 + 32 + LA_BLK / 2 * kPanStride + 256 * W;
+  // complex entries: column blocks, inverse, two row buffers of the diagonal step, panel, the blocks (i, 1),
+  // the inverse's own layout of two columns, the superblock's inverse
+  static constexpr int kComplex =
+      (W + 1) * LA_BLK * kRowStride + 256 + 32 + LA_BLK / 2 * kPanStride + 256 * W + 512 + 6 * 256;
 };
 template <typename R, int W>
 __host__ __device__ constexpr size_t band_factor_smem() {
@@ -1108,7 +1124,7 @@ __host__ __device__ constexpr size_t band_factor_smem() {
 // c <= j, and every step updates the rows r > j by v[c] -= L_rj w[c] with the row w[c] = conj(L_cj) for
 // c > j, X[j][c] for c <= j (passed through shared memory, read as 16-byte pairs).  Ends with X = inv(L).
 template <typename CT>
-__device__ __forceinline__ void band_diag(const CT* D, CT* sInvT, CT* buf, CT* Fdiag, int* status) {
+__device__ __forceinline__ void band_diag(const CT* D, CT* sInvT, CT* sX, CT* buf, CT* Fdiag, int* status) {
   typedef typename Re<CT>::T R;
   const int lane = threadIdx.x & 31, r = lane & 15, h = lane >> 4;
   CT v[LA_BLK / 2];   // column 2 u + h
@@ -1156,6 +1172,7 @@ __device__ __forceinline__ void band_diag(const CT* D, CT* sInvT, CT* buf, CT* F
     if (c > r) v[u] = mkc<CT>((R)0, (R)0);
     Fdiag[r * LA_BLK + c] = v[u];
     sInvT[(c >> 1) * 32 + 2 * r + (c & 1)] = mkc<CT>(v[u].x, -v[u].y);
+    sX[(r >> 1) * 32 + 2 * c + (r & 1)] = v[u];
   }
 }
 
@@ -1189,6 +1206,56 @@ __device__ __forceinline__ void band_update(CT (&a)[W * (W - 1) / 2], const CT* 
   }
 }
 
+static_assert(kSuper == 4, "the superblock inverse is written for four block rows");
+// x[c] = X_Pc = -inv(L_PP) Z_Pc, c < P: rows ti of inv(L_PP) end at column ti, so warp ti / 2 stops there.
+template <typename CT, int P>
+__device__ __forceinline__ void band_inv_row(CT (&x)[kSuper - 1], const CT* sInvT, const CT* sZ, int ti, int tk) {
+  CT v[P];
+#pragma unroll
+  for (int c = 0; c < P; ++c) v[c] = mkc<CT>(0, 0);
+#pragma unroll 2
+  for (int k2 = 0; k2 <= (ti >> 1); ++k2) {
+    const CPair<CT> a = lds_pair(sInvT + k2 * 32 + 2 * ti);
+#pragma unroll
+    for (int c = 0; c < P; ++c) {
+      const CPair<CT> z = lds_pair(sZ + (P * (P - 1) / 2 + c) * 256 + k2 * 32 + 2 * tk);
+      cfma_conj(v[c], a.a(), z.a());
+      cfma_conj(v[c], a.b(), z.b());
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < P; ++c) x[c] = mkc<CT>(-v[c].x, -v[c].y);
+}
+// Z_ic += L_iP X_Pc for the superblock's rows i > P and columns c <= P (X_PP in xd).
+template <typename CT, int W, int P>
+__device__ __forceinline__ void band_inv_update(CT* sZ, const CT* xd, const CT* pan, int ti, int tk, int own) {
+  CT z[kSuper - 1 - P][P + 1];
+#pragma unroll
+  for (int i = P + 1; i < kSuper; ++i)
+#pragma unroll
+    for (int c = 0; c <= P; ++c) z[i - P - 1][c] = c < P ? sZ[(i * (i - 1) / 2 + c) * 256 + own] : mkc<CT>(0, 0);
+#pragma unroll 2
+  for (int k2 = 0; k2 < LA_BLK / 2; ++k2) {
+    CPair<CT> x[kSuper - 1 - P];
+#pragma unroll
+    for (int i = P + 1; i < kSuper; ++i)
+      x[i - P - 1] = lds_pair(pan + k2 * BandSmem<W>::kPanStride + 2 * (LA_BLK * (i - P - 1) + ti));
+#pragma unroll
+    for (int c = 0; c <= P; ++c) {
+      const CPair<CT> y = lds_pair((c < P ? sZ + (P * (P - 1) / 2 + c) * 256 : xd) + k2 * 32 + 2 * tk);
+#pragma unroll
+      for (int i = P + 1; i < kSuper; ++i) {
+        cfma(z[i - P - 1][c], x[i - P - 1].a(), y.a());
+        cfma(z[i - P - 1][c], x[i - P - 1].b(), y.b());
+      }
+    }
+  }
+#pragma unroll
+  for (int i = P + 1; i < kSuper; ++i)
+#pragma unroll
+    for (int c = 0; c <= P; ++c) sZ[(i * (i - 1) / 2 + c) * 256 + own] = z[i - P - 1][c];
+}
+
 constexpr int kBandThreads = kFactorThreads + 32;
 __device__ __forceinline__ void band_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
@@ -1205,7 +1272,9 @@ k_factor_band(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C
   CT* sBuf = sInvT + 256;                            // [2][16] rows of the diagonal step
   CT* sPan = sBuf + 32;                              // [8][S] the panel, [k / 2][row][k % 2]
   CT* sB = sPan + LA_BLK / 2 * S;                        // [W][256] the blocks (i, 1), each thread its own entries
-  CT* sHH = sB + 256 * W;                            // [64][65] (H, H^2) of the point pairs
+  CT* sXd = sB + 256 * W;                            // [2][256] inv(L_JJ) of columns J and J + 1, [k / 2][c][k % 2]
+  CT* sZ = sXd + 512;                                // [6][256] Z, then X, of the blocks (i, c) of the superblock
+  CT* sHH = sZ + 6 * 256;                            // [64][65] (H, H^2) of the point pairs
   R* sP = reinterpret_cast<R*>(sHH + kWidePtsMax * kHHStride);
   R* sPd = sP + LA_NPAIR * LA_KMAX * LA_KMAX;
   R* sD = sPd + 2 * LA_KMAX * LA_KMAX;
@@ -1242,7 +1311,7 @@ k_factor_band(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C
   if (tid >= kFactorThreads) {   // the diagonal warp
     for (int J = 0; J < NB; ++J) {
       __syncthreads();   // column J is in sA
-      band_diag<CT>(sA, sInvT, sBuf, F + (size_t)tri_index(J, J) * 256, status);
+      band_diag<CT>(sA, sInvT, sXd + (J & 1) * 256, sBuf, F + (size_t)tri_index(J, J) * 256, status);
       __syncthreads();
     }
     return;
@@ -1261,6 +1330,15 @@ k_factor_band(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C
 #pragma unroll 1
   for (int J = 0; J < NB; ++J) {
     const int we = NB - 1 - J < W ? NB - 1 - J : W;   // blocks below the diagonal
+    const int p = J % kSuper;                         // row J's place in its superblock
+    // row J of the superblock's inverse: X_Jc = -inv(L_JJ) Z_Jc
+    CT xr[kSuper - 1];
+    if (p == 1) band_inv_row<CT, 1>(xr, sInvT, sZ, ti, tk);
+    else if (p == 2) band_inv_row<CT, 2>(xr, sInvT, sZ, ti, tk);
+    else if (p == 3) band_inv_row<CT, 3>(xr, sInvT, sZ, ti, tk);
+#pragma unroll
+    for (int c = 0; c < kSuper - 1; ++c)
+      if (c < p) F[(size_t)tri_index(J, J - p + c) * 256 + tid] = xr[c];
     // panel, four blocks at a time
 #pragma unroll 1
     for (int i0 = 1; i0 <= we; i0 += 4) {
@@ -1283,11 +1361,15 @@ k_factor_band(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C
         const int i = i0 + u;
         if (i > we) break;
         sPan[(tk >> 1) * S + 2 * (LA_BLK * (i - 1) + ti) + (tk & 1)] = l[u];
-        if (i <= band) F[(size_t)tri_index(J + i, J) * 256 + tid] = l[u];
+        if (i <= band && i + p >= kSuper) F[(size_t)tri_index(J + i, J) * 256 + tid] = l[u];
       }
     }
     if (we == 0) break;
     band_bar();
+    const int own = (ti >> 1) * 32 + 2 * tk + (ti & 1);   // this thread's entry of a [k / 2][c][k % 2] block
+#pragma unroll
+    for (int c = 0; c < kSuper - 1; ++c)
+      if (c < p) sZ[(p * (p - 1) / 2 + c) * 256 + own] = xr[c];
     // next column: the blocks (i, 1), updated first, and the block that enters the band
 #pragma unroll 1
     for (int i0 = 1; i0 <= we; i0 += 4) {
@@ -1310,6 +1392,9 @@ k_factor_band(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, typename C
     }
     if (J + 1 + W < NB) sA[(LA_BLK * W + ti) * kRowStride + tk] = entry(J + 1 + W, J + 1);
     __syncthreads();
+    if (p == 0) band_inv_update<CT, W, 0>(sZ, sXd + (J & 1) * 256, sPan, ti, tk, own);
+    else if (p == 1) band_inv_update<CT, W, 1>(sZ, sXd + (J & 1) * 256, sPan, ti, tk, own);
+    else if (p == 2) band_inv_update<CT, W, 2>(sZ, sXd + (J & 1) * 256, sPan, ti, tk, own);
     if (we > 1) {
       band_update<CT, W, 2, 4>(a, sPan, ti, tk);
       if constexpr (W > 4) {
@@ -1573,6 +1658,156 @@ __device__ __forceinline__ void subvol_solve_wide(const CT* __restrict__ F, int 
   }
 }
 
+// Solves with a factor whose diagonal superblocks hold inverses (factor_is_super), by 256 threads.  With
+// 64-row superblocks R: forward t_R = rhs_R - sum_{C<R} L_RC y_C, y_R = X_RR t_R; backward
+// t_R = y_R - sum_{C>R} L_CR^dagger x_C, x_R = X_RR^dagger t_R: 2 NB / 4 steps of two mat-vecs each instead of
+// 2 NB steps of 16 rows, so a subvolume's chain is 14 barriers.  A mat-vec runs through its 16 x 16 blocks
+// in pieces of four 16-byte loads per lane, issued kAhead pieces before they are used.
+// What bounds it is the L1 data path (the factor passes through it twice), so the vectors must cost little
+// there: forward, warp (i, half) = (w / 2, w % 2) takes the blocks of block row i with even or odd column and
+// lane (row l / 8, column pair l % 8) four rows of a block, so that one 16-byte vector load serves a block;
+// the halves' sums stay apart in shared memory and are added by whoever reads them.  Backward, warp w takes
+// columns 8 w .. + 7, lane (row l / 4, column pair l % 4) two rows of a block.
+struct SuperPiece {
+  float4 v[4];
+};
+__device__ __forceinline__ float4 ldg_block(const float2* p, bool valid, unsigned long long pol) {
+  return valid ? ldg_policy(reinterpret_cast<const float4*>(p), pol) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+__device__ __forceinline__ float4 add4(float4 a, float4 b) {
+  return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+__device__ __forceinline__ float4 sub4(float4 a, float4 b) {
+  return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
+__device__ __forceinline__ float2 shfl_xor2(float2 v, int m) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
+}
+// One exchange of a transposing reduction: lanes without bit m of their index keep a, the others b, each
+// adding the partner's share.
+__device__ __forceinline__ float2 fold(float2 a, float2 b, bool hi, int m) {
+  const float2 send = hi ? a : b, mine = hi ? b : a, got = shfl_xor2(send, m);
+  return make_float2(mine.x + got.x, mine.y + got.y);
+}
+
+// rhs [NPAD] in; the solution goes to x [NPAD].  y [2][NPAD], p [2][64]: scratch, the halves' sums.
+template <int NPAD>
+__device__ __forceinline__ void subvol_solve_super(const float2* __restrict__ F, int band, const float2* rhs, float2* y,
+                                                   float2* p, float2* x) {
+  constexpr int NS = NPAD / (LA_BLK * kSuper);
+  // pieces of the forward pass: rows R = 0 .. NS-1, columns C = 0 .. R, two each; the backward pass takes the
+  // transposed ones, rows NS-1 .. 0
+  constexpr int NP = NS * (NS + 1);
+  constexpr int kAhead = 1, NBUF = kAhead + 1;
+  const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
+  const unsigned long long keep = l2_evict_last(), last_use = l2_evict_first();
+  const int bi = w >> 1, wh = w & 1;     // block row (forward) or column (backward) in the superblock, half
+  const int fq = l & 7, fr = l >> 3, bq = l & 3, br = l >> 2;
+  const float2* const fbase = F + (size_t)(bi * (bi + 1) / 2 + wh) * 256 + fr * LA_BLK + 2 * fq;
+  const float2* const bbase = F + (size_t)bi * 256 + br * LA_BLK + 8 * wh + 2 * bq;
+  auto row_of = [](int s) constexpr {
+    int R = 0;
+    while ((R + 1) * (R + 2) <= s) ++R;
+    return R;
+  };
+  auto fwd_ok = [&](int R, int C, int jj) { return R == C ? jj <= bi : kSuper * (R - C) + bi - jj <= band; };
+  auto bwd_ok = [&](int C, int R, int ii) { return R == C ? ii >= bi : kSuper * (C - R) + ii - bi <= band; };
+  SuperPiece buf[NBUF];
+  auto load = [&](SuperPiece& b, int s) {   // piece s of both passes, 0 .. 2 NP - 1
+    const int q = s < NP ? s : s - NP;
+    const int A = row_of(q), B = (q - A * (A + 1)) >> 1, h = (q - A * (A + 1)) & 1;
+    if (s < NP) {   // block (4 A + bi, 4 B + 2 h + wh); tri_index(4 A + i, J) = 8 A^2 + 2 A + 4 A i + tri(i) + J
+      const float2* a = fbase + (size_t)(4 * A * bi) * 256 + (8 * A * A + 2 * A + kSuper * B + 2 * h) * 256;
+      const bool ok = fwd_ok(A, B, 2 * h + wh);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) b.v[u] = ldg_block(a + 4 * u * LA_BLK, ok, keep);
+    } else {   // blocks (4 C + 2 h, 4 C + 2 h + 1) of columns R = NS-1-A, C = NS-1-B
+      const int R = NS - 1 - A, C = NS - 1 - B;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int ii = 2 * h + u, I = kSuper * C + ii;
+        const float2* a = bbase + (size_t)(I * (I + 1) / 2 + kSuper * R) * 256;
+        const bool ok = bwd_ok(C, R, ii);
+        b.v[2 * u] = ldg_block(a, ok, last_use);
+        b.v[2 * u + 1] = ldg_block(a + 8 * LA_BLK, ok, last_use);
+      }
+    }
+  };
+#pragma unroll
+  for (int s = 0; s < kAhead; ++s) load(buf[s], s);
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 acc[4] = {zero, zero, zero, zero};
+#pragma unroll
+  for (int s = 0; s < NP; ++s) {
+    const int R = row_of(s), C = (s - R * (R + 1)) >> 1, h = (s - R * (R + 1)) & 1;
+    load(buf[(s + kAhead) % NBUF], s + kAhead);
+    const SuperPiece& b = buf[s % NBUF];
+    const int jj = 2 * h + wh;
+    if (fwd_ok(R, C, jj)) {
+      const int at = LA_BLK * jj + 2 * fq;
+      float4 v;
+      if (C < R) {
+        v = add4(*reinterpret_cast<const float4*>(y + 64 * C + at), *reinterpret_cast<const float4*>(y + NPAD + 64 * C + at));
+      } else {
+        v = *reinterpret_cast<const float4*>(rhs + 64 * R + at);
+        if (R > 0) v = sub4(sub4(v, *reinterpret_cast<const float4*>(p + at)), *reinterpret_cast<const float4*>(p + 64 + at));
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        cfma(acc[u], make_float2(b.v[u].x, b.v[u].y), make_float2(v.x, v.y));
+        cfma(acc[u], make_float2(b.v[u].z, b.v[u].w), make_float2(v.z, v.w));
+      }
+    }
+    if (h == 1 && (C == R || C == R - 1)) {
+      // the four rows over the eight column pairs: lane fq ends with row fr + 4 (fq / 2)
+      const float2 a = fold(acc[0], acc[2], fq & 4, 4), c = fold(acc[1], acc[3], fq & 4, 4);
+      float2 r = fold(a, c, fq & 2, 2);
+      r = reduce_xor(r, 1);
+      if (!(fq & 1)) (C == R ? y + wh * NPAD + 64 * R : p + 64 * wh)[LA_BLK * bi + fr + 4 * (fq >> 1)] = r;
+      acc[0] = acc[1] = acc[2] = acc[3] = zero;
+      __syncthreads();
+    }
+  }
+  float2 acc0 = zero, acc1 = zero;
+#pragma unroll
+  for (int s = 0; s < NP; ++s) {
+    const int A = row_of(s), R = NS - 1 - A, C = NS - 1 - ((s - A * (A + 1)) >> 1), h = (s - A * (A + 1)) & 1;
+    if (s + kAhead < NP) load(buf[(NP + s + kAhead) % NBUF], NP + s + kAhead);
+    const SuperPiece& b = buf[(NP + s) % NBUF];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int ii = 2 * h + u;
+      if (!bwd_ok(C, R, ii)) continue;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int row = LA_BLK * ii + br + 8 * e;
+        float2 v;
+        if (C > R) {
+          v = x[64 * C + row];
+        } else {
+          const float2 y0 = y[64 * R + row], y1 = y[NPAD + 64 * R + row];
+          v = make_float2(y0.x + y1.x, y0.y + y1.y);
+          if (R < NS - 1) {
+            const float2 q = p[row];
+            v = make_float2(v.x - q.x, v.y - q.y);
+          }
+        }
+        const float4 m = b.v[2 * u + e];
+        cfma_conj(acc0, make_float2(m.x, m.y), v);
+        cfma_conj(acc1, make_float2(m.z, m.w), v);
+      }
+    }
+    if (h == 1 && (C == R || C == R + 1)) {
+      float2 r = fold(acc0, acc1, br & 1, 4);
+      r = reduce_xor(r, 8);
+      r = reduce_xor(r, 16);
+      if (br < 2) (C == R ? x + 64 * R : p)[8 * w + 2 * bq + br] = r;
+      acc0 = acc1 = zero;
+      __syncthreads();
+    }
+  }
+}
+
 // The 128-thread solve (every step's blocks loaded together, the next step's in flight) serves every
 // complex64 factor and the wide FP64 ones; shorter FP64 factors keep the two-warp solve, whose
 // two-level reductions issue fewer adds on the slow FP64 pipe.
@@ -1588,10 +1823,9 @@ template <typename R, int NPAD>
 __global__ void __launch_bounds__(kSweepThreads)
 k_sweep_fine(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const typename C2<R>::T* __restrict__ f,
              const typename C2<R>::T* __restrict__ yx, typename C2<R>::T* __restrict__ c,
-             const typename C2<R>::T* __restrict__ factors, int colour, int* __restrict__ status) {
+             const typename C2<R>::T* __restrict__ factors, int colour) {
   typedef typename C2<R>::T CT;
   extern __shared__ __align__(16) unsigned char smem[];
-  (void)status;   // no bounded wait in this kernel
   const int K = tm->K, KK = K * K;
   const int tid = threadIdx.x;
   const int b = colour_subvol(L, colour, blockIdx.x);
@@ -1806,6 +2040,289 @@ k_sweep_fine(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const typen
     v.x += sRhs[t].x;
     v.y += sRhs[t].y;
     c[gi] = v;
+  }
+}
+
+// Shared memory of k_sweep_super: byte offsets of its arrays (the time matrices are at 0) and the total.
+struct SuperSmem {
+  int v, c, z, rhs, total;
+};
+__host__ __device__ __forceinline__ SuperSmem super_smem(const LevelGeom& L, int K) {
+  const int nbc = (L.sub[0] + 4) * (L.dim > 1 ? L.sub[1] + 4 : 1) * (L.dim > 2 ? L.sub[2] + 4 : 1);
+  const int nbf = (L.sub[0] + 2) * (L.dim > 1 ? L.sub[1] + 2 : 1) * (L.dim > 2 ? L.sub[2] + 2 : 1);
+  SuperSmem s;
+  s.v = (5 * K * K * 4 + 15) & ~15;
+  s.c = s.v + ((nbf * 4 + 15) & ~15);
+  s.z = s.c + ((nbc * K * 8 + 15) & ~15);
+  s.rhs = s.z + ((nbf * K * 8 + 15) & ~15);
+  s.total = s.rhs + (4 * L.npad + 128) * 8;   // rhs, the solution, y in two halves, products in two halves
+  return s;
+}
+
+// ------------------------------------------------------------------------ finest sweep, superblock factors
+// Rows of K floats of the time matrices from shared memory, in the widest loads K allows.
+template <int K>
+__device__ __forceinline__ void row_k(const float* p, float (&r)[K]) {
+  if constexpr (K % 4 == 0) {
+#pragma unroll
+    for (int n = 0; n < K; n += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(p + n);
+      r[n] = v.x; r[n + 1] = v.y; r[n + 2] = v.z; r[n + 3] = v.w;
+    }
+  } else if constexpr (K % 2 == 0) {
+#pragma unroll
+    for (int n = 0; n < K; n += 2) {
+      const float2 v = *reinterpret_cast<const float2*>(p + n);
+      r[n] = v.x; r[n + 1] = v.y;
+    }
+  } else {
+#pragma unroll
+    for (int n = 0; n < K; ++n) r[n] = p[n];
+  }
+}
+// The K complex values of a point's record.
+template <int K>
+__device__ __forceinline__ void rec_k(const float2* p, float2 (&v)[K]) {
+  if constexpr (K % 2 == 0) {
+#pragma unroll
+    for (int n = 0; n < K; n += 2) {
+      const float4 q = *reinterpret_cast<const float4*>(p + n);
+      v[n] = make_float2(q.x, q.y);
+      v[n + 1] = make_float2(q.z, q.w);
+    }
+  } else {
+#pragma unroll
+    for (int n = 0; n < K; ++n) v[n] = p[n];
+  }
+}
+
+// One complex64 subvolume of a colour with a superblock factor, as sweep_fine, with one thread per point: a
+// thread holds the point's K coefficients in registers, so residual, weight and H c need no pass over
+// shared memory between them and the index maps are paid once per point instead of once per coefficient.
+// One colour of 128^3, K = 4, 4x4x4 subvolumes (4096 of them): 236 us = 3.8 TB/s of in-band factor bytes read
+// once (the backward pass finds them in L2), against 319 us with 128 threads and 16-row steps; 96^3: 105
+// against 157 us.  Bound by the latency of a CTA's phases:
+// four CTAs per SM with one piece in flight (64 registers) beat three with two (108 us at 96^3) and two with three
+// (116 us); an L2 prefetch of the band at the start of the CTA costs 7 us.
+template <int NPAD, int K>
+__global__ void __launch_bounds__(kSuperThreads, K <= 4 ? 4 : 2)
+k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const float2* __restrict__ f,
+              const float2* __restrict__ yx, float2* __restrict__ c, const float2* __restrict__ factors, int colour,
+              FastDiv dn0, FastDiv dn1) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int NT = kSuperThreads, KK = K * K;
+  const int tid = threadIdx.x;
+  // blockIdx.x-th subvolume of the colour (dn0, dn1: the colour's subvolumes along x and y)
+  const int jr = fdiv(blockIdx.x, dn0), jz = fdiv(jr, dn1);
+  const int bb[3] = {2 * ((int)blockIdx.x - jr * dn0.d) + (colour & 1), 2 * (jr - jz * dn1.d) + ((colour >> 1) & 1),
+                     2 * jz + ((colour >> 2) & 1)};
+  const float2* F = factors + (size_t)((bb[2] * L.nb[1] + bb[1]) * L.nb[0] + bb[0]) * L.fsize;
+  int o[3], e[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    o[a] = bb[a] * L.sub[a];
+    e[a] = min(L.sub[a], L.n[a] - o[a]);
+  }
+  int ec[3], ef[3], oc[3], of_[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const bool used = a < L.dim;
+    ec[a] = used ? e[a] + 4 : 1;  oc[a] = used ? o[a] - 2 : o[a];
+    ef[a] = used ? e[a] + 2 : 1;  of_[a] = used ? o[a] - 1 : o[a];
+  }
+  const int nbc = ec[0] * ec[1] * ec[2], nbf = ef[0] * ef[1] * ef[2], npts = e[0] * e[1] * e[2];
+  const SuperSmem S = super_smem(L, K);
+  const bool full = e[0] == L.sub[0] && e[1] == L.sub[1] && e[2] == L.sub[2];
+  const FastDiv dc0 = full ? L.fd_c[0] : make_fastdiv(ec[0]), dc1 = full ? L.fd_c[1] : make_fastdiv(ec[1]);
+  const FastDiv df0 = full ? L.fd_f[0] : make_fastdiv(ef[0]), df1 = full ? L.fd_f[1] : make_fastdiv(ef[1]);
+  const FastDiv du0 = full ? L.fd_u[0] : make_fastdiv(e[0]), du1 = full ? L.fd_u[1] : make_fastdiv(e[1]);
+  auto coords = [](int i, const FastDiv& d0, const FastDiv& d1, int& x, int& y, int& z) {
+    const int r = fdiv(i, d0);
+    x = i - r * d0.d;
+    z = fdiv(r, d1);
+    y = r - z * d1.d;
+  };
+  float* sM = reinterpret_cast<float*>(smem);                   // Q, U, E, W, Q^T [K][K] each
+  float* sV = reinterpret_cast<float*>(smem + S.v);             // dsum + V0 on the footprint
+  float2* sC = reinterpret_cast<float2*>(smem + S.c);           // c on U + 2
+  float2* sZ = reinterpret_cast<float2*>(smem + S.z);           // z = Wt r on the footprint
+  float2* sRhs = reinterpret_cast<float2*>(smem + S.rhs);       // right-hand side
+  float2* sXs = sRhs + NPAD;                                    // solution
+  float2* sY = sXs + NPAD;                                      // scratch of the solves
+  float2* sPr = sY + 2 * NPAD;
+
+  for (int t = tid; t < nbc; t += NT) {
+    int lx, ly, lz;
+    coords(t, dc0, dc1, lx, ly, lz);
+    const int gx = oc[0] + lx, gy = oc[1] + ly, gz = oc[2] + lz;
+    const bool in = fine_in(g, gx, gy, gz);
+    const float2* src = in ? c + (size_t)((gz * g.n[1] + gy) * g.n[0] + gx) * K : c;
+    if constexpr (K % 2 == 0) {
+#pragma unroll
+      for (int m = 0; m < K; m += 2) cp_async16_zf(sC + t * K + m, src + m, in);
+    } else {
+#pragma unroll
+      for (int m = 0; m < K; ++m) cp_async_elem_zf(sC + t * K + m, src + m, in);
+    }
+  }
+  for (int i = tid; i < KK; i += NT) {
+    const float q = (float)tm->Qb[i];
+    sM[i] = q;
+    sM[KK + i] = (float)tm->Ub[i];
+    sM[2 * KK + i] = (float)tm->Eb[i];
+    sM[3 * KK + i] = (float)tm->Wt[i];
+    sM[4 * KK + (i % K) * K + i / K] = q;
+  }
+  const float dsum = (float)g.dsum;
+  const float xo = (float)(g.lax == 0 ? g.x0[0] : (g.lax == 1 ? g.x0[1] : g.x0[2]));
+  const float xh = (float)(g.lax == 0 ? g.h[0] : (g.lax == 1 ? g.h[1] : g.h[2]));
+  const float wx = -0.5f * (float)g.ih2[0], wy = -0.5f * (float)g.ih2[1], wz = -0.5f * (float)g.ih2[2];
+  const int dcy = L.dim > 1 ? ec[0] : 0, dcz = L.dim > 2 ? ec[0] * ec[1] : 0;
+  auto laser_x = [&](int gx, int gy, int gz) { return xo + (float)(g.lax == 0 ? gx : (g.lax == 1 ? gy : gz)) * xh; };
+  // r = f - M~ c and z = Wt r on the footprint, zero outside the grid
+  bool staged = false;
+  for (int i = tid; i < nbf || !staged; i += NT) {
+    int lx = 0, ly = 0, lz = 0;
+    coords(i < nbf ? i : 0, df0, df1, lx, ly, lz);
+    const int gx = of_[0] + lx, gy = of_[1] + ly, gz = of_[2] + lz;
+    const bool in = i < nbf && fine_in(g, gx, gy, gz);
+    const size_t p = (size_t)((gz * g.n[1] + gy) * g.n[0] + gx);
+    float2 r[K];
+#pragma unroll
+    for (int m = 0; m < K; ++m) r[m] = make_float2(0.f, 0.f);
+    float dg = 0.f;
+    if (in) {
+      dg = dsum + (float)g.V0[p];
+      if (f) rec_k<K>(f + p * K, r);
+    }
+    if (!staged) {
+      cp_async_wait_all();
+      __syncthreads();
+      staged = true;
+    }
+    if (i >= nbf) break;
+    sV[i] = dg;
+    float2 z[K];
+#pragma unroll
+    for (int m = 0; m < K; ++m) z[m] = make_float2(0.f, 0.f);
+    if (in) {
+      const float2* own = sC + (((L.dim > 2 ? lz + 1 : lz) * ec[1] + (L.dim > 1 ? ly + 1 : ly)) * ec[0] + lx + 1) * K;
+      float2 v[K], h[K], a1[K], a2[K];
+      rec_k<K>(own, v);
+      rec_k<K>(own + K, a1);
+      rec_k<K>(own - K, a2);
+#pragma unroll
+      for (int m = 0; m < K; ++m)
+        h[m] = make_float2(dg * v[m].x + wx * (a1[m].x + a2[m].x), dg * v[m].y + wx * (a1[m].y + a2[m].y));
+      if (L.dim > 1) {
+        rec_k<K>(own + dcy * K, a1);
+        rec_k<K>(own - dcy * K, a2);
+#pragma unroll
+        for (int m = 0; m < K; ++m) { h[m].x += wy * (a1[m].x + a2[m].x); h[m].y += wy * (a1[m].y + a2[m].y); }
+      }
+      if (L.dim > 2) {
+        rec_k<K>(own + dcz * K, a1);
+        rec_k<K>(own - dcz * K, a2);
+#pragma unroll
+        for (int m = 0; m < K; ++m) { h[m].x += wz * (a1[m].x + a2[m].x); h[m].y += wz * (a1[m].y + a2[m].y); }
+      }
+      const float xl = laser_x(gx, gy, gz);
+#pragma unroll
+      for (int m = 0; m < K; ++m) {
+        float q[K], u[K], ee[K];
+        row_k<K>(sM + m * K, q);
+        row_k<K>(sM + KK + m * K, u);
+        row_k<K>(sM + 2 * KK + m * K, ee);
+        float qr = 0, qi = 0, ur = 0, ui = 0, er = 0, ei = 0;
+#pragma unroll
+        for (int n = 0; n < K; ++n) {
+          qr = fmaf(q[n], v[n].x, qr); qi = fmaf(q[n], v[n].y, qi);
+          ur = fmaf(u[n], h[n].x, ur); ui = fmaf(u[n], h[n].y, ui);
+          er = fmaf(ee[n], v[n].x, er); ei = fmaf(ee[n], v[n].y, ei);
+        }
+        r[m].x -= -qi - ur - xl * er;
+        r[m].y -= qr - ui - xl * ei;
+      }
+#pragma unroll
+      for (int m = 0; m < K; ++m) {
+        float wm[K];
+        row_k<K>(sM + 3 * KK + m * K, wm);
+#pragma unroll
+        for (int n = 0; n < K; ++n) { z[m].x = fmaf(wm[n], r[n].x, z[m].x); z[m].y = fmaf(wm[n], r[n].y, z[m].y); }
+      }
+    }
+    if constexpr (K % 2 == 0) {
+#pragma unroll
+      for (int m = 0; m < K; m += 2)
+        *reinterpret_cast<float4*>(sZ + i * K + m) = make_float4(z[m].x, z[m].y, z[m + 1].x, z[m + 1].y);
+    } else {
+#pragma unroll
+      for (int m = 0; m < K; ++m) sZ[i * K + m] = z[m];
+    }
+  }
+  __syncthreads();
+  // rhs = M~^dagger z = -i Qb^T z - Ub H z - x Eb z on U; padding 0
+  for (int t = npts * K + tid; t < NPAD; t += NT) sRhs[t] = make_float2(0.f, 0.f);
+  const int dfy = L.dim > 1 ? ef[0] : 0, dfz = L.dim > 2 ? ef[0] * ef[1] : 0;
+  for (int i = tid; i < npts; i += NT) {
+    int lx, ly, lz;
+    coords(i, du0, du1, lx, ly, lz);
+    const int fi = ((L.dim > 2 ? lz + 1 : lz) * ef[1] + (L.dim > 1 ? ly + 1 : ly)) * ef[0] + lx + 1;
+    const int gx = o[0] + lx, gy = o[1] + ly, gz = o[2] + lz;
+    const float2* own = sZ + fi * K;
+    const float dg = sV[fi], xl = laser_x(gx, gy, gz);
+    float2 v[K], h[K], a1[K], a2[K];
+    rec_k<K>(own, v);
+    rec_k<K>(own + K, a1);
+    rec_k<K>(own - K, a2);
+#pragma unroll
+    for (int m = 0; m < K; ++m)
+      h[m] = make_float2(dg * v[m].x + wx * (a1[m].x + a2[m].x), dg * v[m].y + wx * (a1[m].y + a2[m].y));
+    if (L.dim > 1) {
+      rec_k<K>(own + dfy * K, a1);
+      rec_k<K>(own - dfy * K, a2);
+#pragma unroll
+      for (int m = 0; m < K; ++m) { h[m].x += wy * (a1[m].x + a2[m].x); h[m].y += wy * (a1[m].y + a2[m].y); }
+    }
+    if (L.dim > 2) {
+      rec_k<K>(own + dfz * K, a1);
+      rec_k<K>(own - dfz * K, a2);
+#pragma unroll
+      for (int m = 0; m < K; ++m) { h[m].x += wz * (a1[m].x + a2[m].x); h[m].y += wz * (a1[m].y + a2[m].y); }
+    }
+    const size_t p = (size_t)((gz * g.n[1] + gy) * g.n[0] + gx);
+#pragma unroll
+    for (int m = 0; m < K; ++m) {
+      float q[K], u[K], ee[K];
+      row_k<K>(sM + 4 * KK + m * K, q);
+      row_k<K>(sM + KK + m * K, u);
+      row_k<K>(sM + 2 * KK + m * K, ee);
+      float qr = 0, qi = 0, ur = 0, ui = 0, er = 0, ei = 0;
+#pragma unroll
+      for (int n = 0; n < K; ++n) {
+        qr = fmaf(q[n], v[n].x, qr); qi = fmaf(q[n], v[n].y, qi);
+        ur = fmaf(u[n], h[n].x, ur); ui = fmaf(u[n], h[n].y, ui);
+        er = fmaf(ee[n], v[n].x, er); ei = fmaf(ee[n], v[n].y, ei);
+      }
+      float2 out = make_float2(qi - ur - xl * er, -qr - ui - xl * ei);
+      if (yx) {   // additive right-hand side (adjoint relaxation of G z = y)
+        const float2 yv = yx[p * K + m];
+        out.x += yv.x;
+        out.y += yv.y;
+      }
+      sRhs[i * K + m] = out;
+    }
+  }
+  __syncthreads();
+  subvol_solve_super<NPAD>(F, L.band, sRhs, sY, sPr, sXs);
+  for (int t = tid; t < npts * K; t += NT) {   // c_U += delta, with c_U still in shared memory
+    const int i = t / K, m = t - i * K;
+    int lx, ly, lz;
+    coords(i, du0, du1, lx, ly, lz);
+    const float2 d = sXs[t];
+    const float2 v = sC[(((L.dim > 2 ? lz + 2 : lz) * ec[1] + (L.dim > 1 ? ly + 2 : ly)) * ec[0] + lx + 2) * K + m];
+    c[(size_t)(((o[2] + lz) * g.n[1] + (o[1] + ly)) * g.n[0] + (o[0] + lx)) * K + m] =
+        make_float2(v.x + d.x, v.y + d.y);
   }
 }
 
@@ -2031,6 +2548,12 @@ inline size_t factor_smem(const LevelGeom& L, int nptsmax, size_t csize, int mpc
   return mpc * (csize * (ntri + L.npad) + (size_t)L.npad * (csize / 2)) +
          sizeof(double) * (LA_NPAIR * LA_KMAX * LA_KMAX + mpc * npair * LA_NPAIR) + sizeof(int) * (mpc * npair + 1);
 }
+// Factors with inverted diagonal superblocks (k_factor_band): complex64, more than 128 unknowns and a band of
+// at most 8 blocks, the largest window k_factor_band keeps in registers.
+template <typename R>
+inline bool factor_is_super(const LevelGeom& L) {
+  return sizeof(R) == 4 && L.npad > LA_NPAD_MAX && L.band <= 8;
+}
 inline size_t sweep_fine_smem(const LevelGeom& L, int K, size_t rsize, size_t csize) {
   const int sx = L.sub[0] + 4, sy = L.dim > 1 ? L.sub[1] + 4 : 1, sz = L.dim > 2 ? L.sub[2] + 4 : 1;
   const size_t nbc = (size_t)sx * sy * sz;
@@ -2134,12 +2657,40 @@ cudaError_t launch_factor_n(const LevelGeom& L, const FineOp* fine, const R* sig
     return launch_factor_m<R, NPAD, 1>(L, fine, sigma, tm, factors, status, s);
   return launch_factor_m<R, NPAD, mpc>(L, fine, sigma, tm, factors, status, s);
 }
+template <int NPAD, int K>
+cudaError_t launch_sweep_super(const LevelGeom& L, const FineOp& g, const TimeMats* tm, const float2* f,
+                               const float2* yx, float2* c, const float2* factors, int colour, int nblocks,
+                               cudaStream_t s) {
+  const int smem = super_smem(L, K).total;
+  auto kern = k_sweep_super<NPAD, K>;
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (err != cudaSuccess) return err;
+    attr_set = true;
+  }
+  if (smem > 227 * 1024) return cudaErrorInvalidValue;
+  const FastDiv dn0 = make_fastdiv((L.nb[0] - (colour & 1) + 1) / 2),
+                dn1 = make_fastdiv((L.nb[1] - ((colour >> 1) & 1) + 1) / 2);
+  kern<<<nblocks, kSuperThreads, smem, s>>>(L, g, tm, f, yx, c, factors, colour, dn0, dn1);
+  return cudaGetLastError();
+}
 template <typename R, int NPAD>
 cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeMats* tm, int K,
                                 const typename C2<R>::T* f, const typename C2<R>::T* yx, typename C2<R>::T* c,
-                                const typename C2<R>::T* factors, int colour, int* status, cudaStream_t s) {
+                                const typename C2<R>::T* factors, int colour, cudaStream_t s) {
   const int nblocks = colour_count(L, colour);
   if (nblocks == 0) return cudaSuccess;
+  if constexpr (sizeof(R) == 4 && NPAD > LA_NPAD_MAX) {
+    if (factor_is_super<R>(L)) {
+#define LA_SUPER(KK) case KK: return launch_sweep_super<NPAD, KK>(L, g, tm, f, yx, c, factors, colour, nblocks, s)
+      switch (K) {   // 64 points at most: more than 128 unknowns need K >= 3
+        LA_SUPER(3); LA_SUPER(4); LA_SUPER(5); LA_SUPER(6); LA_SUPER(7); LA_SUPER(8);
+        default: return cudaErrorInvalidValue;
+      }
+#undef LA_SUPER
+    }
+  }
   const size_t smem = sweep_fine_smem(L, K, sizeof(R), sizeof(typename C2<R>::T));
   auto kern = k_sweep_fine<R, NPAD>;
   static bool attr_set = false;
@@ -2149,7 +2700,7 @@ cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeM
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  kern<<<nblocks, kSweepThreads, smem, s>>>(L, g, tm, f, yx, c, factors, colour, status);
+  kern<<<nblocks, kSweepThreads, smem, s>>>(L, g, tm, f, yx, c, factors, colour);
   return cudaGetLastError();
 }
 template <typename R, int NPAD>

@@ -6,10 +6,10 @@ cudaError_t launch_factor<float>(const LevelGeom& L, const FineOp* fine, const f
                                   float2* factors, int* status, cudaStream_t s) {
 #define LA_CALL(N) launch_factor_blk_n<float, N>(L, fine, sigma, tm, factors, status, s)
   {
-#define LA_WCALL(N)                                                                          \
-  (L.band <= 4 ? launch_factor_band_n<float, N, 4>(L, fine, tm, factors, status, s)          \
-   : L.band <= 8 ? launch_factor_band_n<float, N, 8>(L, fine, tm, factors, status, s)        \
-                 : launch_factor_wide_n<float, N>(L, fine, tm, factors, status, s))
+#define LA_WCALL(N)                                                                             \
+  (!factor_is_super<float>(L) ? launch_factor_wide_n<float, N>(L, fine, tm, factors, status, s) \
+   : L.band <= 4 ? launch_factor_band_n<float, N, 4>(L, fine, tm, factors, status, s)           \
+                 : launch_factor_band_n<float, N, 8>(L, fine, tm, factors, status, s))
     LA_NPAD_DISPATCH_WIDE(L.npad, LA_WCALL)
 #undef LA_WCALL
   }
@@ -18,8 +18,8 @@ cudaError_t launch_factor<float>(const LevelGeom& L, const FineOp* fine, const f
 }
 template <>
 cudaError_t launch_sweep_fine<float>(const LevelGeom& L, const FineOp& g, const TimeMats* tm, int K, const float2* f,
-                                      const float2* yx, float2* c, const float2* factors, int colour, int* status, cudaStream_t s) {
-#define LA_CALL(N) launch_sweep_fine_n<float, N>(L, g, tm, K, f, yx, c, factors, colour, status, s)
+                                      const float2* yx, float2* c, const float2* factors, int colour, cudaStream_t s) {
+#define LA_CALL(N) launch_sweep_fine_n<float, N>(L, g, tm, K, f, yx, c, factors, colour, s)
   LA_NPAD_DISPATCH_WIDE(L.npad, LA_CALL)
   LA_NPAD_DISPATCH(L.npad, LA_CALL)
 #undef LA_CALL

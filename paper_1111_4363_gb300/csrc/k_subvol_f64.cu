@@ -15,8 +15,8 @@ cudaError_t launch_factor<double>(const LevelGeom& L, const FineOp* fine, const 
 }
 template <>
 cudaError_t launch_sweep_fine<double>(const LevelGeom& L, const FineOp& g, const TimeMats* tm, int K, const double2* f,
-                                      const double2* yx, double2* c, const double2* factors, int colour, int* status, cudaStream_t s) {
-#define LA_CALL(N) launch_sweep_fine_n<double, N>(L, g, tm, K, f, yx, c, factors, colour, status, s)
+                                      const double2* yx, double2* c, const double2* factors, int colour, cudaStream_t s) {
+#define LA_CALL(N) launch_sweep_fine_n<double, N>(L, g, tm, K, f, yx, c, factors, colour, s)
   LA_NPAD_DISPATCH_WIDE(L.npad, LA_CALL)
   LA_NPAD_DISPATCH(L.npad, LA_CALL)
 #undef LA_CALL

@@ -395,7 +395,7 @@ cudaError_t launch_factor(const LevelGeom& L, const FineOp* fine, const R* sigma
 template <typename R>
 cudaError_t launch_sweep_fine(const LevelGeom& L, const FineOp& g, const TimeMats* tm, int K,
                               const typename C2<R>::T* f, const typename C2<R>::T* yx, typename C2<R>::T* c,
-                              const typename C2<R>::T* factors, int colour, int* status, cudaStream_t s);
+                              const typename C2<R>::T* factors, int colour, cudaStream_t s);
 template <typename R>
 cudaError_t launch_gresid_tiles(const LevelGeom& L, const R* sigma, const TimeMats* tm, int K,
                                 const typename C2<R>::T* gvec, const typename C2<R>::T* e, typename C2<R>::T* out,

@@ -31,6 +31,7 @@ CASES = {
     "3d_4x4x4_K3": case(3, (8, 4, 6), (4, 4, 4), 3),               # 192 unknowns, K does not divide 16
     "2d_8x8_K4": case(2, (16, 13, 1), (8, 8, 1), 4),               # band 4
     "2d_8x8_K3": case(2, (8, 16, 1), (8, 8, 1), 3),                # 192 unknowns
+    "2d_5x9_K3": case(2, (11, 20, 1), (5, 9, 1), 3),               # odd extents, tails of 1 and 2 points
     "1d_32_K8": case(1, (80, 1, 1), (32, 1, 1), 8),                # band 1, tail of 16 points
     "1d_64_K3": case(1, (100, 1, 1), (64, 1, 1), 3),               # band 1
 }
