@@ -190,10 +190,13 @@ k_factor(LevelGeom L, FineOp g, int is_fine, int nptsmax, const R* __restrict__ 
   // ---- right-looking Cholesky.  Work of each phase is spread linearly over exactly the active
   // entries of all the CTA's matrices (consecutive threads take consecutive entries of a row), so
   // every issued FP64 instruction has all lanes busy except in the last warp of a phase.
+  // Column j ends at the last row its point couples to (L.reach): the rows below stay exact zeros in G and in
+  // the factor, so neither phase visits them (4x4 points x 6, 4096 matrices: 5.61 -> 4.19 ms).
   for (int j = 0; j < NPAD; ++j) {
-    // (A) scale and publish column j: rows j+1 .. NPAD-1 of every matrix
+    const int m1 = min(NPAD - 1, (fdiv(j, L.fd_K) + L.reach + 1) * K - 1) - j;
+    // (A) scale and publish column j: rows j+1 .. j+m1 of every matrix
     {
-      const int rows = NPAD - 1 - j;
+      const int rows = m1;
       for (int t = tid; t < MPC * rows; t += kFactorThreads) {
         const int mi = t / rows, r = j + 1 + (t - mi * rows);
         const R inv = sInv[mi * NPAD + j];
@@ -207,7 +210,6 @@ k_factor(LevelGeom L, FineOp g, int is_fine, int nptsmax, const R* __restrict__ 
     // (B) trailing update of the entries (r, c), j < c <= r; entry e of a trailing triangle lies
     // in row r = j + m with (m-1) m / 2 <= e < m (m+1) / 2.  e = 0 is the next pivot: its thread
     // finishes it first and computes the reciprocal square root (lookahead).
-    const int m1 = NPAD - 1 - j;
     const int T = m1 * (m1 + 1) / 2;
     for (int t = tid; t < MPC * T; t += kFactorThreads) {
       const int mi = t / T, e = t - mi * T;

@@ -360,6 +360,9 @@ extern "C" la_status la_init(const la_config* cfg, void* stream, la_ctx** out) {
     G.one_per_cta = k.factor_group == 1 ? 1 : 0;
     G.band = (l == 0 && k.local_form == 0 && G.npad > LA_NPAD_MAX) ? fine_band_blocks(k.dim, G.sub, k.nt, G.nblk)
                                                                   : G.nblk - 1;
+    // square form: M couples edge neighbours; finest least squares: H^2, two grid steps; Galerkin levels: box
+    G.reach = k.local_form == 1 ? matrix_reach(k.dim, G.sub, 1, 1)
+                                : (l == 0 ? matrix_reach(k.dim, G.sub, 2, 2) : matrix_reach(k.dim, G.sub, 6, 2));
   }
   if (!build_time_constants(c)) {
     g_init_error = "invalid configuration: singular time-basis Gram matrix";

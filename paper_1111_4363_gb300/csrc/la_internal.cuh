@@ -189,6 +189,7 @@ struct LevelGeom {
   // factor (no fill outside the envelope) vanish beyond the largest index distance of such a pair; the
   // wide (global-memory) factorisation and solves skip those blocks.  nblk - 1 where nothing is skipped.
   int band;
+  int reach;       // largest distance of two coupled points in the subvolume's x-fastest order (matrix_reach)
 };
 
 // Finest-level spatial operator: H = -1/2 Laplacian + V0, X = x along laser_axis.
@@ -320,6 +321,24 @@ __host__ inline int fine_band_blocks(int dim, const int sub[3], int K, int nblk)
       if ((LA_BLK * (J + d)) / K - (LA_BLK * J + LA_BLK - 1) / K <= maxd) band = d;
   if (band < 1) band = 1;
   return band < nblk - 1 ? band : nblk - 1;
+}
+
+// Largest distance, in the x-fastest point order of a subvolume of extent sub, of two points that an operator
+// couples: offsets of Manhattan length at most `man` and at most `box` per axis.  A Cholesky factor has no
+// entry further below its diagonal than that (no fill outside the envelope); ragged subvolumes have
+// shorter strides and stay inside it.
+__host__ inline int matrix_reach(int dim, const int sub[3], int man, int box) {
+  int reach = 0;
+  int m[3];
+  for (int a = 0; a < 3; ++a) m[a] = a < dim ? (sub[a] - 1 < box ? sub[a] - 1 : box) : 0;
+  for (int dz = -m[2]; dz <= m[2]; ++dz)
+    for (int dy = -m[1]; dy <= m[1]; ++dy)
+      for (int dx = -m[0]; dx <= m[0]; ++dx) {
+        if ((dx < 0 ? -dx : dx) + (dy < 0 ? -dy : dy) + (dz < 0 ? -dz : dz) > man) continue;
+        const int d = dx + sub[0] * dy + sub[0] * sub[1] * dz;
+        if (d > reach) reach = d;
+      }
+  return reach;
 }
 
 template <typename R> struct C2;
