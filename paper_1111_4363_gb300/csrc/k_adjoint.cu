@@ -76,41 +76,51 @@ __global__ void k_grad_partials(FineOp g, int K, const double2* __restrict__ zne
 
 // grad[j] += 2 h^d Re sum_{m,n'} E^(j)[m][n'] Z[m][n'], E^(j) = [Eb0^(j) | Eb^(j)] of the unit
 // component j at t0 (Gauss-Legendre quadrature as in the time matrices).  One block.
-__global__ void k_grad_final(const TimeMats* __restrict__ tm, double t0, double hd, const double2* __restrict__ partials,
-                             int nblocks, double* __restrict__ grad) {
-  __shared__ double2 Z[LA_KMAX * (LA_KMAX + 1)];
-  const int K = tm->K, npair = K * (K + 1);
-  for (int pr = threadIdx.x; pr < npair; pr += blockDim.x) {
-    double sx = 0.0, sy = 0.0;
-    for (int b = 0; b < nblocks; ++b) {
-      const double2 v = partials[(long long)pr * nblocks + b];
-      sx += v.x;
-      sy += v.y;
+// One warp per pair for the partial sums; then S_q = sum_m b_m(tau_q) (Z_m0 + sum_n b_n(tau_q) Z_mn) per Gauss node
+// and, per component, grad_j += 2 h^d (dt/2) sum_q w_q env_j(t_q) sin(omega_j t_q) S_q: the field of a component
+// is evaluated once per node (not once per node and pair: 493 us at 48x48x44 with 8 components, 20 pairs).
+__global__ void __launch_bounds__(256) k_grad_final(const TimeMats* __restrict__ tm, double t0, double hd,
+                                                    const double2* __restrict__ partials, int nblocks,
+                                                    double* __restrict__ grad) {
+  __shared__ double Z[LA_KMAX * (LA_KMAX + 1)];
+  __shared__ double S[LA_NQ_MAX];
+  __shared__ double acc[LA_NCOMP_MAX][LA_NQ_MAX];
+  const int K = tm->K, npair = K * (K + 1), nq = tm->nq, nc = tm->ncomp;
+  const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
+  const double dt = tm->dt;
+  for (int pr = w; pr < npair; pr += 8) {
+    double sx = 0.0;
+    for (int b = l; b < nblocks; b += 32) sx += partials[(long long)pr * nblocks + b].x;
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, m);
+    if (l == 0) Z[pr] = sx;
+  }
+  for (int i = tid; i < nc * nq; i += blockDim.x) {
+    const int j = i / nq, q = i - j * nq;
+    const double t = t0 + 0.5 * (tm->tau[q] + 1.0) * dt;
+    double env = 1.0;
+    if (tm->sigma[j] > 0.0) {
+      const double u = (t - tm->tc[j]) / tm->sigma[j];
+      env = exp(-u * u);
     }
-    Z[pr] = make_double2(sx, sy);
+    acc[j][q] = tm->wq[q] * env * sin(tm->omega[j] * t);
   }
   __syncthreads();
-  const double dt = tm->dt;
-  for (int j = threadIdx.x; j < tm->ncomp; j += blockDim.x) {
-    double acc = 0.0;
+  if (tid < nq) {
+    const double* bq = tm->bq + tid * LA_KMAX;
+    double s = 0.0;
     for (int m = 0; m < K; ++m) {
-      for (int nn = 0; nn <= K; ++nn) {
-        double e = 0.0;
-        for (int q = 0; q < tm->nq; ++q) {
-          const double t = t0 + 0.5 * (tm->tau[q] + 1.0) * dt;
-          double env = 1.0;
-          if (tm->sigma[j] > 0.0) {
-            const double u = (t - tm->tc[j]) / tm->sigma[j];
-            env = exp(-u * u);
-          }
-          const double fld = env * sin(tm->omega[j] * t);
-          const double bn = nn == 0 ? 1.0 : tm->bq[q * LA_KMAX + (nn - 1)];
-          e += tm->wq[q] * tm->bq[q * LA_KMAX + m] * bn * fld;
-        }
-        acc += 0.5 * dt * e * Z[m * (K + 1) + nn].x;
-      }
+      double e = Z[m * (K + 1)];
+      for (int n = 0; n < K; ++n) e += bq[n] * Z[m * (K + 1) + n + 1];
+      s += bq[m] * e;
     }
-    grad[j] += 2.0 * hd * acc;
+    S[tid] = 0.5 * dt * s;
+  }
+  __syncthreads();
+  if (tid < nc) {
+    double a = 0.0;
+    for (int q = 0; q < nq; ++q) a += acc[tid][q] * S[q];
+    grad[tid] += 2.0 * hd * a;
   }
 }
 
@@ -119,7 +129,7 @@ void launch_grad_contract(const FineOp& g, const TimeMats* tm, int K, double t0,
   const int np = g.n[0] * g.n[1] * g.n[2];
   dim3 grid((np + 255) / 256, K * (K + 1));
   k_grad_partials<<<grid, 256, 0, s>>>(g, K, zneg, psi, c, partials);
-  k_grad_final<<<1, 64, 0, s>>>(tm, t0, hd, partials, grid.x, grad);
+  k_grad_final<<<1, 256, 0, s>>>(tm, t0, hd, partials, grid.x, grad);
 }
 
 // lambda_p += h^d [ (H u)_p + x_p sum_m Eb0_m mu_pm ],  u_q = sum_m Ub0_m mu_qm, mu = -zneg

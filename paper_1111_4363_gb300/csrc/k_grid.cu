@@ -16,63 +16,100 @@ template <typename CT> __device__ __forceinline__ CT cmk(typename CR<CT>::R a, t
   CT r; r.x = a; r.y = b; return r;
 }
 
-// ------------------------------------------------------------------ time matrices (Sec. I, IV)
-// Eb[m,n] = (dt/2) sum_q w_q b_m(tau_q) b_n(tau_q) E(t_q), Eb0[m] = (dt/2) sum_q w_q b_m(tau_q) E(t_q),
-// P_kk' = R_k^T Wt R_k' with R = (Qb, Ub, Eb).  One block.
-__global__ void k_time_matrices(TimeMats* tm, double t0) {
-  __shared__ double Eq[LA_NQ_MAX];
-  __shared__ double R[3][LA_KMAX * LA_KMAX];
-  __shared__ double Wt[LA_KMAX * LA_KMAX];
-  const int K = tm->K, nq = tm->nq, KK = K * K;
-  const double dt = tm->dt;
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-    double t = t0 + 0.5 * (tm->tau[q] + 1.0) * dt;
-    double e = 0.0;
-    for (int k = 0; k < tm->ncomp; ++k) {
-      double env = 1.0;
-      if (tm->sigma[k] > 0.0) {
-        double u = (t - tm->tc[k]) / tm->sigma[k];
-        env = exp(-u * u);
-      }
-      e += tm->amp[k] * env * sin(tm->omega[k] * t);
+// Counts the CTAs of a launch that have finished their part; true in every thread of the last one, whose
+// reads see what the others wrote before.  The counter is 0 again after the launch.
+__device__ __forceinline__ bool last_cta(unsigned* count, unsigned ncta) {
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(count, 1u) + 1 == ncta;
+    if (last) {
+      *count = 0;
+      __threadfence();
     }
-    Eq[q] = e;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < KK; i += blockDim.x) {
-    int m = i / K, n = i % K;
-    double s = 0.0;
-    for (int q = 0; q < nq; ++q) s += tm->wq[q] * tm->bq[q * LA_KMAX + m] * tm->bq[q * LA_KMAX + n] * Eq[q];
-    s *= 0.5 * dt;
-    tm->Eb[i] = s;
-    R[2][i] = s;
+  return last;
+}
+
+// ------------------------------------------------------------------ time matrices (Sec. I, IV)
+// Eb[m,n] = (dt/2) sum_q w_q b_m(tau_q) b_n(tau_q) E(t_q), Eb0[m] = (dt/2) sum_q w_q b_m(tau_q) E(t_q),
+// P_kk' = R_k^T (Wt R_k') with R = (Qb, Ub, Eb).  With a field, CTA q evaluates E(t_q), one pulse component
+// per thread (FP64 exp and sin cost a few hundred instructions each and one SM issues two lanes a
+// clock, so the nodes go to different SMs), and the last CTA forms the matrices: 8 us with 32
+// components, against 67 us for one CTA with one thread per node.
+__global__ void __launch_bounds__(256) k_time_matrices(TimeMats* tm, double t0) {
+  __shared__ double Eq[LA_NQ_MAX], tau[LA_NQ_MAX], wq[LA_NQ_MAX], bq[LA_NQ_MAX][LA_KMAX];
+  __shared__ double R[3][LA_KMAX * LA_KMAX], WR[3][LA_KMAX * LA_KMAX], Wt[LA_KMAX * LA_KMAX];
+  __shared__ double part[LA_NCOMP_MAX];
+  const int tid = threadIdx.x, K = tm->K, nq = tm->nq, KK = K * K;
+  const double dt = tm->dt;
+  if (gridDim.x > 1) {
+    const int q = blockIdx.x, nc = tm->ncomp;
+    const double t = t0 + 0.5 * (tm->tau[q] + 1.0) * dt;
+    if (tid < nc) {
+      double env = 1.0;
+      if (tm->sigma[tid] > 0.0) {
+        const double u = (t - tm->tc[tid]) / tm->sigma[tid];
+        env = exp(-u * u);
+      }
+      part[tid] = tm->amp[tid] * env * sin(tm->omega[tid] * t);
+    }
+    __syncthreads();
+    if (tid == 0) {
+      double e = 0.0;
+      for (int k = 0; k < nc; ++k) e += part[k];
+      tm->Eq[q] = e;
+    }
+    if (!last_cta(&tm->done, gridDim.x)) return;
+  }
+  if (tid < nq) {
+    Eq[tid] = gridDim.x > 1 ? __ldcg(&tm->Eq[tid]) : 0.0;
+    tau[tid] = tm->tau[tid];
+    wq[tid] = tm->wq[tid];
+  }
+  for (int i = tid; i < nq * LA_KMAX; i += blockDim.x) bq[i / LA_KMAX][i % LA_KMAX] = tm->bq[i];
+  for (int i = tid; i < KK; i += blockDim.x) {
     R[0][i] = tm->Qb[i];
     R[1][i] = tm->Ub[i];
     Wt[i] = tm->Wt[i];
   }
-  for (int m = threadIdx.x; m < K; m += blockDim.x) {
+  __syncthreads();
+  for (int i = tid; i < KK; i += blockDim.x) {
+    const int m = i / K, n = i % K;
     double s = 0.0;
-    for (int q = 0; q < nq; ++q) s += tm->wq[q] * tm->bq[q * LA_KMAX + m] * Eq[q];
+    for (int q = 0; q < nq; ++q) s += wq[q] * bq[q][m] * bq[q][n] * Eq[q];
+    s *= 0.5 * dt;
+    tm->Eb[i] = s;
+    R[2][i] = s;
+  }
+  for (int m = blockDim.x - 1 - tid; m < K; m += blockDim.x) {
+    double s = 0.0;
+    for (int q = 0; q < nq; ++q) s += wq[q] * bq[q][m] * Eq[q];
     tm->Eb0[m] = 0.5 * dt * s;
   }
-  if (threadIdx.x == 0) tm->t0 = t0;
+  if (tid == 0) tm->t0 = t0;
   __syncthreads();
-  for (int i = threadIdx.x; i < LA_NPAIR * KK; i += blockDim.x) {
-    int kk = i / KK, mn = i % KK, m = mn / K, n = mn % K;
-    int k = kk / 3, kp = kk % 3;
+  for (int i = tid; i < 3 * KK; i += blockDim.x) {
+    const int k = i / KK, mn = i - k * KK, a = mn / K, n = mn % K;
+    double t = 0.0;
+    for (int b = 0; b < K; ++b) t += Wt[a * K + b] * R[k][b * K + n];
+    WR[k][mn] = t;
+  }
+  __syncthreads();
+  for (int i = tid; i < LA_NPAIR * KK; i += blockDim.x) {
+    const int kk = i / KK, mn = i - kk * KK, m = mn / K, n = mn % K;
+    const int k = kk / 3, kp = kk % 3;
     double s = 0.0;
-    for (int a = 0; a < K; ++a) {
-      double ra = R[k][a * K + m];
-      if (ra == 0.0) continue;
-      double t = 0.0;
-      for (int b = 0; b < K; ++b) t += Wt[a * K + b] * R[kp][b * K + n];
-      s += ra * t;
-    }
+    for (int a = 0; a < K; ++a) s += R[k][a * K + m] * WR[kp][a * K + n];
     tm->P[kk][mn] = s;
   }
 }
 
-void launch_time_matrices(TimeMats* tm, double t0, cudaStream_t s) { k_time_matrices<<<1, 256, 0, s>>>(tm, t0); }
+void launch_time_matrices(TimeMats* tm, int ncta, double t0, cudaStream_t s) {
+  k_time_matrices<<<ncta, 256, 0, s>>>(tm, t0);
+}
 
 // ------------------------------------------------------------------ fine-level stencil helpers
 __device__ __forceinline__ void pcoords(const FineOp& g, int p, int& x, int& y, int& z) {
@@ -95,6 +132,12 @@ __device__ __forceinline__ void load_k(const CT* __restrict__ v, long long p, CT
       out[2 * m] = cmk<CT>(q.x, q.y);
       out[2 * m + 1] = cmk<CT>(q.z, q.w);
     }
+  } else if constexpr (sizeof(CT) == 16 && K % 2 == 0) {   // records of 32 K / 2 bytes: full-sector accesses
+#pragma unroll
+    for (int m = 0; m < K; m += 2)
+      asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                   : "=d"(out[m].x), "=d"(out[m].y), "=d"(out[m + 1].x), "=d"(out[m + 1].y)
+                   : "l"(src + m));
   } else {
 #pragma unroll
     for (int m = 0; m < K; ++m) out[m] = src[m];
@@ -107,6 +150,12 @@ __device__ __forceinline__ void store_k(CT* __restrict__ v, long long p, const C
     float4* d4 = reinterpret_cast<float4*>(dst);
 #pragma unroll
     for (int m = 0; m < K / 2; ++m) d4[m] = make_float4(in[2 * m].x, in[2 * m].y, in[2 * m + 1].x, in[2 * m + 1].y);
+  } else if constexpr (sizeof(CT) == 16 && K % 2 == 0) {
+#pragma unroll
+    for (int m = 0; m < K; m += 2)
+      asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(dst + m), "d"(in[m].x), "d"(in[m].y), "d"(in[m + 1].x),
+                   "d"(in[m + 1].y)
+                   : "memory");
   } else {
 #pragma unroll
     for (int m = 0; m < K; ++m) dst[m] = in[m];
@@ -159,8 +208,9 @@ __device__ __forceinline__ void apply_H(const FineOp& g, const CT* __restrict__ 
   }
 
 // f~[p, m] = Ub0[m] (H psi0)_p + x_p Eb0[m] psi0_p (the psi0 P_0 part moved to the right-hand side).
-__global__ void k_rhs(FineOp g, const TimeMats* __restrict__ tm, const double2* __restrict__ psi0,
-                      double2* __restrict__ f) {
+template <int K>
+__global__ void __launch_bounds__(256) k_rhs(FineOp g, const TimeMats* __restrict__ tm,
+                                             const double2* __restrict__ psi0, double2* __restrict__ f) {
   int np = g.n[0] * g.n[1] * g.n[2];
   int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= np) return;
@@ -169,36 +219,88 @@ __global__ void k_rhs(FineOp g, const TimeMats* __restrict__ tm, const double2* 
   double2 hp[1], pv[1];
   apply_H<double2, double, 1>(g, psi0, p, x, y, z, pv, hp);
   const double xl = fine_x(g, x, y, z);
-  const double2 ps = pv[0];
-  const int K = tm->K;
+  const double2 ps = make_double2(xl * pv[0].x, xl * pv[0].y);
+  double2 out[K];
+#pragma unroll
   for (int m = 0; m < K; ++m) {
-    double a = tm->Ub0[m], b = xl * tm->Eb0[m];
-    f[(long long)p * K + m] = make_double2(a * hp[0].x + b * ps.x, a * hp[0].y + b * ps.y);
+    const double a = tm->Ub0[m], b = tm->Eb0[m];
+    out[m] = make_double2(a * hp[0].x + b * ps.x, a * hp[0].y + b * ps.y);
   }
+  store_k<double2, K>(f, p, out);
 }
 
-void launch_rhs(const FineOp& g, const TimeMats* tm, const double2* psi0, double2* f, cudaStream_t s) {
+void launch_rhs(const FineOp& g, const TimeMats* tm, int K, const double2* psi0, double2* f, cudaStream_t s) {
   int np = g.n[0] * g.n[1] * g.n[2];
-  k_rhs<<<(np + 255) / 256, 256, 0, s>>>(g, tm, psi0, f);
+#define LA_CALL(KK) k_rhs<KK><<<(np + 255) / 256, 256, 0, s>>>(g, tm, psi0, f)
+  LA_K_DISPATCH(K, LA_CALL)
+#undef LA_CALL
 }
 
 int norm_blocks(int np) { return (np + 255) / 256; }
 
-// r = f~ - M~ c with (M~ c)_p = i Qb c_p - Ub (H c)_p - x_p Eb c_p; z = Wt r; partials of r^dagger Wt r.
-// One thread per point, 256 threads per block, no grid stride (fixed block-to-point map so the
-// norm reduction is deterministic).  f may be null (f = 0).  K is a template parameter so the
-// per-point K-vectors live in registers.
-template <typename CT, int K>
-__global__ void __launch_bounds__(256) k_mresid(FineOp g, const TimeMats* __restrict__ tm,
-                                                const CT* __restrict__ f, const CT* __restrict__ c,
-                                                CT* __restrict__ rout, CT* __restrict__ zout,
-                                                double* __restrict__ partials) {
-  typedef typename CR<CT>::R RR;
-  __shared__ RR Qb[K * K], Ub[K * K], Eb[K * K], Wt[K * K];
-  __shared__ double red[256];
-  for (int i = threadIdx.x; i < K * K; i += blockDim.x) {
-    Qb[i] = (RR)tm->Qb[i]; Ub[i] = (RR)tm->Ub[i]; Eb[i] = (RR)tm->Eb[i]; Wt[i] = (RR)tm->Wt[i];
+// Products with the static time matrices in closed form, s_m = (-1)^m, m = 1..K (index m - 1):
+//   Ub = dt (diag(1/(2m+1)) + s s^T);   Qb[m][n] = 2 [n > m, n - m odd] - s_m (1 - s_n);
+//   Ub^{-1} = (1/dt) (D - D s s^T D / (K+1)^2), D = diag(2m+1)   (sum_m D_m = K (K+2)).
+// A product costs 2 to 3 K operations instead of K^2: the FP64 residual is bound by FP64 issue.
+template <int K>
+struct TimeProducts {
+  static __device__ __forceinline__ constexpr double sgn(int i) { return (i & 1) ? 1.0 : -1.0; }   // s_{i+1}
+  // out += Ub v (real vectors)
+  static __device__ __forceinline__ void add_U(double dt, const double (&v)[K], double (&out)[K]) {
+    double S = 0.0;
+#pragma unroll
+    for (int n = 0; n < K; ++n) S += sgn(n) * v[n];
+    S *= dt;
+#pragma unroll
+    for (int m = 0; m < K; ++m) out[m] = fma(dt * (1.0 / (2 * m + 3)), v[m], out[m] + sgn(m) * S);
   }
+  // out += sign Qb v
+  static __device__ __forceinline__ void add_Q(double sign, const double (&v)[K], double (&out)[K]) {
+    double odd = 0.0;   // sum over odd n (index even)
+#pragma unroll
+    for (int n = 0; n < K; n += 2) odd += v[n];
+    double tail[2] = {0.0, 0.0};   // sums of v over n > m of each parity of the index
+#pragma unroll
+    for (int m = K - 1; m >= 0; --m) {
+      out[m] = fma(2.0 * sign, tail[(m + 1) & 1] - sgn(m) * odd, out[m]);
+      tail[m & 1] += v[m];
+    }
+  }
+  // v = Wt v
+  static __device__ __forceinline__ void weight(int kind, double dt, double idt, const double (&v)[K], double (&out)[K]) {
+    if (kind == 0) {
+      double T = 0.0;
+#pragma unroll
+      for (int n = 0; n < K; ++n) T = fma(sgn(n) * (2 * n + 3) / ((K + 1.0) * (K + 1.0)), v[n], T);
+#pragma unroll
+      for (int m = 0; m < K; ++m) out[m] = idt * (2 * m + 3) * (v[m] - sgn(m) * T);
+    } else if (kind == 1) {
+#pragma unroll
+      for (int m = 0; m < K; ++m) out[m] = 0.0;
+      add_U(dt, v, out);
+    } else {
+#pragma unroll
+      for (int m = 0; m < K; ++m) out[m] = v[m];
+    }
+  }
+};
+
+// FP64: r = f~ - M~ c with (M~ c)_p = i Qb c_p - Ub (H c)_p - x_p Eb c_p; z = Wt r; N = nscale r^dagger Wt r.
+// One thread per point, 256 threads per block, no grid stride: the partial sums of the blocks are added by
+// the last block in a fixed order, so the norm is deterministic.  f may be null (f = 0), and c (c = 0, r = f).
+// K is a template parameter so the per-point K-vectors live in registers.
+// 128^3, K = 4: 0.84 ms with r stored, bound by FP64 issue (about 195 operations per point).  In mixed
+// precision the complex64 copy replaces the FP64 residual and the pass that rounded it.
+template <int K>
+__global__ void __launch_bounds__(256) k_residual(FineOp g, const TimeMats* __restrict__ tm,
+                                                  const double2* __restrict__ f, const double2* __restrict__ c,
+                                                  double2* __restrict__ zout, ResidOut out) {
+  typedef TimeProducts<K> TP;
+  __shared__ double Eb[K * K];
+  __shared__ double red[256];
+  for (int i = threadIdx.x; i < K * K; i += blockDim.x) Eb[i] = tm->Eb[i];
+  const double dt = tm->dt, idt = 1.0 / dt;
+  const int kind = tm->weight;
   __syncthreads();
   const int np = g.n[0] * g.n[1] * g.n[2];
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -206,52 +308,142 @@ __global__ void __launch_bounds__(256) k_mresid(FineOp g, const TimeMats* __rest
   if (p < np) {
     int x, y, z;
     pcoords(g, p, x, y, z);
-    CT r[K];
-    if (f) load_k<CT, K>(f, p, r);
-    else {
+    double rx[K], ry[K];
+    double2 v[K];
+    if (f) {
+      load_k<double2, K>(f, p, v);
 #pragma unroll
-      for (int m = 0; m < K; ++m) r[m] = cmk<CT>(0, 0);
+      for (int m = 0; m < K; ++m) { rx[m] = v[m].x; ry[m] = v[m].y; }
+    } else {
+#pragma unroll
+      for (int m = 0; m < K; ++m) rx[m] = ry[m] = 0.0;
     }
     if (c) {   // c absent: c = 0 and r = f, with no stencil to apply
-      CT cp[K], hc[K];
-      apply_H<CT, RR, K>(g, c, p, x, y, z, cp, hc);
-      const RR xl = (RR)fine_x(g, x, y, z);
+      double2 cp[K], hc[K];
+      apply_H<double2, double, K>(g, c, p, x, y, z, cp, hc);
+      const double xl = fine_x(g, x, y, z);
+      double cx[K], cy[K], hx[K], hy[K];
+#pragma unroll
+      for (int m = 0; m < K; ++m) { cx[m] = cp[m].x; cy[m] = cp[m].y; hx[m] = hc[m].x; hy[m] = hc[m].y; }
+      // -i Qb c = Qb c.y - i Qb c.x
+      TP::add_Q(1.0, cy, rx);
+      TP::add_Q(-1.0, cx, ry);
+      TP::add_U(dt, hx, rx);
+      TP::add_U(dt, hy, ry);
 #pragma unroll
       for (int m = 0; m < K; ++m) {
-        RR qr = 0, qi = 0, ur = 0, ui = 0, er = 0, ei = 0;
+        double er = 0, ei = 0;
 #pragma unroll
         for (int n = 0; n < K; ++n) {
-          const RR q = Qb[m * K + n], u = Ub[m * K + n], e = Eb[m * K + n];
-          qr += q * cp[n].x; qi += q * cp[n].y;
-          ur += u * hc[n].x; ui += u * hc[n].y;
-          er += e * cp[n].x; ei += e * cp[n].y;
+          const double e = Eb[m * K + n];
+          er = fma(e, cx[n], er);
+          ei = fma(e, cy[n], ei);
         }
-        // i (qr + i qi) = -qi + i qr
-        r[m].x = r[m].x - (-qi - ur - xl * er);
-        r[m].y = r[m].y - (qr - ui - xl * ei);
+        rx[m] = fma(xl, er, rx[m]);
+        ry[m] = fma(xl, ei, ry[m]);
       }
     }
-    CT zv[K];
+    if (zout || out.partials) {
+      double zx[K], zy[K];
+      TP::weight(kind, dt, idt, rx, zx);
+      TP::weight(kind, dt, idt, ry, zy);
+      if (out.partials)
 #pragma unroll
-    for (int m = 0; m < K; ++m) {
-      RR zr = 0, zi = 0;
+        for (int m = 0; m < K; ++m) nsum = fma(rx[m], zx[m], fma(ry[m], zy[m], nsum));
+      if (zout) {
 #pragma unroll
-      for (int n = 0; n < K; ++n) { zr += Wt[m * K + n] * r[n].x; zi += Wt[m * K + n] * r[n].y; }
-      zv[m] = cmk<CT>(zr, zi);
-      if (partials) nsum += (double)r[m].x * (double)zr + (double)r[m].y * (double)zi;
+        for (int m = 0; m < K; ++m) v[m] = make_double2(zx[m], zy[m]);
+        store_k<double2, K>(zout, p, v);
+      }
     }
-    if (zout) store_k<CT, K>(zout, p, zv);
-    if (rout) store_k<CT, K>(rout, p, r);
+    if (out.r) {
+#pragma unroll
+      for (int m = 0; m < K; ++m) v[m] = make_double2(out.rscale * rx[m], out.rscale * ry[m]);
+      store_k<double2, K>(out.r, p, v);
+    }
+    if (out.r32) {
+      float2 w[K];
+#pragma unroll
+      for (int m = 0; m < K; ++m) w[m] = make_float2((float)rx[m], (float)ry[m]);
+      store_k<float2, K>(out.r32, p, w);
+#pragma unroll
+      for (int m = 0; m < K; ++m) w[m] = make_float2(0.f, 0.f);
+      if (out.zero32) store_k<float2, K>(out.zero32, p, w);
+    }
   }
-  if (partials) {
+  if (out.partials) {
     red[threadIdx.x] = nsum;
     __syncthreads();
     for (int s = 128; s > 0; s >>= 1) {
       if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
       __syncthreads();
     }
-    if (threadIdx.x == 0) partials[blockIdx.x] = red[0];
+    if (threadIdx.x == 0) out.partials[blockIdx.x] = red[0];
+    if (!last_cta(out.count, gridDim.x)) return;
+    double s = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) s += __ldcg(out.partials + i);
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int k = 128; k > 0; k >>= 1) {
+      if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+      *out.N = red[0] * out.nscale;
+      if (out.N_host) *out.N_host = red[0] * out.nscale;
+    }
   }
+}
+void launch_residual(const FineOp& g, const TimeMats* tm, int K, const double2* f, const double2* c, double2* z,
+                     const ResidOut& out, cudaStream_t s) {
+  const int nb = norm_blocks(g.n[0] * g.n[1] * g.n[2]);
+#define LA_CALL(KK) k_residual<KK><<<nb, 256, 0, s>>>(g, tm, f, c, z, out)
+  LA_K_DISPATCH(K, LA_CALL)
+#undef LA_CALL
+}
+
+// complex64 z = Wt (f - M~ c) of fields without a tensor map (1D grids, odd K); f may be null.
+template <int K>
+__global__ void __launch_bounds__(256) k_mresid(FineOp g, const TimeMats* __restrict__ tm, const float2* __restrict__ f,
+                                                const float2* __restrict__ c, float2* __restrict__ zout) {
+  __shared__ float Qb[K * K], Ub[K * K], Eb[K * K], Wt[K * K];
+  for (int i = threadIdx.x; i < K * K; i += blockDim.x) {
+    Qb[i] = (float)tm->Qb[i]; Ub[i] = (float)tm->Ub[i]; Eb[i] = (float)tm->Eb[i]; Wt[i] = (float)tm->Wt[i];
+  }
+  __syncthreads();
+  const int np = g.n[0] * g.n[1] * g.n[2];
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= np) return;
+  int x, y, z;
+  pcoords(g, p, x, y, z);
+  float2 r[K], cp[K], hc[K], zv[K];
+#pragma unroll
+  for (int m = 0; m < K; ++m) r[m] = make_float2(0.f, 0.f);
+  if (f) load_k<float2, K>(f, p, r);
+  apply_H<float2, float, K>(g, c, p, x, y, z, cp, hc);
+  const float xl = (float)fine_x(g, x, y, z);
+#pragma unroll
+  for (int m = 0; m < K; ++m) {
+    float qr = 0, qi = 0, ur = 0, ui = 0, er = 0, ei = 0;
+#pragma unroll
+    for (int n = 0; n < K; ++n) {
+      const float q = Qb[m * K + n], u = Ub[m * K + n], e = Eb[m * K + n];
+      qr += q * cp[n].x; qi += q * cp[n].y;
+      ur += u * hc[n].x; ui += u * hc[n].y;
+      er += e * cp[n].x; ei += e * cp[n].y;
+    }
+    // i (qr + i qi) = -qi + i qr
+    r[m].x = r[m].x - (-qi - ur - xl * er);
+    r[m].y = r[m].y - (qr - ui - xl * ei);
+  }
+#pragma unroll
+  for (int m = 0; m < K; ++m) {
+    float zr = 0, zi = 0;
+#pragma unroll
+    for (int n = 0; n < K; ++n) { zr += Wt[m * K + n] * r[n].x; zi += Wt[m * K + n] * r[n].y; }
+    zv[m] = make_float2(zr, zi);
+  }
+  store_k<float2, K>(zout, p, zv);
 }
 
 // ------------------------------------------------------------------ TMA-staged stencils (2D, 3D)
@@ -533,24 +725,21 @@ static bool launch_stencil_tma(const FineOp& g, const CUtensorMap* map, const Ti
   return true;
 }
 
-template <typename R>
-void launch_mresid(const FineOp& g, const TimeMats* tm, int K, const typename C2<R>::T* f,
-                   const typename C2<R>::T* c, typename C2<R>::T* r, typename C2<R>::T* z, double* partials, int nb,
-                   cudaStream_t s, const CUtensorMap* cmap, int* status) {
-  if constexpr (sizeof(R) == 4) {
-    // the complex64 V-cycle residual (z out only) of a field with a tensor map takes the TMA kernel
-    if (!r && !partials && z && launch_stencil_tma<false>(g, cmap, tm, K, f, z, nullptr, status, s)) return;
-  } else {
-    (void)cmap; (void)status;
-  }
-#define LA_CALL(KK) k_mresid<typename C2<R>::T, KK><<<nb, 256, 0, s>>>(g, tm, f, c, r, z, partials)
+template <>
+void launch_mresid<float>(const FineOp& g, const TimeMats* tm, int K, const float2* f, const float2* c, float2* z,
+                          cudaStream_t s, const CUtensorMap* cmap, int* status) {
+  // a field with a tensor map takes the TMA kernel
+  if (launch_stencil_tma<false>(g, cmap, tm, K, f, z, nullptr, status, s)) return;
+  const int nb = norm_blocks(g.n[0] * g.n[1] * g.n[2]);
+#define LA_CALL(KK) k_mresid<KK><<<nb, 256, 0, s>>>(g, tm, f, c, z)
   LA_K_DISPATCH(K, LA_CALL)
 #undef LA_CALL
 }
-template void launch_mresid<double>(const FineOp&, const TimeMats*, int, const double2*, const double2*, double2*,
-                                    double2*, double*, int, cudaStream_t, const CUtensorMap*, int*);
-template void launch_mresid<float>(const FineOp&, const TimeMats*, int, const float2*, const float2*, float2*,
-                                   float2*, double*, int, cudaStream_t, const CUtensorMap*, int*);
+template <>
+void launch_mresid<double>(const FineOp& g, const TimeMats* tm, int K, const double2* f, const double2* c, double2* z,
+                           cudaStream_t s, const CUtensorMap*, int*) {
+  launch_residual(g, tm, K, f, c, z, ResidOut{}, s);
+}
 
 // s = M~^dagger z: s_p = -i Qb^T z_p - Ub (H z)_p - x_p Eb z_p.
 template <typename CT, int K>
@@ -639,7 +828,8 @@ __device__ __forceinline__ bool parent_1d(int a, int t, int nc, bool used, int& 
 }
 
 template <typename CT, int K>
-__global__ void k_restrict(LevelGeom F, LevelGeom C, const CT* __restrict__ sf, CT* __restrict__ gc) {
+__global__ void k_restrict(LevelGeom F, LevelGeom C, const CT* __restrict__ sf, CT* __restrict__ gc,
+                           CT* __restrict__ ec) {
   typedef typename CR<CT>::R RR;
   const int J = blockIdx.x * blockDim.x + threadIdx.x;
   if (J >= C.np) return;
@@ -665,6 +855,9 @@ __global__ void k_restrict(LevelGeom F, LevelGeom C, const CT* __restrict__ sf, 
     }
   }
   store_k<CT, K>(gc, J, acc);
+#pragma unroll
+  for (int m = 0; m < K; ++m) acc[m] = cmk<CT>(0, 0);
+  store_k<CT, K>(ec, J, acc);
 }
 
 // Restriction I^T on 2D and 3D levels, one CTA per tile of kRx x kRy x kRz coarse points: the fine points the
@@ -674,7 +867,7 @@ __global__ void k_restrict(LevelGeom F, LevelGeom C, const CT* __restrict__ sf, 
 constexpr int kRx = 8, kRy = 4, kRz = 2;
 template <typename CT, int K>
 __global__ void __launch_bounds__(256) k_restrict_tile(LevelGeom F, LevelGeom C, const CT* __restrict__ sf,
-                                                       CT* __restrict__ gc) {
+                                                       CT* __restrict__ gc, CT* __restrict__ ec) {
   typedef typename CR<CT>::R RR;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CT* box = reinterpret_cast<CT*>(smem_raw);
@@ -718,7 +911,9 @@ __global__ void __launch_bounds__(256) k_restrict_tile(LevelGeom F, LevelGeom C,
         }
       }
     }
-    gc[((long long)(jz * C.n[1] + jy) * C.n[0] + jx) * K + m] = acc;
+    const long long at = ((long long)(jz * C.n[1] + jy) * C.n[0] + jx) * K + m;
+    gc[at] = acc;
+    ec[at] = cmk<CT>(0, 0);   // the level's relaxation starts from zero
   }
 }
 
@@ -752,7 +947,7 @@ __global__ void k_prolong_add(LevelGeom F, LevelGeom C, const CT* __restrict__ e
 
 template <typename R>
 void launch_restrict(const LevelGeom& F, const LevelGeom& C, int K, const typename C2<R>::T* sf,
-                     typename C2<R>::T* gc, cudaStream_t s) {
+                     typename C2<R>::T* gc, typename C2<R>::T* ec, cudaStream_t s) {
   typedef typename C2<R>::T CT;
   if (F.dim >= 2) {
     const int ty = kRy, tz = F.dim > 2 ? kRz : 1;
@@ -765,7 +960,7 @@ void launch_restrict(const LevelGeom& F, const LevelGeom& C, int K, const typena
       cudaFuncSetAttribute(k_restrict_tile<CT, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); \
       attr = true;                                                                                         \
     }                                                                                                      \
-    k_restrict_tile<CT, KK><<<grid, 256, smem, s>>>(F, C, sf, gc);                                         \
+    k_restrict_tile<CT, KK><<<grid, 256, smem, s>>>(F, C, sf, gc, ec);                                     \
   } while (0)
     switch (K) {
       case 1: LA_CALL(1); break;
@@ -780,7 +975,7 @@ void launch_restrict(const LevelGeom& F, const LevelGeom& C, int K, const typena
 #undef LA_CALL
     return;
   }
-#define LA_CALL(KK) k_restrict<typename C2<R>::T, KK><<<(C.np + 127) / 128, 128, 0, s>>>(F, C, sf, gc)
+#define LA_CALL(KK) k_restrict<typename C2<R>::T, KK><<<(C.np + 127) / 128, 128, 0, s>>>(F, C, sf, gc, ec)
   LA_K_DISPATCH(K, LA_CALL)
 #undef LA_CALL
 }
@@ -791,8 +986,10 @@ void launch_prolong_add(const LevelGeom& F, const LevelGeom& C, int K, const typ
   LA_K_DISPATCH(K, LA_CALL)
 #undef LA_CALL
 }
-template void launch_restrict<double>(const LevelGeom&, const LevelGeom&, int, const double2*, double2*, cudaStream_t);
-template void launch_restrict<float>(const LevelGeom&, const LevelGeom&, int, const float2*, float2*, cudaStream_t);
+template void launch_restrict<double>(const LevelGeom&, const LevelGeom&, int, const double2*, double2*, double2*,
+                                      cudaStream_t);
+template void launch_restrict<float>(const LevelGeom&, const LevelGeom&, int, const float2*, float2*, float2*,
+                                     cudaStream_t);
 template void launch_prolong_add<double>(const LevelGeom&, const LevelGeom&, int, const double2*, double2*,
                                          cudaStream_t);
 template void launch_prolong_add<float>(const LevelGeom&, const LevelGeom&, int, const float2*, float2*, cudaStream_t);
@@ -819,7 +1016,7 @@ void launch_norm_final(const double* partials, int n, double scale, double* out,
 // Trial or zero start of a step's relaxation, decided on the device: the extrapolated trial is kept when
 // its action is below N(0), else c = 0 and r = f (the residual of c = 0).
 __global__ void k_seed_select(long long n, const double* __restrict__ Nslot, int tried, LoopState* st,
-                              double2* __restrict__ c, double2* __restrict__ r, const double2* __restrict__ f) {
+                              double2* __restrict__ c, float2* __restrict__ r32, const double2* __restrict__ f) {
   const double Nt = Nslot[0], N0 = Nslot[1];
   const bool keep = tried && Nt < N0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -827,16 +1024,16 @@ __global__ void k_seed_select(long long n, const double* __restrict__ Nslot, int
     st->N = keep ? Nt : N0;
     st->cyc = 0;
   }
-  if (keep || !tried) return;   // without a trial c is already 0 and r = f
+  if (keep || !tried) return;   // without a trial c is already 0 and r32 = f
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     c[i] = make_double2(0.0, 0.0);
-    r[i] = f[i];
+    if (r32) r32[i] = make_float2((float)f[i].x, (float)f[i].y);
   }
 }
-void launch_seed_select(long long n, const double* Nslot, int tried, LoopState* st, double2* c, double2* r,
+void launch_seed_select(long long n, const double* Nslot, int tried, LoopState* st, double2* c, float2* r32,
                         const double2* f, cudaStream_t s) {
   const long long nb = std::min<long long>((n + 255) / 256, 4096);
-  k_seed_select<<<(int)nb, 256, 0, s>>>(n, Nslot, tried, st, c, r, f);
+  k_seed_select<<<(int)nb, 256, 0, s>>>(n, Nslot, tried, st, c, r32, f);
 }
 
 // The loop's condition (one thread): after a cycle, take its action and count it; continue while the

@@ -30,9 +30,9 @@ struct la_ctx {
   TimeMats* d_tm = nullptr;
   double* d_V0 = nullptr;
   // finest level, FP64
-  double2 *d_psi = nullptr, *d_f = nullptr, *d_c = nullptr, *d_r = nullptr, *d_z = nullptr, *d_s = nullptr;
+  double2 *d_psi = nullptr, *d_f = nullptr, *d_c = nullptr, *d_z = nullptr, *d_s = nullptr;
   // finest level, FP32 (mixed precision correction problem)
-  float2 *d_f32 = nullptr, *d_e32 = nullptr, *d_r32 = nullptr, *d_z32 = nullptr, *d_s32 = nullptr;
+  float2 *d_f32 = nullptr, *d_e32 = nullptr, *d_z32 = nullptr, *d_s32 = nullptr;
   // levels >= 1 (precision of the V-cycle), and factors of every level
   void* d_e[LA_MAX_LEVELS] = {};
   void* d_g[LA_MAX_LEVELS] = {};
@@ -44,6 +44,7 @@ struct la_ctx {
   double* d_gtab[2] = {};           // 1D Galerkin tables of two successive levels (la_set_hamiltonian)
   double* d_partials = nullptr;
   double* d_N = nullptr;
+  unsigned* d_count = nullptr;      // finished CTAs of a residual launch
   int* d_status = nullptr;
   int* d_perm = nullptr;            // square local form: row permutation of every finest factor
   int nparts = 0;
@@ -384,13 +385,11 @@ extern "C" la_status la_init(const la_config* cfg, void* stream, la_ctx** out) {
   ALLOC(c->d_psi, sizeof(double2) * c->np0);
   ALLOC(c->d_f, v64);
   ALLOC(c->d_c, v64);
-  ALLOC(c->d_r, v64);
   ALLOC(c->d_z, v64);
   ALLOC(c->d_s, v64);
   if (k.precision == 1) {
     ALLOC(c->d_f32, v32);
     ALLOC(c->d_e32, v32);
-    ALLOC(c->d_r32, v32);
     ALLOC(c->d_z32, v32);
     ALLOC(c->d_s32, v32);
   }
@@ -411,6 +410,7 @@ extern "C" la_status la_init(const la_config* cfg, void* stream, la_ctx** out) {
   c->nparts = norm_blocks(c->np0);
   ALLOC(c->d_partials, sizeof(double) * c->nparts);
   ALLOC(c->d_N, sizeof(double) * 2);
+  ALLOC(c->d_count, sizeof(unsigned));
   ALLOC(c->d_status, sizeof(int));
   if (k.local_form == 1) ALLOC(c->d_perm, sizeof(int) * (size_t)c->geo[0].nsub * c->geo[0].npad);
   for (int j = 0; j < k.trial; ++j) ALLOC(c->d_hist[j], sizeof(double2) * (size_t)c->nunk0);
@@ -431,6 +431,7 @@ extern "C" la_status la_init(const la_config* cfg, void* stream, la_ctx** out) {
   }
   cudaError_t e = cudaMemcpyAsync(c->d_tm, &c->htm, sizeof(TimeMats), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_count, 0, sizeof(unsigned), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_V0, 0, sizeof(double) * c->np0, c->stream);
   if (e != cudaSuccess) {
     la_finalize(c);
@@ -614,14 +615,12 @@ template <typename R> struct Fine;
 template <> struct Fine<double> {
   static double2* f(la_ctx* c) { return c->d_f; }
   static double2* e(la_ctx* c) { return c->d_c; }
-  static double2* r(la_ctx* c) { return c->d_r; }
   static double2* z(la_ctx* c) { return c->d_z; }
   static double2* s(la_ctx* c) { return c->d_s; }
 };
 template <> struct Fine<float> {
   static float2* f(la_ctx* c) { return c->d_f32; }
   static float2* e(la_ctx* c) { return c->d_e32; }
-  static float2* r(la_ctx* c) { return c->d_r32; }
   static float2* z(la_ctx* c) { return c->d_z32; }
   static float2* s(la_ctx* c) { return c->d_s32; }
 };
@@ -729,8 +728,8 @@ static la_status vcycle(la_ctx* c, int l) {
     // (adjoint mode: s = y - G~ e)
     cudaEvent_t e0, e1;
     const bool timed = prof_begin(c, &e0, &e1);
-    launch_mresid<R>(c->fine, c->d_tm, c->K, c->adj ? nullptr : Fine<R>::f(c), Fine<R>::e(c), nullptr, Fine<R>::z(c),
-                     nullptr, c->nparts, c->stream, stencil_map(c, Fine<R>::e(c)), c->d_status);
+    launch_mresid<R>(c->fine, c->d_tm, c->K, c->adj ? nullptr : Fine<R>::f(c), Fine<R>::e(c), Fine<R>::z(c), c->stream,
+                     stencil_map(c, Fine<R>::e(c)), c->d_status);
     if (timed) prof_end(c, e0, e1, sizeof(R) == 8 ? 1 : 2, resid_bytes(c, sizeof(CT), !c->adj));
     launch_mnormal<R>(c->fine, c->d_tm, c->K, Fine<R>::z(c), Fine<R>::s(c), c->stream,
                       c->adj ? (const CT*)c->adj_y : nullptr, stencil_map(c, Fine<R>::z(c)), c->d_status);
@@ -747,13 +746,12 @@ static la_status vcycle(la_ctx* c, int l) {
     // finest-level transfer timed for the roofline: s (fine) in, g (level 1) out
     cudaEvent_t e0, e1;
     const bool timed = l == 0 && prof_begin(c, &e0, &e1);
-    launch_restrict<R>(c->geo[l], c->geo[l + 1], c->K, sfine, (CT*)c->d_g[l + 1], c->stream);
+    launch_restrict<R>(c->geo[l], c->geo[l + 1], c->K, sfine, (CT*)c->d_g[l + 1], (CT*)c->d_e[l + 1], c->stream);
     if (timed)
       prof_end(c, e0, e1, 3, (double)sizeof(CT) * c->K * ((double)c->geo[0].np + (double)c->geo[1].np));
   }
   ++c->launches;
   LA_CHECK_LAUNCH(c);
-  LA_CUDA(c, cudaMemsetAsync(c->d_e[l + 1], 0, sizeof(CT) * (size_t)c->geo[l + 1].np * c->K, c->stream));
   LA_TRY(vcycle<R>(c, l + 1));
   CT* efine = l == 0 ? Fine<R>::e(c) : (CT*)c->d_e[l];
   {
@@ -769,19 +767,25 @@ static la_status vcycle(la_ctx* c, int l) {
   return sweep_level<R>(c, l, nu2);
 }
 
-// N of the current FP64 iterate into h_N[slot] (stores r~ = f~ - M~ c in d_r); enqueue only.  zero_c:
-// the iterate is known to be c = 0, so r~ = f~ and no stencil is applied.
+// N of the current FP64 iterate into d_N[slot] and (unless device_norm) h_N[slot]; enqueue only.  zero_c: the
+// iterate is known to be c = 0, so r~ = f~ and no stencil is applied.  In mixed precision the residual
+// r~ = f~ - M~ c, rounded to complex64, becomes the right-hand side of the next correction problem
+// (d_f32), whose start d_e32 is set to zero.
 static la_status action_enqueue(la_ctx* c, int slot = 0, bool zero_c = false) {
   cudaEvent_t e0, e1;
   const bool timed = !zero_c && prof_begin(c, &e0, &e1);   // the stencil launches carry the roofline
-  launch_mresid<double>(c->fine, c->d_tm, c->K, c->d_f, zero_c ? nullptr : c->d_c, c->d_r, nullptr, c->d_partials,
-                        c->nparts, c->stream);
+  ResidOut o;
+  o.r32 = c->d_f32;
+  o.zero32 = c->d_e32;
+  o.partials = c->d_partials;
+  o.nscale = c->nscale;
+  o.N = c->d_N + slot;
+  o.N_host = c->device_norm ? nullptr : c->h_N + slot;
+  o.count = c->d_count;
+  launch_residual(c->fine, c->d_tm, c->K, c->d_f, zero_c ? nullptr : c->d_c, nullptr, o, c->stream);
   if (timed) prof_end(c, e0, e1, 1, resid_bytes(c, sizeof(double2), true));
-  launch_norm_final(c->d_partials, c->nparts, c->nscale, c->d_N + slot, c->stream);
-  c->launches += 2;
+  c->launches += 1;
   LA_CHECK_LAUNCH(c);
-  if (!c->device_norm)
-    LA_CUDA(c, cudaMemcpyAsync(c->h_N + slot, c->d_N + slot, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   return LA_OK;
 }
 // N of the current FP64 iterate; synchronises.
@@ -797,12 +801,10 @@ static la_status cycle_body(la_ctx* c) {
   if (c->cfg.precision == 0) {
     LA_TRY(vcycle<double>(c, 0));
   } else {
-    // refinement: correction problem M~ e = r~ (r~ from the last action evaluation) in complex64
-    launch_c128_to_c64(c->nunk0, c->d_r, c->d_f32, c->stream);
-    LA_CUDA(c, cudaMemsetAsync(c->d_e32, 0, sizeof(float2) * (size_t)c->nunk0, c->stream));
+    // refinement: correction problem M~ e = r~ in complex64 (r~ and e = 0 from the last action evaluation)
     LA_TRY(vcycle<float>(c, 0));
     launch_axpy_c64_to_c128(c->nunk0, c->d_e32, c->d_c, c->stream);
-    c->launches += 2;
+    c->launches += 1;
     LA_CHECK_LAUNCH(c);
   }
   return action_enqueue(c);
@@ -869,10 +871,13 @@ static la_status run_cycle(la_ctx* c, double* N) {
   return cycle_complete(c, N);
 }
 
+// CTAs of k_time_matrices: one per Gauss node where there is a field to evaluate
+static int time_ctas(const la_ctx* c) { return c->htm.ncomp > 0 ? c->htm.nq : 1; }
+
 // time matrices and right-hand side for initial state d_psi at t0
 static la_status setup_step(la_ctx* c, double t0) {
-  launch_time_matrices(c->d_tm, t0, c->stream);
-  launch_rhs(c->fine, c->d_tm, c->d_psi, c->d_f, c->stream);
+  launch_time_matrices(c->d_tm, time_ctas(c), t0, c->stream);
+  launch_rhs(c->fine, c->d_tm, c->K, c->d_psi, c->d_f, c->stream);
   c->launches += 2;
   LA_CHECK_LAUNCH(c);
   return LA_OK;
@@ -895,7 +900,8 @@ static la_status hist_push(la_ctx* c) {
 }
 
 // Enqueue the starting iterate of a step: N(0) into h_N[1]; with a history (and use_trial) the
-// extrapolated trial into d_c and its action into h_N[0].  d_r ends as the residual of d_c.
+// extrapolated trial into d_c and its action into h_N[0].  In mixed precision d_f32 ends as the
+// residual of d_c.
 static la_status seed_enqueue(la_ctx* c, bool use_trial, bool* tried) {
   LA_CUDA(c, cudaMemsetAsync(c->d_c, 0, sizeof(double2) * (size_t)c->nunk0, c->stream));
   LA_TRY(action_enqueue(c, 1, true));
@@ -1023,7 +1029,7 @@ static la_status adjoint_solve(la_ctx* c, int* cycles) {
   const int nb = (int)std::min<long long>((n + 255) / 256, 4096);
   LA_CUDA(c, cudaMemsetAsync(c->d_c, 0, sizeof(double2) * (size_t)n, c->stream));
   auto rho_norm = [&](double* out) -> la_status {
-    launch_mresid<double>(c->fine, c->d_tm, c->K, nullptr, c->d_c, nullptr, c->d_z, nullptr, c->nparts, c->stream);
+    launch_mresid<double>(c->fine, c->d_tm, c->K, nullptr, c->d_c, c->d_z, c->stream);
     launch_mnormal<double>(c->fine, c->d_tm, c->K, c->d_z, c->d_rho, c->stream, c->d_y);
     launch_norm2_partials(n, c->d_rho, c->d_partials, std::min(nb, c->nparts), c->stream);
     launch_norm_final(c->d_partials, std::min(nb, c->nparts), 1.0, c->d_N, c->stream);
@@ -1333,7 +1339,7 @@ extern "C" la_status la_step_batch(la_ctx* const* ctxs, int nctx, void* const* p
         c->device_norm = false;
       }
       if (st == LA_OK) {
-        launch_seed_select(c->nunk0, c->d_N, tried ? 1 : 0, c->d_lstate, c->d_c, c->d_r, c->d_f, c->stream);
+        launch_seed_select(c->nunk0, c->d_N, tried ? 1 : 0, c->d_lstate, c->d_c, c->d_f32, c->d_f, c->stream);
         const cudaError_t e = cudaGraphLaunch(c->loop_exec, c->stream);
         if (e != cudaSuccess) st = fail(c, LA_ECUDA, "relaxation loop launch: %s", cudaGetErrorString(e));
       }
@@ -1426,18 +1432,36 @@ extern "C" la_status la_residual(la_ctx* c, const void* psi0, double t0, const v
   if (!c || !psi0 || !cin) return c ? fail(c, LA_EINVAL, "invalid argument") : LA_EINVAL;
   if (!c->have_ham) return fail(c, LA_ESTATE, "la_set_hamiltonian must be called first");
   LA_TRY(load_any(c, c->d_psi, psi0, sizeof(double2) * (size_t)c->np0));
-  LA_TRY(load_any(c, c->d_c, cin, sizeof(double2) * (size_t)c->nunk0));
-  LA_TRY(setup_step(c, t0));
-  double N = 0.0;
-  LA_TRY(action_now(c, &N));
-  if (action) *action = N;
-  if (r_out) {
-    // the kernels work with r~ = r / h^d (overlap factor O = h^d dropped); return the paper's r
-    launch_scale_c128(c->nunk0, c->hd, c->d_r, c->d_z, c->stream);
-    LA_CHECK_LAUNCH(c);
-    LA_TRY(store_any(c, r_out, c->d_z, sizeof(double2) * (size_t)c->nunk0));
+  // coefficients and residual that live on the device, aligned as the kernel reads them, are used in place
+  const auto in_place = [](const void* p) { return is_device_ptr(p) && (reinterpret_cast<uintptr_t>(p) & 31) == 0; };
+  const size_t cb = sizeof(double2) * (size_t)c->nunk0;
+  const double2* cd = (const double2*)cin;
+  const unsigned char *c0 = (const unsigned char*)cin, *r0 = (const unsigned char*)r_out;
+  const bool overlap = r_out && c0 < r0 + cb && r0 < c0 + cb;   // the kernel reads c's neighbours while it writes r
+  if (!in_place(cin) || overlap) {
+    LA_TRY(load_any(c, c->d_c, cin, cb));
+    cd = c->d_c;
   }
+  LA_TRY(setup_step(c, t0));
+  // the kernels work with r~ = r / h^d (overlap factor O = h^d dropped); return the paper's r
+  const bool direct = r_out && in_place(r_out);
+  ResidOut o;
+  o.r = r_out ? (direct ? (double2*)r_out : c->d_z) : nullptr;
+  o.rscale = c->hd;
+  o.partials = c->d_partials;
+  o.nscale = c->nscale;
+  o.N = c->d_N;
+  o.N_host = c->h_N;
+  o.count = c->d_count;
+  cudaEvent_t e0, e1;
+  const bool timed = prof_begin(c, &e0, &e1);
+  launch_residual(c->fine, c->d_tm, c->K, c->d_f, cd, nullptr, o, c->stream);
+  if (timed) prof_end(c, e0, e1, 1, resid_bytes(c, sizeof(double2), true));
+  ++c->launches;
+  LA_CHECK_LAUNCH(c);
+  if (r_out && !direct) LA_TRY(store_any(c, r_out, c->d_z, cb));
   LA_CUDA(c, cudaStreamSynchronize(c->stream));
+  if (action) *action = *c->h_N;
   return LA_OK;
 }
 
@@ -1479,7 +1503,7 @@ extern "C" la_status la_relax_colour(la_ctx* c, const void* psi0, double t0, int
 
 extern "C" la_status la_time_matrices(la_ctx* c, double t0, double* out) {
   if (!c || !out) return LA_EINVAL;
-  launch_time_matrices(c->d_tm, t0, c->stream);
+  launch_time_matrices(c->d_tm, time_ctas(c), t0, c->stream);
   LA_CHECK_LAUNCH(c);
   TimeMats t;
   LA_CUDA(c, cudaMemcpyAsync(&t, c->d_tm, sizeof(TimeMats), cudaMemcpyDeviceToHost, c->stream));

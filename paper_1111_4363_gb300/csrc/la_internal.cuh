@@ -39,6 +39,7 @@ struct TimeMats {
   int K;
   int nq;
   double dt;
+  int weight;                     // residual-norm weight: 0 = Ub^{-1}, 1 = Ub, 2 = identity
   double Qb[LA_KMAX * LA_KMAX];   // int b_m b_n'          (test m, trial n)
   double Ub[LA_KMAX * LA_KMAX];   // (dt/2) int b_m b_n
   double Wt[LA_KMAX * LA_KMAX];   // time part of the residual-norm weight
@@ -53,6 +54,8 @@ struct TimeMats {
   double Eb[LA_KMAX * LA_KMAX];
   double Eb0[LA_KMAX];
   double P[LA_NPAIR][LA_KMAX * LA_KMAX];  // R_k^T Wt R_k', R = (Qb, Ub, Eb)
+  double Eq[LA_NQ_MAX];           // E(t_q), scratch of k_time_matrices
+  unsigned done;                  // its finished CTAs (0 between launches)
 };
 // Theta_kk' = phase_kk' * P_kk' with phase = conj(alpha_k) alpha_k', alpha = (i, -1, -1):
 // (0,0) -> 1, (0,1),(0,2) -> +i, (1,0),(2,0) -> -i, others 1.
@@ -119,6 +122,7 @@ __host__ inline bool fill_time_constants(int K, double dt, int weight, TimeMats&
   memset(&t, 0, sizeof t);
   t.K = K;
   t.dt = dt;
+  t.weight = weight;
   for (int m = 1; m <= K; ++m) {
     const double sm = (m % 2) ? -1.0 : 1.0;
     t.Ub0[m - 1] = -sm * dt;
@@ -347,13 +351,25 @@ template <> struct C2<float> { typedef float2 T; };
 
 // ---------------------------------------------------------------- launch wrappers
 // time basis
-void launch_time_matrices(TimeMats* tm, double t0, cudaStream_t s);
+void launch_time_matrices(TimeMats* tm, int ncta, double t0, cudaStream_t s);   // ncta: 1 without a field, else nq
 // grid kernels (FP64 unless noted)
-void launch_rhs(const FineOp& g, const TimeMats* tm, const double2* psi0, double2* f, cudaStream_t s);
+void launch_rhs(const FineOp& g, const TimeMats* tm, int K, const double2* psi0, double2* f, cudaStream_t s);
+// What the FP64 residual kernel writes besides z: each pointer may be null.
+struct ResidOut {
+  double2* r = nullptr;         // the residual times rscale
+  double rscale = 1.0;
+  float2* r32 = nullptr;        // the residual rounded to complex64, the right-hand side of a correction problem
+  float2* zero32 = nullptr;     // set to zero: the correction's start
+  double* partials = nullptr;   // with the four below: N = nscale r^dagger Wt r, summed by the last CTA
+  double nscale = 0.0;
+  double *N = nullptr, *N_host = nullptr;   // device result and, if not null, a host-mapped copy
+  unsigned* count = nullptr;    // CTAs that finished (0 between launches)
+};
+void launch_residual(const FineOp& g, const TimeMats* tm, int K, const double2* f, const double2* c, double2* z,
+                     const ResidOut& out, cudaStream_t s);
 template <typename R>
 void launch_mresid(const FineOp& g, const TimeMats* tm, int K, const typename C2<R>::T* f, const typename C2<R>::T* c,
-                   typename C2<R>::T* r, typename C2<R>::T* z, double* partials, int nblocks_norm, cudaStream_t s,
-                   const CUtensorMap* cmap = nullptr, int* status = nullptr);
+                   typename C2<R>::T* z, cudaStream_t s, const CUtensorMap* cmap = nullptr, int* status = nullptr);
 template <typename R>
 void launch_mnormal(const FineOp& g, const TimeMats* tm, int K, const typename C2<R>::T* z, typename C2<R>::T* out,
                     cudaStream_t s, const typename C2<R>::T* yadd = nullptr, const CUtensorMap* zmap = nullptr,
@@ -369,7 +385,7 @@ void launch_lambda_update(const FineOp& g, const TimeMats* tm, double hd, const 
                           cudaStream_t s);
 template <typename R>
 void launch_restrict(const LevelGeom& fine, const LevelGeom& coarse, int K, const typename C2<R>::T* sf,
-                     typename C2<R>::T* gc, cudaStream_t s);
+                     typename C2<R>::T* gc, typename C2<R>::T* ec, cudaStream_t s);   // also sets ec = 0
 template <typename R>
 void launch_prolong_add(const LevelGeom& fine, const LevelGeom& coarse, int K, const typename C2<R>::T* ec,
                         typename C2<R>::T* ef, cudaStream_t s);
@@ -394,8 +410,8 @@ struct LoopRecord {
   int cycles, pad;
 };
 // keep the trial (c from the extrapolation) when its action Nslot[0] is below N(0) = Nslot[1], else c = 0
-// and r = f; initialises the loop state
-void launch_seed_select(long long n, const double* Nslot, int tried, LoopState* st, double2* c, double2* r,
+// and (r32 not null) r32 = f; initialises the loop state
+void launch_seed_select(long long n, const double* Nslot, int tried, LoopState* st, double2* c, float2* r32,
                         const double2* f, cudaStream_t s);
 // sets the loop's condition: first = 1 before the first cycle, else after a cycle (N from Nnew[0], cycle
 // counted); continue while N is finite, below max_cycles and (when check) above tol N(0)

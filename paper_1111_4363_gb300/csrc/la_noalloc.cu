@@ -278,7 +278,7 @@ extern "C" la_status la_action_noalloc(const la_config* cfg, const double* V0, c
   const double nscale = k.weight == 0 ? hd : (k.weight == 1 ? hd * hd * hd : hd * hd);
   cudaError_t e = cudaMemcpyAsync(tm, &htm, sizeof(TimeMats), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) {
-    launch_time_matrices(tm, t0, s);
+    launch_time_matrices(tm, nc > 0 ? htm.nq : 1, t0, s);
     k_action_partials<<<nblocks, kThreads, 0, s>>>(g, tm, static_cast<const double2*>(psi0),
                                                    static_cast<const double2*>(c), partials);
     launch_norm_final(partials, nblocks, nscale, d_N, s);
