@@ -98,8 +98,9 @@ typedef struct {
                            most 96 unknowns per subvolume; la_backward rejects it (LA_EINVAL) */
   int factor_group;     /* CTA packing of the shared-memory subvolume factorisations (up to 128 unknowns):
                            0 = several small matrices per CTA on levels of 512 or more subvolumes (8 up to
-                           32 unknowns, 2 up to 64; complex64: 4 up to 32, 2 up to 48), chosen by size;
-                           1 = one matrix per CTA on every level */
+                           32 unknowns, 2 up to 64; complex64: 2 up to 48, and up to 32 unknowns four warps
+                           of one or two matrices each on levels of 1216 or more), chosen by size;
+                           1 = one matrix (complex64 up to 32 unknowns: one warp) per CTA on every level */
 } la_config;
 
 /* Laser field E(t) = sum_k amp[k] * env_k(t) * sin(omega[k] t), env_k = exp(-((t - t_center[k])/sigma[k])^2)

@@ -283,8 +283,8 @@ k_factor(LevelGeom L, FineOp g, int is_fine, int nptsmax, const R* __restrict__ 
 // broadcasts, column reads are consecutive), so the per-entry bookkeeping is paid once per 16
 // columns instead of once per column.
 // Matrices per CTA of the blocked factorisation: small ones share the column barriers (their
-// per-thread register tiles stay small: NT = 3 complex for NPAD 32, 6 for NPAD 48).
-__host__ __device__ constexpr int factor_c64_mpc(int npad) { return npad <= 32 ? 4 : (npad <= 48 ? 2 : 1); }
+// per-thread register tiles stay small: NT = 6 complex for NPAD 48).  Up to 32 unknowns: k_factor_small.
+__host__ __device__ constexpr int factor_c64_mpc(int npad) { return npad <= 48 ? 2 : 1; }
 
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
@@ -1810,6 +1810,79 @@ __device__ __forceinline__ void subvol_solve_super(const float2* __restrict__ F,
   }
 }
 
+// Solves with the stored inverse X = inv(L) of a complex64 factor of at most 32 unknowns (factor_is_inverse):
+// y = X rhs, x = X^dagger y, two mat-vecs by 128 threads instead of four block steps with eight barriers.  The
+// factor's entries (at most seven 16-byte loads per thread) are loaded before the right-hand side is formed.
+// Forward, thread (row t / 4, quarter t % 4) takes four columns of each block; backward, thread (row t / 8,
+// column pair t % 8) one row of each block; the four warps' sums are added by the caller, x_i = sum_w part[32 w + i].
+template <int NPAD>
+struct InverseFactor {
+  static constexpr int NB = NPAD / LA_BLK;
+  float4 f[2 * NB], b[2 * NB - 1];
+  __device__ __forceinline__ void load(const float2* __restrict__ F) {
+    const int t = threadIdx.x, r = t >> 2, q = t & 3, rr = t >> 3, q8 = t & 7;
+    const bool row = r < NPAD;
+#pragma unroll
+    for (int J = 0; J < NB; ++J)
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        f[2 * J + u] = row && J <= (r >> 4)
+                           ? __ldg(reinterpret_cast<const float4*>(F + tri_index(r >> 4, J) * 256 + (r & 15) * LA_BLK + 4 * q + 2 * u))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 2 * NB - 1; ++u)   // blocks (0,0), (1,0), (1,1)
+      b[u] = __ldg(reinterpret_cast<const float4*>(F + u * 256 + rr * LA_BLK + 2 * q8));
+  }
+  __device__ __forceinline__ void solve(const float2* rhs, float2* y, float2* part) const {
+    const int t = threadIdx.x, r = t >> 2, q = t & 3, l = t & 31, rr = t >> 3, q8 = t & 7;
+    float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+#pragma unroll
+    for (int J = 0; J < NB; ++J)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float2* x = rhs + LA_BLK * J + 4 * q + 2 * u;
+        cfma(a0, make_float2(f[2 * J + u].x, f[2 * J + u].y), x[0]);
+        cfma(a1, make_float2(f[2 * J + u].z, f[2 * J + u].w), x[1]);
+      }
+    float2 a = make_float2(a0.x + a1.x, a0.y + a1.y);
+    a = reduce_xor(a, 1);
+    a = reduce_xor(a, 2);
+    if (q == 0 && r < NPAD) y[r] = a;
+    __syncthreads();
+    // columns 2 q8, 2 q8 + 1 of block column 0 (c0, c1) and 1 (c2, c3)
+    float2 c0 = make_float2(0.f, 0.f), c1 = c0, c2 = c0, c3 = c0;
+    const float2 y0 = y[rr];
+    cfma_conj(c0, make_float2(b[0].x, b[0].y), y0);
+    cfma_conj(c1, make_float2(b[0].z, b[0].w), y0);
+    if (NB > 1) {
+      const float2 y1 = y[LA_BLK + rr];
+      cfma_conj(c0, make_float2(b[2 * NB - 3 > 0 ? 1 : 0].x, b[2 * NB - 3 > 0 ? 1 : 0].y), y1);
+      cfma_conj(c1, make_float2(b[2 * NB - 3 > 0 ? 1 : 0].z, b[2 * NB - 3 > 0 ? 1 : 0].w), y1);
+      cfma_conj(c2, make_float2(b[2 * NB - 2].x, b[2 * NB - 2].y), y1);
+      cfma_conj(c3, make_float2(b[2 * NB - 2].z, b[2 * NB - 2].w), y1);
+    }
+    // over the warp's four rows (lane bits 3, 4): lane (bit 3, bit 4) ends with column 2 q8 + bit 3 of block bit 4
+    float2 s = fold(c0, c1, l & 8, 8);
+    if (NB > 1) s = fold(s, fold(c2, c3, l & 8, 8), l & 16, 16);
+    else s = reduce_xor(s, 16);
+    if (NB > 1 || !(l & 16)) part[(t & ~31) + ((l & 16) ? LA_BLK : 0) + 2 * q8 + ((l >> 3) & 1)] = s;
+    __syncthreads();
+  }
+  __device__ __forceinline__ static float2 result(const float2* part, int i) {
+    float2 s = part[i];
+#pragma unroll
+    for (int w = 1; w < 4; ++w) { s.x += part[32 * w + i].x; s.y += part[32 * w + i].y; }
+    return s;
+  }
+};
+// complex64 factors of at most 32 unknowns are stored as the inverse of L (k_factor_small).
+template <typename R, int NPAD>
+__host__ __device__ constexpr bool factor_is_inverse() {
+  return sizeof(R) == 4 && NPAD <= 32;
+}
+template <typename R, int NPAD, bool ON> struct MaybeInverse {};
+template <typename R, int NPAD> struct MaybeInverse<R, NPAD, true> : InverseFactor<NPAD> {};
+
 // The 128-thread solve (every step's blocks loaded together, the next step's in flight) serves every
 // complex64 factor and the wide FP64 ones; shorter FP64 factors keep the two-warp solve, whose
 // two-level reductions issue fewer adds on the slow FP64 pipe.
@@ -2098,65 +2171,71 @@ __device__ __forceinline__ void rec_k(const float2* p, float2 (&v)[K]) {
   }
 }
 
-// One complex64 subvolume of a colour with a superblock factor, as sweep_fine, with one thread per point: a
-// thread holds the point's K coefficients in registers, so residual, weight and H c need no pass over
-// shared memory between them and the index maps are paid once per point instead of once per coefficient.
-// One colour of 128^3, K = 4, 4x4x4 subvolumes (4096 of them): 236 us = 3.8 TB/s of in-band factor bytes read
-// once (the backward pass finds them in L2), against 319 us with 128 threads and 16-row steps; 96^3: 105
-// against 157 us.  Bound by the latency of a CTA's phases:
-// four CTAs per SM with one piece in flight (64 registers) beat three with two (108 us at 96^3) and two with three
-// (116 us); an L2 prefetch of the band at the start of the CTA costs 7 us.
-template <int NPAD, int K>
-__global__ void __launch_bounds__(kSuperThreads, K <= 4 ? 4 : 2)
-k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const float2* __restrict__ f,
-              const float2* __restrict__ yx, float2* __restrict__ c, const float2* __restrict__ factors, int colour,
-              FastDiv dn0, FastDiv dn1) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int NT = kSuperThreads, KK = K * K;
-  const int tid = threadIdx.x;
-  // blockIdx.x-th subvolume of the colour (dn0, dn1: the colour's subvolumes along x and y)
-  const int jr = fdiv(blockIdx.x, dn0), jz = fdiv(jr, dn1);
-  const int bb[3] = {2 * ((int)blockIdx.x - jr * dn0.d) + (colour & 1), 2 * (jr - jz * dn1.d) + ((colour >> 1) & 1),
-                     2 * jz + ((colour >> 2) & 1)};
-  const float2* F = factors + (size_t)((bb[2] * L.nb[1] + bb[1]) * L.nb[0] + bb[0]) * L.fsize;
-  int o[3], e[3];
+// Geometry of one subvolume of a colour for the point-per-thread right-hand side: origin and extent of U, of
+// U + 1 (footprint) and of U + 2 (c box), and the multiply-shift divisors of their index maps (the level's for
+// a full subvolume, its own for a ragged one).
+struct SweepBox {
+  int o[3], e[3], ec[3], ef[3], oc[3], of_[3];
+  FastDiv dc0, dc1, df0, df1, du0, du1;
+  // j-th subvolume of the colour; dn0, dn1 divide by the colour's subvolumes along x and y.  Returns its index.
+  __device__ __forceinline__ int init(const LevelGeom& L, int colour, int j, const FastDiv& dn0, const FastDiv& dn1) {
+    const int jr = fdiv(j, dn0), jz = fdiv(jr, dn1);
+    const int bb[3] = {2 * (j - jr * dn0.d) + (colour & 1), 2 * (jr - jz * dn1.d) + ((colour >> 1) & 1),
+                       2 * jz + ((colour >> 2) & 1)};
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    o[a] = bb[a] * L.sub[a];
-    e[a] = min(L.sub[a], L.n[a] - o[a]);
+    for (int a = 0; a < 3; ++a) {
+      const bool used = a < L.dim;
+      o[a] = bb[a] * L.sub[a];
+      e[a] = min(L.sub[a], L.n[a] - o[a]);
+      ec[a] = used ? e[a] + 4 : 1;  oc[a] = used ? o[a] - 2 : o[a];
+      ef[a] = used ? e[a] + 2 : 1;  of_[a] = used ? o[a] - 1 : o[a];
+    }
+    const bool full = e[0] == L.sub[0] && e[1] == L.sub[1] && e[2] == L.sub[2];
+    dc0 = full ? L.fd_c[0] : make_fastdiv(ec[0]);  dc1 = full ? L.fd_c[1] : make_fastdiv(ec[1]);
+    df0 = full ? L.fd_f[0] : make_fastdiv(ef[0]);  df1 = full ? L.fd_f[1] : make_fastdiv(ef[1]);
+    du0 = full ? L.fd_u[0] : make_fastdiv(e[0]);   du1 = full ? L.fd_u[1] : make_fastdiv(e[1]);
+    return (bb[2] * L.nb[1] + bb[1]) * L.nb[0] + bb[0];
   }
-  int ec[3], ef[3], oc[3], of_[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const bool used = a < L.dim;
-    ec[a] = used ? e[a] + 4 : 1;  oc[a] = used ? o[a] - 2 : o[a];
-    ef[a] = used ? e[a] + 2 : 1;  of_[a] = used ? o[a] - 1 : o[a];
-  }
-  const int nbc = ec[0] * ec[1] * ec[2], nbf = ef[0] * ef[1] * ef[2], npts = e[0] * e[1] * e[2];
-  const SuperSmem S = super_smem(L, K);
-  const bool full = e[0] == L.sub[0] && e[1] == L.sub[1] && e[2] == L.sub[2];
-  const FastDiv dc0 = full ? L.fd_c[0] : make_fastdiv(ec[0]), dc1 = full ? L.fd_c[1] : make_fastdiv(ec[1]);
-  const FastDiv df0 = full ? L.fd_f[0] : make_fastdiv(ef[0]), df1 = full ? L.fd_f[1] : make_fastdiv(ef[1]);
-  const FastDiv du0 = full ? L.fd_u[0] : make_fastdiv(e[0]), du1 = full ? L.fd_u[1] : make_fastdiv(e[1]);
-  auto coords = [](int i, const FastDiv& d0, const FastDiv& d1, int& x, int& y, int& z) {
+  __device__ __forceinline__ static void coords(int i, const FastDiv& d0, const FastDiv& d1, int& x, int& y, int& z) {
     const int r = fdiv(i, d0);
     x = i - r * d0.d;
     z = fdiv(r, d1);
     y = r - z * d1.d;
+  }
+};
+// The time matrices in complex64 as the right-hand side reads them: Q, U, E, W, Q^T, K x K floats each.
+template <int K>
+__device__ __forceinline__ void load_time_f32(const TimeMats* __restrict__ tm, float* sM) {
+  constexpr int KK = K * K;
+  for (int i = threadIdx.x; i < KK; i += blockDim.x) {
+    const float q = (float)tm->Qb[i];
+    sM[i] = q;
+    sM[KK + i] = (float)tm->Ub[i];
+    sM[2 * KK + i] = (float)tm->Eb[i];
+    sM[3 * KK + i] = (float)tm->Wt[i];
+    sM[4 * KK + (i % K) * K + i / K] = q;
+  }
+}
+// complex64 right-hand side (M~^dagger Wt (f - M~ c))_U (+ yx) of one subvolume, by a CTA of NT threads or, WARP, by
+// one warp: a thread holds a point's K coefficients in registers, so residual, weight and H c need no pass over
+// shared memory between them and the index maps are paid once per point instead of once per coefficient.
+// sC: c on U + 2, sZ: Wt r on U + 1, sV: dsum + V0 on U + 1; sRhs [npad] with zeros in the padding.
+// Synchronised on return.  sM may still be on its way when the call begins (the first barrier covers it).
+template <int K, bool WARP>
+__device__ __forceinline__ void sweep_rhs(const LevelGeom& L, const FineOp& g, const SweepBox& B, int tid, int NT,
+                                          int npad, const float* sM, float* sV, float2* sC, float2* sZ, float2* sRhs,
+                                          const float2* __restrict__ f, const float2* __restrict__ yx,
+                                          const float2* __restrict__ c) {
+  constexpr int KK = K * K;
+  auto sync = [] {
+    if (WARP) __syncwarp();
+    else __syncthreads();
   };
-  float* sM = reinterpret_cast<float*>(smem);                   // Q, U, E, W, Q^T [K][K] each
-  float* sV = reinterpret_cast<float*>(smem + S.v);             // dsum + V0 on the footprint
-  float2* sC = reinterpret_cast<float2*>(smem + S.c);           // c on U + 2
-  float2* sZ = reinterpret_cast<float2*>(smem + S.z);           // z = Wt r on the footprint
-  float2* sRhs = reinterpret_cast<float2*>(smem + S.rhs);       // right-hand side
-  float2* sXs = sRhs + NPAD;                                    // solution
-  float2* sY = sXs + NPAD;                                      // scratch of the solves
-  float2* sPr = sY + 2 * NPAD;
-
+  const int nbc = B.ec[0] * B.ec[1] * B.ec[2], nbf = B.ef[0] * B.ef[1] * B.ef[2], npts = B.e[0] * B.e[1] * B.e[2];
   for (int t = tid; t < nbc; t += NT) {
     int lx, ly, lz;
-    coords(t, dc0, dc1, lx, ly, lz);
-    const int gx = oc[0] + lx, gy = oc[1] + ly, gz = oc[2] + lz;
+    SweepBox::coords(t, B.dc0, B.dc1, lx, ly, lz);
+    const int gx = B.oc[0] + lx, gy = B.oc[1] + ly, gz = B.oc[2] + lz;
     const bool in = fine_in(g, gx, gy, gz);
     const float2* src = in ? c + (size_t)((gz * g.n[1] + gy) * g.n[0] + gx) * K : c;
     if constexpr (K % 2 == 0) {
@@ -2167,26 +2246,54 @@ k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const floa
       for (int m = 0; m < K; ++m) cp_async_elem_zf(sC + t * K + m, src + m, in);
     }
   }
-  for (int i = tid; i < KK; i += NT) {
-    const float q = (float)tm->Qb[i];
-    sM[i] = q;
-    sM[KK + i] = (float)tm->Ub[i];
-    sM[2 * KK + i] = (float)tm->Eb[i];
-    sM[3 * KK + i] = (float)tm->Wt[i];
-    sM[4 * KK + (i % K) * K + i / K] = q;
-  }
   const float dsum = (float)g.dsum;
   const float xo = (float)(g.lax == 0 ? g.x0[0] : (g.lax == 1 ? g.x0[1] : g.x0[2]));
   const float xh = (float)(g.lax == 0 ? g.h[0] : (g.lax == 1 ? g.h[1] : g.h[2]));
   const float wx = -0.5f * (float)g.ih2[0], wy = -0.5f * (float)g.ih2[1], wz = -0.5f * (float)g.ih2[2];
-  const int dcy = L.dim > 1 ? ec[0] : 0, dcz = L.dim > 2 ? ec[0] * ec[1] : 0;
   auto laser_x = [&](int gx, int gy, int gz) { return xo + (float)(g.lax == 0 ? gx : (g.lax == 1 ? gy : gz)) * xh; };
+  // h = H v at a point of a staged field (records of K, strides dy, dz points)
+  auto apply = [&](const float2* own, float dg, int dy, int dz, float2 (&v)[K], float2 (&h)[K]) {
+    float2 a1[K], a2[K];
+    rec_k<K>(own, v);
+    rec_k<K>(own + K, a1);
+    rec_k<K>(own - K, a2);
+#pragma unroll
+    for (int m = 0; m < K; ++m)
+      h[m] = make_float2(dg * v[m].x + wx * (a1[m].x + a2[m].x), dg * v[m].y + wx * (a1[m].y + a2[m].y));
+    if (L.dim > 1) {
+      rec_k<K>(own + dy * K, a1);
+      rec_k<K>(own - dy * K, a2);
+#pragma unroll
+      for (int m = 0; m < K; ++m) { h[m].x += wy * (a1[m].x + a2[m].x); h[m].y += wy * (a1[m].y + a2[m].y); }
+    }
+    if (L.dim > 2) {
+      rec_k<K>(own + dz * K, a1);
+      rec_k<K>(own - dz * K, a2);
+#pragma unroll
+      for (int m = 0; m < K; ++m) { h[m].x += wz * (a1[m].x + a2[m].x); h[m].y += wz * (a1[m].y + a2[m].y); }
+    }
+  };
+  // q.v, u.h and e.v of one row of the matrices at offsets 0 (Q or Q^T), U, E
+  auto row_products = [&](const float* sQ, int m, const float2 (&v)[K], const float2 (&h)[K], float2& qv, float2& uh,
+                          float2& ev) {
+    float q[K], u[K], ee[K];
+    row_k<K>(sQ + m * K, q);
+    row_k<K>(sM + KK + m * K, u);
+    row_k<K>(sM + 2 * KK + m * K, ee);
+    qv = uh = ev = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int n = 0; n < K; ++n) {
+      qv.x = fmaf(q[n], v[n].x, qv.x); qv.y = fmaf(q[n], v[n].y, qv.y);
+      uh.x = fmaf(u[n], h[n].x, uh.x); uh.y = fmaf(u[n], h[n].y, uh.y);
+      ev.x = fmaf(ee[n], v[n].x, ev.x); ev.y = fmaf(ee[n], v[n].y, ev.y);
+    }
+  };
   // r = f - M~ c and z = Wt r on the footprint, zero outside the grid
   bool staged = false;
   for (int i = tid; i < nbf || !staged; i += NT) {
     int lx = 0, ly = 0, lz = 0;
-    coords(i < nbf ? i : 0, df0, df1, lx, ly, lz);
-    const int gx = of_[0] + lx, gy = of_[1] + ly, gz = of_[2] + lz;
+    SweepBox::coords(i < nbf ? i : 0, B.df0, B.df1, lx, ly, lz);
+    const int gx = B.of_[0] + lx, gy = B.of_[1] + ly, gz = B.of_[2] + lz;
     const bool in = i < nbf && fine_in(g, gx, gy, gz);
     const size_t p = (size_t)((gz * g.n[1] + gy) * g.n[0] + gx);
     float2 r[K];
@@ -2199,7 +2306,7 @@ k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const floa
     }
     if (!staged) {
       cp_async_wait_all();
-      __syncthreads();
+      sync();
       staged = true;
     }
     if (i >= nbf) break;
@@ -2208,42 +2315,17 @@ k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const floa
 #pragma unroll
     for (int m = 0; m < K; ++m) z[m] = make_float2(0.f, 0.f);
     if (in) {
-      const float2* own = sC + (((L.dim > 2 ? lz + 1 : lz) * ec[1] + (L.dim > 1 ? ly + 1 : ly)) * ec[0] + lx + 1) * K;
-      float2 v[K], h[K], a1[K], a2[K];
-      rec_k<K>(own, v);
-      rec_k<K>(own + K, a1);
-      rec_k<K>(own - K, a2);
-#pragma unroll
-      for (int m = 0; m < K; ++m)
-        h[m] = make_float2(dg * v[m].x + wx * (a1[m].x + a2[m].x), dg * v[m].y + wx * (a1[m].y + a2[m].y));
-      if (L.dim > 1) {
-        rec_k<K>(own + dcy * K, a1);
-        rec_k<K>(own - dcy * K, a2);
-#pragma unroll
-        for (int m = 0; m < K; ++m) { h[m].x += wy * (a1[m].x + a2[m].x); h[m].y += wy * (a1[m].y + a2[m].y); }
-      }
-      if (L.dim > 2) {
-        rec_k<K>(own + dcz * K, a1);
-        rec_k<K>(own - dcz * K, a2);
-#pragma unroll
-        for (int m = 0; m < K; ++m) { h[m].x += wz * (a1[m].x + a2[m].x); h[m].y += wz * (a1[m].y + a2[m].y); }
-      }
+      const float2* own =
+          sC + (((L.dim > 2 ? lz + 1 : lz) * B.ec[1] + (L.dim > 1 ? ly + 1 : ly)) * B.ec[0] + lx + 1) * K;
+      float2 v[K], h[K];
+      apply(own, dg, B.ec[0], B.ec[0] * B.ec[1], v, h);
       const float xl = laser_x(gx, gy, gz);
 #pragma unroll
       for (int m = 0; m < K; ++m) {
-        float q[K], u[K], ee[K];
-        row_k<K>(sM + m * K, q);
-        row_k<K>(sM + KK + m * K, u);
-        row_k<K>(sM + 2 * KK + m * K, ee);
-        float qr = 0, qi = 0, ur = 0, ui = 0, er = 0, ei = 0;
-#pragma unroll
-        for (int n = 0; n < K; ++n) {
-          qr = fmaf(q[n], v[n].x, qr); qi = fmaf(q[n], v[n].y, qi);
-          ur = fmaf(u[n], h[n].x, ur); ui = fmaf(u[n], h[n].y, ui);
-          er = fmaf(ee[n], v[n].x, er); ei = fmaf(ee[n], v[n].y, ei);
-        }
-        r[m].x -= -qi - ur - xl * er;
-        r[m].y -= qr - ui - xl * ei;
+        float2 q, u, ev;
+        row_products(sM, m, v, h, q, u, ev);
+        r[m].x -= -q.y - u.x - xl * ev.x;
+        r[m].y -= q.x - u.y - xl * ev.y;
       }
 #pragma unroll
       for (int m = 0; m < K; ++m) {
@@ -2262,51 +2344,23 @@ k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const floa
       for (int m = 0; m < K; ++m) sZ[i * K + m] = z[m];
     }
   }
-  __syncthreads();
+  sync();
   // rhs = M~^dagger z = -i Qb^T z - Ub H z - x Eb z on U; padding 0
-  for (int t = npts * K + tid; t < NPAD; t += NT) sRhs[t] = make_float2(0.f, 0.f);
-  const int dfy = L.dim > 1 ? ef[0] : 0, dfz = L.dim > 2 ? ef[0] * ef[1] : 0;
+  for (int t = npts * K + tid; t < npad; t += NT) sRhs[t] = make_float2(0.f, 0.f);
   for (int i = tid; i < npts; i += NT) {
     int lx, ly, lz;
-    coords(i, du0, du1, lx, ly, lz);
-    const int fi = ((L.dim > 2 ? lz + 1 : lz) * ef[1] + (L.dim > 1 ? ly + 1 : ly)) * ef[0] + lx + 1;
-    const int gx = o[0] + lx, gy = o[1] + ly, gz = o[2] + lz;
-    const float2* own = sZ + fi * K;
-    const float dg = sV[fi], xl = laser_x(gx, gy, gz);
-    float2 v[K], h[K], a1[K], a2[K];
-    rec_k<K>(own, v);
-    rec_k<K>(own + K, a1);
-    rec_k<K>(own - K, a2);
-#pragma unroll
-    for (int m = 0; m < K; ++m)
-      h[m] = make_float2(dg * v[m].x + wx * (a1[m].x + a2[m].x), dg * v[m].y + wx * (a1[m].y + a2[m].y));
-    if (L.dim > 1) {
-      rec_k<K>(own + dfy * K, a1);
-      rec_k<K>(own - dfy * K, a2);
-#pragma unroll
-      for (int m = 0; m < K; ++m) { h[m].x += wy * (a1[m].x + a2[m].x); h[m].y += wy * (a1[m].y + a2[m].y); }
-    }
-    if (L.dim > 2) {
-      rec_k<K>(own + dfz * K, a1);
-      rec_k<K>(own - dfz * K, a2);
-#pragma unroll
-      for (int m = 0; m < K; ++m) { h[m].x += wz * (a1[m].x + a2[m].x); h[m].y += wz * (a1[m].y + a2[m].y); }
-    }
+    SweepBox::coords(i, B.du0, B.du1, lx, ly, lz);
+    const int fi = ((L.dim > 2 ? lz + 1 : lz) * B.ef[1] + (L.dim > 1 ? ly + 1 : ly)) * B.ef[0] + lx + 1;
+    const int gx = B.o[0] + lx, gy = B.o[1] + ly, gz = B.o[2] + lz;
+    const float xl = laser_x(gx, gy, gz);
+    float2 v[K], h[K];
+    apply(sZ + fi * K, sV[fi], B.ef[0], B.ef[0] * B.ef[1], v, h);
     const size_t p = (size_t)((gz * g.n[1] + gy) * g.n[0] + gx);
 #pragma unroll
     for (int m = 0; m < K; ++m) {
-      float q[K], u[K], ee[K];
-      row_k<K>(sM + 4 * KK + m * K, q);
-      row_k<K>(sM + KK + m * K, u);
-      row_k<K>(sM + 2 * KK + m * K, ee);
-      float qr = 0, qi = 0, ur = 0, ui = 0, er = 0, ei = 0;
-#pragma unroll
-      for (int n = 0; n < K; ++n) {
-        qr = fmaf(q[n], v[n].x, qr); qi = fmaf(q[n], v[n].y, qi);
-        ur = fmaf(u[n], h[n].x, ur); ui = fmaf(u[n], h[n].y, ui);
-        er = fmaf(ee[n], v[n].x, er); ei = fmaf(ee[n], v[n].y, ei);
-      }
-      float2 out = make_float2(qi - ur - xl * er, -qr - ui - xl * ei);
+      float2 q, u, ev;
+      row_products(sM + 4 * KK, m, v, h, q, u, ev);
+      float2 out = make_float2(q.y - u.x - xl * ev.x, -q.x - u.y - xl * ev.y);
       if (yx) {   // additive right-hand side (adjoint relaxation of G z = y)
         const float2 yv = yx[p * K + m];
         out.x += yv.x;
@@ -2315,17 +2369,151 @@ k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const floa
       sRhs[i * K + m] = out;
     }
   }
-  __syncthreads();
+  sync();
+}
+// c of unknown t of U plus delta, with c_U still in sC.
+template <int K>
+__device__ __forceinline__ void sweep_update(const LevelGeom& L, const FineOp& g, const SweepBox& B, int t, float2 d,
+                                             const float2* sC, float2* __restrict__ c) {
+  const int i = t / K, m = t - i * K;
+  int lx, ly, lz;
+  SweepBox::coords(i, B.du0, B.du1, lx, ly, lz);
+  const float2 v = sC[(((L.dim > 2 ? lz + 2 : lz) * B.ec[1] + (L.dim > 1 ? ly + 2 : ly)) * B.ec[0] + lx + 2) * K + m];
+  c[(size_t)(((B.o[2] + lz) * g.n[1] + (B.o[1] + ly)) * g.n[0] + (B.o[0] + lx)) * K + m] =
+      make_float2(v.x + d.x, v.y + d.y);
+}
+
+// One complex64 subvolume of a colour with a superblock factor per CTA.
+// One colour of 128^3, K = 4, 4x4x4 subvolumes (4096 of them): 236 us = 3.8 TB/s of in-band factor bytes read
+// once (the backward pass finds them in L2), against 319 us with 128 threads and 16-row steps; 96^3: 105
+// against 157 us.  Bound by the latency of a CTA's phases:
+// four CTAs per SM with one piece in flight (64 registers) beat three with two (108 us at 96^3) and two with three
+// (116 us); an L2 prefetch of the band at the start of the CTA costs 7 us.
+template <int NPAD, int K>
+__global__ void __launch_bounds__(kSuperThreads, K <= 4 ? 4 : 2)
+k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const float2* __restrict__ f,
+              const float2* __restrict__ yx, float2* __restrict__ c, const float2* __restrict__ factors, int colour,
+              FastDiv dn0, FastDiv dn1) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int tid = threadIdx.x;
+  SweepBox B;
+  const float2* F = factors + (size_t)B.init(L, colour, blockIdx.x, dn0, dn1) * L.fsize;
+  const SuperSmem S = super_smem(L, K);
+  float* sM = reinterpret_cast<float*>(smem);
+  float2* sC = reinterpret_cast<float2*>(smem + S.c);
+  float2* sRhs = reinterpret_cast<float2*>(smem + S.rhs);       // right-hand side
+  float2* sXs = sRhs + NPAD;                                    // solution
+  float2* sY = sXs + NPAD;                                      // scratch of the solves
+  float2* sPr = sY + 2 * NPAD;
+  load_time_f32<K>(tm, sM);
+  sweep_rhs<K, false>(L, g, B, tid, kSuperThreads, NPAD, sM, reinterpret_cast<float*>(smem + S.v), sC,
+                      reinterpret_cast<float2*>(smem + S.z), sRhs, f, yx, c);
   subvol_solve_super<NPAD>(F, L.band, sRhs, sY, sPr, sXs);
-  for (int t = tid; t < npts * K; t += NT) {   // c_U += delta, with c_U still in shared memory
-    const int i = t / K, m = t - i * K;
-    int lx, ly, lz;
-    coords(i, du0, du1, lx, ly, lz);
-    const float2 d = sXs[t];
-    const float2 v = sC[(((L.dim > 2 ? lz + 2 : lz) * ec[1] + (L.dim > 1 ? ly + 2 : ly)) * ec[0] + lx + 2) * K + m];
-    c[(size_t)(((o[2] + lz) * g.n[1] + (o[1] + ly)) * g.n[0] + (o[0] + lx)) * K + m] =
-        make_float2(v.x + d.x, v.y + d.y);
+  for (int t = tid; t < B.e[0] * B.e[1] * B.e[2] * K; t += kSuperThreads) sweep_update<K>(L, g, B, t, sXs[t], sC, c);
+}
+
+// ------------------------------------------------------------------------ finest sweep, small subvolumes
+// complex64 subvolumes of at most 32 unknowns, whose factor is stored as X = inv(L): one warp per subvolume,
+// four per CTA, so nothing waits on a CTA barrier and the time matrices are converted once for four.  The warp
+// loads X (at most twelve 16-byte loads per lane) before it forms the right-hand side and uses the same
+// registers for y = X rhs and x = X^dagger y: lane (row l / 4 of each group of eight, quarter l % 4 of each block's
+// columns), the sums folded across the lanes so that each ends with one unknown.
+// One colour of 256^2, K = 4, 4x2 subvolumes (2048 of them): 10.1 us; 128 threads per subvolume with the same
+// inverse took 19.4 us, a third of it conversions of the time matrices and barriers.
+constexpr int kSmallSweepWarps = 4;
+__host__ __device__ __forceinline__ SuperSmem small_smem(const LevelGeom& L, int K) {
+  const int nbc = (L.sub[0] + 4) * (L.dim > 1 ? L.sub[1] + 4 : 1) * (L.dim > 2 ? L.sub[2] + 4 : 1);
+  const int nbf = (L.sub[0] + 2) * (L.dim > 1 ? L.sub[1] + 2 : 1) * (L.dim > 2 ? L.sub[2] + 2 : 1);
+  SuperSmem s;   // per warp, after the time matrices; total: one warp's bytes
+  s.v = 0;
+  s.c = (nbf * 4 + 15) & ~15;
+  s.z = s.c + ((nbc * K * 8 + 15) & ~15);
+  s.rhs = s.z + ((nbf * K * 8 + 15) & ~15);
+  s.total = s.rhs + 2 * 32 * 8;   // rhs, y
+  return s;
+}
+template <int NPAD, int K>
+__global__ void __launch_bounds__(32 * kSmallSweepWarps)
+k_sweep_small(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const float2* __restrict__ f,
+              const float2* __restrict__ yx, float2* __restrict__ c, const float2* __restrict__ factors, int colour,
+              FastDiv dn0, FastDiv dn1, int count) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int NB = NPAD / LA_BLK, NG = NPAD / 8;   // blocks per side; groups of eight rows
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, row = l >> 2, q = l & 3;
+  const int j = blockIdx.x * kSmallSweepWarps + w;
+  float* sM = reinterpret_cast<float*>(smem);
+  load_time_f32<K>(tm, sM);
+  __syncthreads();
+  if (j >= count) return;
+  SweepBox B;
+  const float2* F = factors + (size_t)B.init(L, colour, j, dn0, dn1) * L.fsize;
+  // X[8 G + row][16 J + 4 q + ..] of the blocks J <= G / 2
+  float4 X[NG][NB][2];
+#pragma unroll
+  for (int G = 0; G < NG; ++G)
+#pragma unroll
+    for (int J = 0; J <= G / 2; ++J)
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        X[G][J][u] = __ldg(reinterpret_cast<const float4*>(F + tri_index(G / 2, J) * 256 +
+                                                           (8 * (G & 1) + row) * LA_BLK + 4 * q + 2 * u));
+  const SuperSmem S = small_smem(L, K);
+  unsigned char* base = smem + ((5 * K * K * 4 + 15) & ~15) + w * S.total;
+  float2* sC = reinterpret_cast<float2*>(base + S.c);
+  float2* sRhs = reinterpret_cast<float2*>(base + S.rhs);
+  float2* sY = sRhs + 32;
+  sweep_rhs<K, true>(L, g, B, l, 32, NPAD, sM, reinterpret_cast<float*>(base), sC, reinterpret_cast<float2*>(base + S.z),
+                     sRhs, f, yx, c);
+  const float2 zero = make_float2(0.f, 0.f);
+  {
+    float2 a[NG];
+#pragma unroll
+    for (int G = 0; G < NG; ++G) a[G] = zero;
+#pragma unroll
+    for (int J = 0; J < NB; ++J)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float4 v = *reinterpret_cast<const float4*>(sRhs + LA_BLK * J + 4 * q + 2 * u);
+#pragma unroll
+        for (int G = 2 * J; G < NG; ++G) {
+          cfma(a[G], make_float2(X[G][J][u].x, X[G][J][u].y), make_float2(v.x, v.y));
+          cfma(a[G], make_float2(X[G][J][u].z, X[G][J][u].w), make_float2(v.z, v.w));
+        }
+      }
+    // over the four quarters: lane q ends with group 2 (q & 1) + (q / 2) (NPAD 16: group q & 1)
+    float2 s = fold(a[0], a[NG / 2], l & 1, 1);
+    if constexpr (NG > 2) s = fold(s, fold(a[1], a[3], l & 1, 1), l & 2, 2);
+    else s = reduce_xor(s, 2);
+    const int G = NG > 2 ? 2 * (q & 1) + (q >> 1) : (q & 1);
+    if (NG > 2 || q < 2) sY[8 * G + row] = s;
   }
+  __syncwarp();
+  float2 x[NB][4];
+#pragma unroll
+  for (int J = 0; J < NB; ++J)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[J][u] = zero;
+#pragma unroll
+  for (int G = 0; G < NG; ++G) {
+    const float2 y = sY[8 * G + row];
+#pragma unroll
+    for (int J = 0; J <= G / 2; ++J)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        cfma_conj(x[J][2 * u], make_float2(X[G][J][u].x, X[G][J][u].y), y);
+        cfma_conj(x[J][2 * u + 1], make_float2(X[G][J][u].z, X[G][J][u].w), y);
+      }
+  }
+  // over the eight rows (lane bits 2, 3, 4): column 4 q + 2 bit 2 + bit 3 of block bit 4
+  float2 s[NB];
+#pragma unroll
+  for (int J = 0; J < NB; ++J)
+    s[J] = fold(fold(x[J][0], x[J][2], l & 4, 4), fold(x[J][1], x[J][3], l & 4, 4), l & 8, 8);
+  float2 d;
+  if constexpr (NB > 1) d = fold(s[0], s[1], l & 16, 16);
+  else d = reduce_xor(s[0], 16);
+  const int t = (NB > 1 ? (l >> 4) * LA_BLK : 0) + 4 * q + ((l & 4) ? 2 : 0) + ((l & 8) ? 1 : 0);
+  if ((NB > 1 || l < 16) && t < B.e[0] * B.e[1] * B.e[2] * K) sweep_update<K>(L, g, B, t, d, sC, c);
 }
 
 // ======================================================================== Galerkin-level sweep
@@ -2491,10 +2679,17 @@ k_sweep_coarse(LevelGeom L, const R* __restrict__ sigma, const TimeMats* __restr
   int o[3], e[3];
   subvol_box(L, b, o, e);
   const int npts = e[0] * e[1] * e[2];
+  constexpr bool kInv = factor_is_inverse<R, NPAD>();
+  MaybeInverse<R, NPAD, kInv> inv;
+  if constexpr (kInv) inv.load(factors + (size_t)b * L.fsize);
   CoarseSmem<R> S = coarse_smem_layout<R>(smem, L, K, NPAD);
   coarse_rhs<R>(L, sigma, tm, gvec, ev, o, e, NPAD, S);
-  subvol_solve<CT, NPAD>(factors + (size_t)b * L.fsize, S.Rhs, S.Y, S.T, S.Red);
-  __syncthreads();
+  if constexpr (kInv) {
+    inv.solve(S.Rhs, S.Y, S.Red);
+  } else {
+    subvol_solve<CT, NPAD>(factors + (size_t)b * L.fsize, S.Rhs, S.Y, S.T, S.Red);
+    __syncthreads();
+  }
   const SubvolDiv dv(L, e);
   for (int t = threadIdx.x; t < npts * K; t += kSweepThreads) {
     int i, m;
@@ -2502,9 +2697,11 @@ k_sweep_coarse(LevelGeom L, const R* __restrict__ sigma, const TimeMats* __restr
     int lx, ly, lz;
     SubvolDiv::coords(i, dv.u0, dv.u1, lx, ly, lz);
     const size_t gi = (size_t)(((o[2] + lz) * L.n[1] + (o[1] + ly)) * L.n[0] + (o[0] + lx)) * K + m;
-    CT v = ev[gi];
-    v.x += S.Rhs[t].x;
-    v.y += S.Rhs[t].y;
+    CT v = ev[gi], d;
+    if constexpr (kInv) d = inv.result(S.Red, t);
+    else d = S.Rhs[t];
+    v.x += d.x;
+    v.y += d.y;
     ev[gi] = v;
   }
 }
@@ -2677,12 +2874,39 @@ cudaError_t launch_sweep_super(const LevelGeom& L, const FineOp& g, const TimeMa
   kern<<<nblocks, kSuperThreads, smem, s>>>(L, g, tm, f, yx, c, factors, colour, dn0, dn1);
   return cudaGetLastError();
 }
+template <int NPAD, int K>
+cudaError_t launch_sweep_small(const LevelGeom& L, const FineOp& g, const TimeMats* tm, const float2* f,
+                               const float2* yx, float2* c, const float2* factors, int colour, int nblocks,
+                               cudaStream_t s) {
+  const size_t smem = ((5 * K * K * 4 + 15) & ~15) + (size_t)kSmallSweepWarps * small_smem(L, K).total;
+  auto kern = k_sweep_small<NPAD, K>;
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (err != cudaSuccess) return err;
+    attr_set = true;
+  }
+  if (smem > 227 * 1024) return cudaErrorInvalidValue;
+  const FastDiv dn0 = make_fastdiv((L.nb[0] - (colour & 1) + 1) / 2),
+                dn1 = make_fastdiv((L.nb[1] - ((colour >> 1) & 1) + 1) / 2);
+  kern<<<(nblocks + kSmallSweepWarps - 1) / kSmallSweepWarps, 32 * kSmallSweepWarps, smem, s>>>(
+      L, g, tm, f, yx, c, factors, colour, dn0, dn1, nblocks);
+  return cudaGetLastError();
+}
 template <typename R, int NPAD>
 cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeMats* tm, int K,
                                 const typename C2<R>::T* f, const typename C2<R>::T* yx, typename C2<R>::T* c,
                                 const typename C2<R>::T* factors, int colour, cudaStream_t s) {
   const int nblocks = colour_count(L, colour);
   if (nblocks == 0) return cudaSuccess;
+  if constexpr (factor_is_inverse<R, NPAD>()) {
+#define LA_SMALL(KK) case KK: return launch_sweep_small<NPAD, KK>(L, g, tm, f, yx, c, factors, colour, nblocks, s)
+    switch (K) {
+      LA_SMALL(1); LA_SMALL(2); LA_SMALL(3); LA_SMALL(4); LA_SMALL(5); LA_SMALL(6); LA_SMALL(7); LA_SMALL(8);
+      default: return cudaErrorInvalidValue;
+    }
+#undef LA_SMALL
+  } else {
   if constexpr (sizeof(R) == 4 && NPAD > LA_NPAD_MAX) {
     if (factor_is_super<R>(L)) {
 #define LA_SUPER(KK) case KK: return launch_sweep_super<NPAD, KK>(L, g, tm, f, yx, c, factors, colour, nblocks, s)
@@ -2704,6 +2928,7 @@ cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeM
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   kern<<<nblocks, kSweepThreads, smem, s>>>(L, g, tm, f, yx, c, factors, colour);
   return cudaGetLastError();
+  }
 }
 template <typename R, int NPAD>
 cudaError_t launch_sweep_coarse_n(const LevelGeom& L, const R* sigma, const TimeMats* tm, int K,

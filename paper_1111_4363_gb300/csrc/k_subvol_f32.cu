@@ -4,6 +4,7 @@ namespace la {
 template <>
 cudaError_t launch_factor<float>(const LevelGeom& L, const FineOp* fine, const float* sigma, const TimeMats* tm,
                                   float2* factors, int* status, cudaStream_t s) {
+  if (L.npad <= 32) return launch_factor_small(L, fine, sigma, tm, factors, status, s);
 #define LA_CALL(N) launch_factor_blk_n<float, N>(L, fine, sigma, tm, factors, status, s)
   {
 #define LA_WCALL(N)                                                                             \
@@ -13,7 +14,13 @@ cudaError_t launch_factor<float>(const LevelGeom& L, const FineOp* fine, const f
     LA_NPAD_DISPATCH_WIDE(L.npad, LA_WCALL)
 #undef LA_WCALL
   }
-  LA_NPAD_DISPATCH(L.npad, LA_CALL)
+  switch (L.npad) {
+    case 48: return LA_CALL(48);
+    case 64: return LA_CALL(64);
+    case 96: return LA_CALL(96);
+    case 128: return LA_CALL(128);
+    default: return cudaErrorInvalidValue;
+  }
 #undef LA_CALL
 }
 template <>

@@ -427,6 +427,9 @@ void launch_galerkin(const FineOp& g, const LevelGeom* geo, int levels, double* 
 template <typename R>
 cudaError_t launch_factor(const LevelGeom& L, const FineOp* fine, const R* sigma, const TimeMats* tm,
                           typename C2<R>::T* factors, int* status, cudaStream_t s);
+// complex64 subvolumes of at most 32 unknowns: the inverse of the Cholesky factor
+cudaError_t launch_factor_small(const LevelGeom& L, const FineOp* fine, const float* sigma, const TimeMats* tm,
+                                float2* factors, int* status, cudaStream_t s);
 template <typename R>
 cudaError_t launch_sweep_fine(const LevelGeom& L, const FineOp& g, const TimeMats* tm, int K,
                               const typename C2<R>::T* f, const typename C2<R>::T* yx, typename C2<R>::T* c,
