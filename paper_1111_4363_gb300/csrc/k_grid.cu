@@ -296,6 +296,7 @@ __global__ void __launch_bounds__(256) k_residual(FineOp g, const TimeMats* __re
                                                   const double2* __restrict__ f, const double2* __restrict__ c,
                                                   double2* __restrict__ zout, ResidOut out) {
   typedef TimeProducts<K> TP;
+  overlap_trigger();
   __shared__ double Eb[K * K];
   __shared__ double red[256];
   for (int i = threadIdx.x; i < K * K; i += blockDim.x) Eb[i] = tm->Eb[i];
@@ -506,6 +507,7 @@ __global__ void __launch_bounds__(kTX * kTY, K <= 4 ? 4 : 2) k_stencil_tma(FineO
                                                                const float2* __restrict__ f, float2* __restrict__ out,
                                                                const float2* __restrict__ yadd, int* status, int zc) {
   extern __shared__ __align__(128) unsigned char smem[];
+  overlap_trigger();
   constexpr unsigned kPlaneBytes = kPS * K * 8;
   constexpr int kStage = stage_f2(K);
   float2* stage = reinterpret_cast<float2*>(smem);                                  // [kNST][kPS][K] (padded)
@@ -870,6 +872,8 @@ __global__ void __launch_bounds__(256) k_restrict_tile(LevelGeom F, LevelGeom C,
                                                        CT* __restrict__ gc, CT* __restrict__ ec) {
   typedef typename CR<CT>::R RR;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  overlap_trigger();
+  overlap_wait();
   CT* box = reinterpret_cast<CT*>(smem_raw);
   const bool uy = F.dim > 1, uz = F.dim > 2;
   const int tx = kRx, ty = uy ? kRy : 1, tz = uz ? kRz : 1;
@@ -920,6 +924,8 @@ __global__ void __launch_bounds__(256) k_restrict_tile(LevelGeom F, LevelGeom C,
 template <typename CT, int K>
 __global__ void k_prolong_add(LevelGeom F, LevelGeom C, const CT* __restrict__ ec, CT* __restrict__ ef) {
   typedef typename CR<CT>::R RR;
+  overlap_trigger();
+  overlap_wait();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= F.np) return;
   int x, y, z;
@@ -960,7 +966,7 @@ void launch_restrict(const LevelGeom& F, const LevelGeom& C, int K, const typena
       cudaFuncSetAttribute(k_restrict_tile<CT, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); \
       attr = true;                                                                                         \
     }                                                                                                      \
-    k_restrict_tile<CT, KK><<<grid, 256, smem, s>>>(F, C, sf, gc, ec);                                     \
+    launch_overlapped(F.overlap, k_restrict_tile<CT, KK>, grid, 256, smem, s, F, C, sf, gc, ec);           \
   } while (0)
     switch (K) {
       case 1: LA_CALL(1); break;
@@ -982,7 +988,8 @@ void launch_restrict(const LevelGeom& F, const LevelGeom& C, int K, const typena
 template <typename R>
 void launch_prolong_add(const LevelGeom& F, const LevelGeom& C, int K, const typename C2<R>::T* ec,
                         typename C2<R>::T* ef, cudaStream_t s) {
-#define LA_CALL(KK) k_prolong_add<typename C2<R>::T, KK><<<(F.np + 127) / 128, 128, 0, s>>>(F, C, ec, ef)
+#define LA_CALL(KK) \
+  launch_overlapped(F.overlap, k_prolong_add<typename C2<R>::T, KK>, (F.np + 127) / 128, 128, 0, s, F, C, ec, ef)
   LA_K_DISPATCH(K, LA_CALL)
 #undef LA_CALL
 }

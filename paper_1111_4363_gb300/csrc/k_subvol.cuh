@@ -1901,6 +1901,7 @@ k_sweep_fine(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const typen
              const typename C2<R>::T* __restrict__ factors, int colour) {
   typedef typename C2<R>::T CT;
   extern __shared__ __align__(16) unsigned char smem[];
+  overlap_trigger();
   const int K = tm->K, KK = K * K;
   const int tid = threadIdx.x;
   const int b = colour_subvol(L, colour, blockIdx.x);
@@ -1951,6 +1952,7 @@ k_sweep_fine(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const typen
   for (int i = tid; i < KK; i += kSweepThreads) {
     sQ[i] = (R)tm->Qb[i]; sU[i] = (R)tm->Ub[i]; sW[i] = (R)tm->Wt[i]; sE[i] = (R)tm->Eb[i];
   }
+  overlap_wait();
   const unsigned long long stream = l2_evict_first();   // c and f: read once per launch
   for (int t = tid; t < nbc * K; t += kSweepThreads) {
     int i, m;
@@ -2232,6 +2234,7 @@ __device__ __forceinline__ void sweep_rhs(const LevelGeom& L, const FineOp& g, c
     else __syncthreads();
   };
   const int nbc = B.ec[0] * B.ec[1] * B.ec[2], nbf = B.ef[0] * B.ef[1] * B.ef[2], npts = B.e[0] * B.e[1] * B.e[2];
+  overlap_wait();   // c and f are read from here on
   for (int t = tid; t < nbc; t += NT) {
     int lx, ly, lz;
     SweepBox::coords(t, B.dc0, B.dc1, lx, ly, lz);
@@ -2395,6 +2398,7 @@ k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const floa
               const float2* __restrict__ yx, float2* __restrict__ c, const float2* __restrict__ factors, int colour,
               FastDiv dn0, FastDiv dn1) {
   extern __shared__ __align__(16) unsigned char smem[];
+  overlap_trigger();
   const int tid = threadIdx.x;
   SweepBox B;
   const float2* F = factors + (size_t)B.init(L, colour, blockIdx.x, dn0, dn1) * L.fsize;
@@ -2441,6 +2445,7 @@ k_sweep_small(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const floa
   constexpr int NB = NPAD / LA_BLK, NG = NPAD / 8;   // blocks per side; groups of eight rows
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, row = l >> 2, q = l & 3;
   const int j = blockIdx.x * kSmallSweepWarps + w;
+  overlap_trigger();
   float* sM = reinterpret_cast<float*>(smem);
   load_time_f32<K>(tm, sM);
   __syncthreads();
@@ -2593,8 +2598,17 @@ __device__ inline void coarse_rhs(const LevelGeom& L, const R* __restrict__ sigm
   const int nbox = box5_count(L.dim);
   const SubvolDiv dv(L, e);
   for (int i = tid; i < LA_NPAIR * KK; i += nthr) S.P[i] = (R)tm->P[i / KK][i % KK];
-  // e on U + 2 (zero outside the grid) and the stencils of U's points reach shared memory by cp.async,
-  // every copy of a thread in flight at once instead of one dependent load per loop trip
+  // the stencils of U's points and e on U + 2 (zero outside the grid) reach shared memory by cp.async, every copy
+  // of a thread in flight at once instead of one dependent load per loop trip; e once its writers have finished
+  const int per_pt = LA_NPAIR * nbox;
+  for (int t = tid; t < npts * per_pt; t += nthr) {
+    const int i = fdiv(t, L.fd_pair), w = t - i * per_pt;
+    int lx, ly, lz;
+    SubvolDiv::coords(i, dv.u0, dv.u1, lx, ly, lz);
+    const int p = ((o[2] + lz) * L.n[1] + (o[1] + ly)) * L.n[0] + (o[0] + lx);
+    cp_async_real(S.Sg + t, sigma + (size_t)p * per_pt + w);
+  }
+  overlap_wait();
   for (int t = tid; t < nbc * K; t += nthr) {
     int i, m;
     dv.item(t, i, m);
@@ -2603,14 +2617,6 @@ __device__ inline void coarse_rhs(const LevelGeom& L, const R* __restrict__ sigm
     const int gx = oc[0] + lx, gy = oc[1] + ly, gz = oc[2] + lz;
     const bool in = gx >= 0 && gy >= 0 && gz >= 0 && gx < L.n[0] && gy < L.n[1] && gz < L.n[2];
     cp_async_elem_zf(S.E + t, in ? ev + (size_t)((gz * L.n[1] + gy) * L.n[0] + gx) * K + m : ev, in);
-  }
-  const int per_pt = LA_NPAIR * nbox;
-  for (int t = tid; t < npts * per_pt; t += nthr) {
-    const int i = fdiv(t, L.fd_pair), w = t - i * per_pt;
-    int lx, ly, lz;
-    SubvolDiv::coords(i, dv.u0, dv.u1, lx, ly, lz);
-    const int p = ((o[2] + lz) * L.n[1] + (o[1] + ly)) * L.n[0] + (o[0] + lx);
-    cp_async_real(S.Sg + t, sigma + (size_t)p * per_pt + w);
   }
   cp_async_wait_all();
   __syncthreads();
@@ -2674,6 +2680,7 @@ k_sweep_coarse(LevelGeom L, const R* __restrict__ sigma, const TimeMats* __restr
                const typename C2<R>::T* __restrict__ factors, int colour, int* __restrict__ status) {
   typedef typename C2<R>::T CT;
   extern __shared__ __align__(16) unsigned char smem[];
+  overlap_trigger();
   const int K = tm->K;
   const int b = colour_subvol(L, colour, blockIdx.x);
   int o[3], e[3];
@@ -2714,6 +2721,7 @@ k_gresid_tiles(LevelGeom L, const R* __restrict__ sigma, const TimeMats* __restr
                typename C2<R>::T* __restrict__ out, int npad) {
   typedef typename C2<R>::T CT;
   extern __shared__ __align__(16) unsigned char smem[];
+  overlap_trigger();
   const int K = tm->K;
   int o[3], e[3];
   subvol_box(L, blockIdx.x, o, e);
@@ -2871,8 +2879,7 @@ cudaError_t launch_sweep_super(const LevelGeom& L, const FineOp& g, const TimeMa
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   const FastDiv dn0 = make_fastdiv((L.nb[0] - (colour & 1) + 1) / 2),
                 dn1 = make_fastdiv((L.nb[1] - ((colour >> 1) & 1) + 1) / 2);
-  kern<<<nblocks, kSuperThreads, smem, s>>>(L, g, tm, f, yx, c, factors, colour, dn0, dn1);
-  return cudaGetLastError();
+  return launch_overlapped(L.overlap, kern, nblocks, kSuperThreads, smem, s, L, g, tm, f, yx, c, factors, colour, dn0, dn1);
 }
 template <int NPAD, int K>
 cudaError_t launch_sweep_small(const LevelGeom& L, const FineOp& g, const TimeMats* tm, const float2* f,
@@ -2889,9 +2896,8 @@ cudaError_t launch_sweep_small(const LevelGeom& L, const FineOp& g, const TimeMa
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   const FastDiv dn0 = make_fastdiv((L.nb[0] - (colour & 1) + 1) / 2),
                 dn1 = make_fastdiv((L.nb[1] - ((colour >> 1) & 1) + 1) / 2);
-  kern<<<(nblocks + kSmallSweepWarps - 1) / kSmallSweepWarps, 32 * kSmallSweepWarps, smem, s>>>(
-      L, g, tm, f, yx, c, factors, colour, dn0, dn1, nblocks);
-  return cudaGetLastError();
+  return launch_overlapped(L.overlap, kern, (nblocks + kSmallSweepWarps - 1) / kSmallSweepWarps, 32 * kSmallSweepWarps,
+                           smem, s, L, g, tm, f, yx, c, factors, colour, dn0, dn1, nblocks);
 }
 template <typename R, int NPAD>
 cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeMats* tm, int K,
@@ -2926,8 +2932,7 @@ cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeM
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  kern<<<nblocks, kSweepThreads, smem, s>>>(L, g, tm, f, yx, c, factors, colour);
-  return cudaGetLastError();
+  return launch_overlapped(L.overlap, kern, nblocks, kSweepThreads, smem, s, L, g, tm, f, yx, c, factors, colour);
   }
 }
 template <typename R, int NPAD>
@@ -2945,8 +2950,7 @@ cudaError_t launch_sweep_coarse_n(const LevelGeom& L, const R* sigma, const Time
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  kern<<<nblocks, kSweepThreads, smem, s>>>(L, sigma, tm, gvec, e, factors, colour, status);
-  return cudaGetLastError();
+  return launch_overlapped(L.overlap, kern, nblocks, kSweepThreads, smem, s, L, sigma, tm, gvec, e, factors, colour, status);
 }
 
 template <typename R>
@@ -2962,8 +2966,7 @@ cudaError_t launch_gresid_tiles_r(const LevelGeom& L, const R* sigma, const Time
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  kern<<<L.nsub, kSweepThreads, smem, s>>>(L, sigma, tm, gvec, e, out, L.npad);
-  return cudaGetLastError();
+  return launch_overlapped(L.overlap, kern, L.nsub, kSweepThreads, smem, s, L, sigma, tm, gvec, e, out, L.npad);
 }
 
 // finest-level sweeps and factorisations also take the wide sizes

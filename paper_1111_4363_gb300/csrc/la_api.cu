@@ -359,6 +359,7 @@ extern "C" la_status la_init(const la_config* cfg, void* stream, la_ctx** out) {
     }
     G.fd_pair = make_fastdiv(LA_NPAIR * box5_count(k.dim));
     G.one_per_cta = k.factor_group == 1 ? 1 : 0;
+    G.overlap = 1;
     G.band = (l == 0 && k.local_form == 0 && G.npad > LA_NPAD_MAX) ? fine_band_blocks(k.dim, G.sub, k.nt, G.nblk)
                                                                   : G.nblk - 1;
     // square form: M couples edge neighbours; finest least squares: H^2, two grid steps; Galerkin levels: box
@@ -1265,7 +1266,9 @@ static la_status build_loop_graph(la_ctx* c) {
       c->stream = c->cap;
       c->capturing = true;
       c->device_norm = true;
+      for (int l = 0; l < c->L; ++l) c->geo[l].overlap = 0;   // a conditional body takes plain kernel nodes
       st = cycle_body(c);
+      for (int l = 0; l < c->L; ++l) c->geo[l].overlap = 1;
       if (st == LA_OK) launch_loop_cond(c->d_lstate, c->d_N, k.tol, k.max_cycles, check, 0, h, c->cap);
       cudaError_t ee = cudaStreamEndCapture(c->cap, &out);
       c->stream = user;
