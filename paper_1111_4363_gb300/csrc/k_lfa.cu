@@ -324,16 +324,18 @@ bool build_case(const la_lfa_case& cs, CaseMats& out, std::string& why) {
 
 // ------------------------------------------------------------------ kernels
 // overlaps a[k][e][i] = int exp(i k x_e(y)) P_i(y) dy (x_0 = y for one element; x_e = (y - 1)/2 + e
-// for two) and b[w][n] = int exp(i w y) P_n(y) dy, by a Gauss-Legendre rule
-__global__ void k_lfa_overlaps(const double* __restrict__ k, int nk, const double* __restrict__ w, int nw,
+// for two) and b[w][n] = int exp(i w y) P_n(y) dy, by a Gauss-Legendre rule.  One warp per CTA and element: the
+// FP64 sine and cosine of every node keep an SM's two FP64 lanes busy, so the warps go to as many SMs as
+// there are (128 + 128 points, two elements: 250 us with four warps per CTA and both elements in one thread).
+__global__ void __launch_bounds__(32) k_lfa_overlaps(const double* __restrict__ k, int nk, const double* __restrict__ w, int nw,
                                const double* __restrict__ qy, const double* __restrict__ qw, int nel, int nx, int nt,
                                double2* __restrict__ a, double2* __restrict__ b) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nk + nw) return;
   const bool space = t < nk;
   const double kk = space ? k[t] : w[t - nk];
-  const int nf = space ? nx : nt, ne = space ? nel : 1;
-  for (int e = 0; e < ne; ++e) {
+  const int nf = space ? nx : nt, e = blockIdx.y;
+  if (e < (space ? nel : 1)) {
     double2 acc[8];
     for (int i = 0; i < 8; ++i) acc[i] = make_double2(0.0, 0.0);
     for (int q = 0; q < kLfaQuad; ++q) {
@@ -530,11 +532,9 @@ extern "C" la_status la_lfa_maps(const la_lfa_case* cases, int ncases, const dou
     const double2* G = reinterpret_cast<const double2*>(B + off_g) + goff[c];
     const double* Wt = reinterpret_cast<const double*>(B + off_wt) + woff[c];
     if (F.nel != tab_nel || F.nx != tab_nx || F.nt != tab_nt) {
-      k_lfa_overlaps<<<(nk + nw + 127) / 128, 128, 0, s>>>(reinterpret_cast<double*>(B + off_k), nk,
-                                                           reinterpret_cast<double*>(B + off_w), nw,
-                                                           reinterpret_cast<double*>(B + off_qy),
-                                                           reinterpret_cast<double*>(B + off_qw), F.nel, F.nx, F.nt,
-                                                           a, b);
+      k_lfa_overlaps<<<dim3((nk + nw + 31) / 32, F.nel), 32, 0, s>>>(
+          reinterpret_cast<double*>(B + off_k), nk, reinterpret_cast<double*>(B + off_w), nw,
+          reinterpret_cast<double*>(B + off_qy), reinterpret_cast<double*>(B + off_qw), F.nel, F.nx, F.nt, a, b);
       tab_nel = F.nel;
       tab_nx = F.nx;
       tab_nt = F.nt;

@@ -1436,22 +1436,28 @@ __device__ __forceinline__ CT reduce4(CT v) {
 }
 
 template <typename CT, int NPAD>
-__device__ __forceinline__ void subvol_solve(const CT* __restrict__ F, CT* rhs, CT* y, CT* tvec, CT* red) {
+__device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __restrict__ F, CT* rhs, CT* y, CT* tvec) {
   constexpr int NB = NPAD / LA_BLK;
-  (void)red;
   const int tid = threadIdx.x;
   if (tid >= 64) return;
-  const int r = tid >> 2, l = tid & 3;
+  const int r = tid >> 2, l = tid & 3, r0 = r & 8;   // r0: the warp's first row of a block
+  // A factor has no entry further than L.reach points from its diagonal: a warp's eight rows start at the first
+  // column its first row couples to and (backward) its eight columns end at the last row its last column
+  // couples to, in steps of the four columns that the lanes of a row take together.  Predicated lanes would
+  // still occupy the FP64 pipe, so the bounds are the warp's.
+  const int K = L.fd_K.d;
   // forward: y_I = inv(L_II) (rhs_I - sum_{J<I} L_IJ y_J)
   for (int I = 0; I < NB; ++I) {
     const CT* rowblk = F + (size_t)(I * (I + 1) / 2) * 256;
+    const int c0 = max((fdiv(I * LA_BLK + r0, L.fd_K) - L.reach) * K, 0) >> 2;   // first group of four columns
     CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
-    for (int J = 0; J < I; ++J) {
+    for (int J = c0 >> 2; J < I; ++J) {
       const CT* blk = rowblk + J * 256 + r * LA_BLK;
       const CT* yy = y + J * LA_BLK;
-      cfma(acc0, blk[l], yy[l]);
-      cfma(acc1, blk[l + 4], yy[l + 4]);
-      cfma(acc0, blk[l + 8], yy[l + 8]);
+      const int k0 = c0 - 4 * J;
+      if (k0 <= 0) cfma(acc0, blk[l], yy[l]);
+      if (k0 <= 1) cfma(acc1, blk[l + 4], yy[l + 4]);
+      if (k0 <= 2) cfma(acc0, blk[l + 8], yy[l + 8]);
       cfma(acc1, blk[l + 12], yy[l + 12]);
     }
     CT acc = reduce4(mkc<CT>(acc0.x + acc1.x, acc0.y + acc1.y));
@@ -1462,6 +1468,7 @@ __device__ __forceinline__ void subvol_solve(const CT* __restrict__ F, CT* rhs, 
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int c = l + 4 * k;
+      if (4 * k > r0 + 7) break;
       if (c <= r) cfma(acc0, dblk[c], tvec[c]);
     }
     acc = reduce4(acc0);
@@ -1470,14 +1477,16 @@ __device__ __forceinline__ void subvol_solve(const CT* __restrict__ F, CT* rhs, 
   }
   // backward: x_I = inv(L_II)^dagger (y_I - sum_{J>I} L_JI^dagger x_J), x stored in rhs
   for (int I = NB - 1; I >= 0; --I) {
+    const int e4 = min((fdiv(I * LA_BLK + r0 + 7, L.fd_K) + L.reach + 1) * K - 1, NPAD - 1) >> 2;   // last group of rows
     CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
-    for (int J = I + 1; J < NB; ++J) {
+    for (int J = I + 1; J <= (e4 >> 2); ++J) {
       const CT* blk = F + (size_t)(J * (J + 1) / 2 + I) * 256;
       const CT* xx = rhs + J * LA_BLK;
+      const int k1 = e4 - 4 * J;
       cfma_conj(acc0, blk[l * LA_BLK + r], xx[l]);
-      cfma_conj(acc1, blk[(l + 4) * LA_BLK + r], xx[l + 4]);
-      cfma_conj(acc0, blk[(l + 8) * LA_BLK + r], xx[l + 8]);
-      cfma_conj(acc1, blk[(l + 12) * LA_BLK + r], xx[l + 12]);
+      if (k1 >= 1) cfma_conj(acc1, blk[(l + 4) * LA_BLK + r], xx[l + 4]);
+      if (k1 >= 2) cfma_conj(acc0, blk[(l + 8) * LA_BLK + r], xx[l + 8]);
+      if (k1 >= 3) cfma_conj(acc1, blk[(l + 12) * LA_BLK + r], xx[l + 12]);
     }
     CT acc = reduce4(mkc<CT>(acc0.x + acc1.x, acc0.y + acc1.y));
     if (l == 0) tvec[r] = mkc<CT>(y[I * LA_BLK + r].x - acc.x, y[I * LA_BLK + r].y - acc.y);
@@ -1487,6 +1496,7 @@ __device__ __forceinline__ void subvol_solve(const CT* __restrict__ F, CT* rhs, 
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int cc = l + 4 * k;
+      if (4 * k + 3 < r0) continue;
       if (cc >= r) cfma_conj(acc0, dblk[cc * LA_BLK + r], tvec[cc]);
     }
     acc = reduce4(acc0);
@@ -2105,7 +2115,7 @@ k_sweep_fine(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const typen
   if (use_wide_solve<R, NPAD>())
     subvol_solve_wide<CT, NPAD>(factors + (size_t)b * L.fsize, L.band, sRhs, sY, sT, sRed);
   else
-    subvol_solve<CT, NPAD>(factors + (size_t)b * L.fsize, sRhs, sY, sT, sRed);
+    subvol_solve<CT, NPAD>(L, factors + (size_t)b * L.fsize, sRhs, sY, sT);
   __syncthreads();
   for (int t = tid; t < npts * K; t += kSweepThreads) {
     int i, m;
@@ -2694,7 +2704,7 @@ k_sweep_coarse(LevelGeom L, const R* __restrict__ sigma, const TimeMats* __restr
   if constexpr (kInv) {
     inv.solve(S.Rhs, S.Y, S.Red);
   } else {
-    subvol_solve<CT, NPAD>(factors + (size_t)b * L.fsize, S.Rhs, S.Y, S.T, S.Red);
+    subvol_solve<CT, NPAD>(L, factors + (size_t)b * L.fsize, S.Rhs, S.Y, S.T);
     __syncthreads();
   }
   const SubvolDiv dv(L, e);
