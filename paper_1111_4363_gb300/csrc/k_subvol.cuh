@@ -32,6 +32,12 @@ template <typename CT> __device__ __forceinline__ void cfma_conj(CT& acc, const 
   acc.y = fma(a.x, b.y, acc.y); acc.y = fma(-a.y, b.x, acc.y);
 }
 
+// a -= x conj(y)
+template <typename CT> __device__ __forceinline__ void sub_conj(CT& a, const CT x, const CT y) {
+  a.x = fma(-x.x, y.x, a.x); a.x = fma(-x.y, y.y, a.x);
+  a.y = fma(-x.y, y.x, a.y); a.y = fma(x.x, y.y, a.y);
+}
+
 constexpr int kFactorThreads = 256;
 constexpr int kSweepThreads = 128;
 constexpr int kSuperThreads = 256;   // sweeps with superblock factors
@@ -47,16 +53,22 @@ __device__ __forceinline__ void local_coords(int i, const int e[3], int& x, int&
 // One 256-thread CTA per subvolume of a level; two CTAs per SM.  The padded matrix lives in
 // shared memory as a packed lower triangle (assembled tile-cyclically: thread (tid/16, tid%16)
 // writes entries (16 I + tid/16, 16 J + tid%16)).  Right-looking Cholesky with two barriers per
-// column: (A) column j is scaled by 1/L_jj and published, (B) the trailing triangle is updated
-// with its entries spread linearly over the threads; the thread that updates the next pivot does
-// it first and computes its reciprocal square root while the others are still updating
-// (lookahead), so the pivot chain is off the critical path.
+// pair of columns: (A) the columns are scaled and published, (B) the trailing triangle takes both
+// with its entries spread linearly over the threads; one thread updates the next two pivots first
+// and computes their reciprocal square roots while the others are still updating (lookahead), so
+// the pivot chain is off the critical path.
 __host__ __device__ constexpr int tri_index(int r, int c) { return r * (r + 1) / 2 + c; }
 
 // Small matrices leave most threads of a CTA idle in the later columns, so a CTA factorises
 // factor_mpc(NPAD) matrices together: each phase's work is split over the entries of all of them and
 // they share the two barriers per column.
 __host__ __device__ constexpr int factor_mpc(int npad) { return npad <= 32 ? 8 : (npad <= 64 ? 2 : 1); }
+
+// Bytes of one matrix's pair table, whose place holds a column of the factorisation later.
+__host__ __device__ constexpr size_t factor_pair_bytes(int npair, int npad, size_t csize) {
+  const size_t p = sizeof(double) * (size_t)npair * LA_NPAIR, c = csize * (size_t)npad;
+  return p > c ? p : c;
+}
 
 template <typename R, int NPAD, int MPC>
 __global__ void __launch_bounds__(kFactorThreads, 2)
@@ -69,11 +81,13 @@ k_factor(LevelGeom L, FineOp g, int is_fine, int nptsmax, const R* __restrict__ 
   const int K = tm->K, KK = K * K;
   const int npair_max = nptsmax * (nptsmax + 1) / 2;
   CT* sA = reinterpret_cast<CT*>(smem);                       // [MPC][NTRI] packed lower triangles
-  CT* sCol = sA + MPC * NTRI;                                 // [MPC][NPAD] scaled column j
+  CT* sCol = sA + MPC * NTRI;                                 // [MPC][NPAD] scaled column j of the pair
   R* sInv = reinterpret_cast<R*>(sCol + MPC * NPAD);          // [MPC][NPAD] 1/L_jj
   double* sP = reinterpret_cast<double*>(sInv + MPC * NPAD);  // [9][K*K]
   double* sPair = sP + LA_NPAIR * LA_KMAX * LA_KMAX;          // [MPC][npair_max][9], point pairs i >= j
-  int* sMask = reinterpret_cast<int*>(sPair + (size_t)MPC * npair_max * LA_NPAIR);  // [MPC][npair_max]
+  int* sMask = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(sPair) +
+                                      MPC * factor_pair_bytes(npair_max, NPAD, sizeof(CT)));  // [MPC][npair_max]
+  CT* sCol1 = reinterpret_cast<CT*>(sPair);   // [MPC][NPAD] scaled column j + 1, in the pairs' place after the assembly
 
   const int tid = threadIdx.x, ti = tid >> 4, tk = tid & 15;
   // the CTA's matrices; slots past the last subvolume factorise an identity and store nothing
@@ -177,57 +191,78 @@ k_factor(LevelGeom L, FineOp g, int is_fine, int nptsmax, const R* __restrict__ 
     sA[mi * NTRI + tri_index(r, c)] = mkc<CT>((R)re, (R)im);
   }
   __syncthreads();
-  if (tid < MPC) {
-    CT* A = sA + tid * NTRI;
-    R d2 = A[0].x;
-    if (!(d2 > (R)0)) { atomicOr(status, 1); d2 = (R)1; }
-    const R inv = rsqrt(d2);
-    A[0] = mkc<CT>(d2 * inv, (R)0);
-    sInv[tid * NPAD] = inv;
-  }
-  __syncthreads();
-
-  // ---- right-looking Cholesky.  Work of each phase is spread linearly over exactly the active
-  // entries of all the CTA's matrices (consecutive threads take consecutive entries of a row), so
+  // ---- right-looking Cholesky, two columns at a time.  Work of each phase is spread linearly over exactly the
+  // active entries of all the CTA's matrices (consecutive threads take consecutive entries of a row), so
   // every issued FP64 instruction has all lanes busy except in the last warp of a phase.
-  // Column j ends at the last row its point couples to (L.reach): the rows below stay exact zeros in G and in
-  // the factor, so neither phase visits them (4x4 points x 6, 4096 matrices: 5.61 -> 4.19 ms).
-  for (int j = 0; j < NPAD; ++j) {
-    const int m1 = min(NPAD - 1, (fdiv(j, L.fd_K) + L.reach + 1) * K - 1) - j;
-    // (A) scale and publish column j: rows j+1 .. j+m1 of every matrix
-    {
-      const int rows = m1;
-      for (int t = tid; t < MPC * rows; t += kFactorThreads) {
-        const int mi = t / rows, r = j + 1 + (t - mi * rows);
-        const R inv = sInv[mi * NPAD + j];
-        CT v = sA[mi * NTRI + tri_index(r, j)];
-        v.x *= inv; v.y *= inv;
-        sA[mi * NTRI + tri_index(r, j)] = v;
-        sCol[mi * NPAD + r] = v;
-      }
+  // Columns j, j + 1 end at the last row that the point of j + 1 couples to (L.reach): the rows below stay exact
+  // zeros in G and in the factor, so no phase visits them.  4x4 points x 6, 4096 matrices: 5.61 ms dense and one
+  // column at a time, 4.18 ms with the zeros left out, 3.84 ms with two columns per pair of
+  // barriers.
+  // The pivots of columns j and j + 1 and the entry between them, by one thread per matrix; u0, u1: the values
+  // still to be subtracted from the rows j and j + 1 (of the two columns before).
+  auto pivots = [&](int mi, int j, const CT* c0, const CT* c1, int last) {
+    CT* A = sA + mi * NTRI;
+    const CT zero = mkc<CT>((R)0, (R)0);
+    CT a00 = A[tri_index(j, j)], a10 = A[tri_index(j + 1, j)], a11 = A[tri_index(j + 1, j + 1)];
+    if (c0) {
+      const CT x0 = j <= last ? c0[j] : zero, x1 = j <= last ? c1[j] : zero;
+      const CT y0 = j + 1 <= last ? c0[j + 1] : zero, y1 = j + 1 <= last ? c1[j + 1] : zero;
+      sub_conj(a00, x0, x0); sub_conj(a00, x1, x1);
+      sub_conj(a10, y0, x0); sub_conj(a10, y1, x1);
+      sub_conj(a11, y0, y0); sub_conj(a11, y1, y1);
+    }
+    R d0 = a00.x;
+    if (!(d0 > (R)0)) { atomicOr(status, 1); d0 = (R)1; }
+    const R i0 = rsqrt(d0);
+    const CT l = mkc<CT>(a10.x * i0, a10.y * i0);
+    sub_conj(a11, l, l);
+    R d1 = a11.x;
+    if (!(d1 > (R)0)) { atomicOr(status, 1); d1 = (R)1; }
+    const R i1 = rsqrt(d1);
+    A[tri_index(j, j)] = mkc<CT>(d0 * i0, (R)0);
+    A[tri_index(j + 1, j)] = l;
+    A[tri_index(j + 1, j + 1)] = mkc<CT>(d1 * i1, (R)0);
+    sInv[mi * NPAD + j] = i0;
+    sInv[mi * NPAD + j + 1] = i1;
+  };
+  if (tid < MPC) pivots(tid, 0, nullptr, nullptr, 0);
+  __syncthreads();
+  for (int j = 0; j + 2 < NPAD; j += 2) {
+    const int last = min(NPAD - 1, (fdiv(j + 1, L.fd_K) + L.reach + 1) * K - 1);
+    const int rows = last - j - 1;   // rows j + 2 .. last
+    // (A) columns j and j + 1, scaled and published
+    for (int t = tid; t < MPC * rows; t += kFactorThreads) {
+      const int mi = t / rows, r = j + 2 + (t - mi * rows);
+      CT* A = sA + mi * NTRI;
+      const R i0 = sInv[mi * NPAD + j], i1 = sInv[mi * NPAD + j + 1];
+      CT v = A[tri_index(r, j)], w = A[tri_index(r, j + 1)];
+      v.x *= i0; v.y *= i0;
+      sub_conj(w, v, A[tri_index(j + 1, j)]);
+      w.x *= i1; w.y *= i1;
+      A[tri_index(r, j)] = v;
+      A[tri_index(r, j + 1)] = w;
+      sCol[mi * NPAD + r] = v;
+      sCol1[mi * NPAD + r] = w;
     }
     __syncthreads();
-    // (B) trailing update of the entries (r, c), j < c <= r; entry e of a trailing triangle lies
-    // in row r = j + m with (m-1) m / 2 <= e < m (m+1) / 2.  e = 0 is the next pivot: its thread
-    // finishes it first and computes the reciprocal square root (lookahead).
-    const int T = m1 * (m1 + 1) / 2;
-    for (int t = tid; t < MPC * T; t += kFactorThreads) {
-      const int mi = t / T, e = t - mi * T;
+    // (B) trailing update of the entries (r, c), j + 2 <= c <= r <= last; entry e of a trailing triangle lies in row
+    // j + 1 + m with (m-1) m / 2 <= e < m (m+1) / 2.  The first three hold the next two pivots: one thread per
+    // matrix updates them and takes the reciprocal square roots while the others go on (lookahead).
+    if (tid < MPC) {
+      pivots(tid, j + 2, sCol + tid * NPAD, sCol1 + tid * NPAD, last);
+    }
+    const int T = rows * (rows + 1) / 2 - 3;
+    for (int t = kFactorThreads - 1 - tid; t < MPC * T; t += kFactorThreads) {
+      const int mi = MPC > 1 ? t / T : 0, e = t - mi * T + 3;
       int m = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)e)) * 0.5f);
       while ((m - 1) * m / 2 > e) --m;
       while (m * (m + 1) / 2 <= e) ++m;
-      const int r = j + m, c = j + 1 + (e - (m - 1) * m / 2);
-      const CT xr = sCol[mi * NPAD + r], y = sCol[mi * NPAD + c];
+      const int r = j + 1 + m, c = j + 2 + (e - (m - 1) * m / 2);
+      const CT* c0 = sCol + mi * NPAD;
+      const CT* c1 = sCol1 + mi * NPAD;
       CT a = sA[mi * NTRI + tri_index(r, c)];
-      a.x = fma(-xr.x, y.x, a.x); a.x = fma(-xr.y, y.y, a.x);
-      a.y = fma(-xr.y, y.x, a.y); a.y = fma(xr.x, y.y, a.y);
-      if (e == 0) {
-        R d2 = a.x;
-        if (!(d2 > (R)0)) { atomicOr(status, 1); d2 = (R)1; }
-        const R inv = rsqrt(d2);
-        a = mkc<CT>(d2 * inv, (R)0);
-        sInv[mi * NPAD + j + 1] = inv;
-      }
+      sub_conj(a, c0[r], c0[c]);
+      sub_conj(a, c1[r], c1[c]);
       sA[mi * NTRI + tri_index(r, c)] = a;
     }
     __syncthreads();
@@ -1588,6 +1623,7 @@ __device__ __forceinline__ void subvol_solve_wide(const CT* __restrict__ F, int 
       CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
 #pragma unroll
       for (int J = 0; J < I; ++J) {
+        if (J < I - band) continue;   // zero blocks: their products would still take the pipe
         cfma(acc0, cur[J].a(), y[J * LA_BLK + 2 * q]);
         cfma(acc1, cur[J].b(), y[J * LA_BLK + 2 * q + 1]);
       }
@@ -1636,6 +1672,7 @@ __device__ __forceinline__ void subvol_solve_wide(const CT* __restrict__ F, int 
       CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
 #pragma unroll
       for (int J = I + 1; J < NB; ++J) {
+        if (J > I + band) continue;
         cfma_conj(acc0, cur[J].a(), rhs[J * LA_BLK + 2 * q]);
         cfma_conj(acc1, cur[J].b(), rhs[J * LA_BLK + 2 * q + 1]);
       }
@@ -2763,7 +2800,8 @@ inline size_t factor_smem(const LevelGeom& L, int nptsmax, size_t csize, int mpc
   const size_t npair = (size_t)nptsmax * (nptsmax + 1) / 2;
   const size_t mpc = (size_t)mpc_;
   return mpc * (csize * (ntri + L.npad) + (size_t)L.npad * (csize / 2)) +
-         sizeof(double) * (LA_NPAIR * LA_KMAX * LA_KMAX + mpc * npair * LA_NPAIR) + sizeof(int) * (mpc * npair + 1);
+         sizeof(double) * LA_NPAIR * LA_KMAX * LA_KMAX + mpc * factor_pair_bytes((int)npair, L.npad, csize) +
+         sizeof(int) * (mpc * npair + 1);
 }
 // Factors with inverted diagonal superblocks (k_factor_band): complex64, more than 128 unknowns and a band of
 // at most 8 blocks, the largest window k_factor_band keeps in registers.
