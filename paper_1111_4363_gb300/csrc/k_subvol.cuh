@@ -1479,20 +1479,27 @@ __device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __res
   // A factor has no entry further than L.reach points from its diagonal: a warp's eight rows start at the first
   // column its first row couples to and (backward) its eight columns end at the last row its last column
   // couples to, in steps of the four columns that the lanes of a row take together.  Predicated lanes would
-  // still occupy the FP64 pipe, so the bounds are the warp's.
+  // still occupy the FP64 pipe, so the bounds are the warp's.  The block that a bound cuts stands outside the loop
+  // over whole blocks, whose loads can then be issued ahead.
   const int K = L.fd_K.d;
   // forward: y_I = inv(L_II) (rhs_I - sum_{J<I} L_IJ y_J)
   for (int I = 0; I < NB; ++I) {
     const CT* rowblk = F + (size_t)(I * (I + 1) / 2) * 256;
     const int c0 = max((fdiv(I * LA_BLK + r0, L.fd_K) - L.reach) * K, 0) >> 2;   // first group of four columns
     CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
-    for (int J = c0 >> 2; J < I; ++J) {
+    if ((c0 & 3) && (c0 >> 2) < I) {
+      const CT* blk = rowblk + (c0 >> 2) * 256 + r * LA_BLK;
+      const CT* yy = y + (c0 >> 2) * LA_BLK;
+      if ((c0 & 3) <= 1) cfma(acc1, blk[l + 4], yy[l + 4]);
+      if ((c0 & 3) <= 2) cfma(acc0, blk[l + 8], yy[l + 8]);
+      cfma(acc1, blk[l + 12], yy[l + 12]);
+    }
+    for (int J = (c0 + 3) >> 2; J < I; ++J) {
       const CT* blk = rowblk + J * 256 + r * LA_BLK;
       const CT* yy = y + J * LA_BLK;
-      const int k0 = c0 - 4 * J;
-      if (k0 <= 0) cfma(acc0, blk[l], yy[l]);
-      if (k0 <= 1) cfma(acc1, blk[l + 4], yy[l + 4]);
-      if (k0 <= 2) cfma(acc0, blk[l + 8], yy[l + 8]);
+      cfma(acc0, blk[l], yy[l]);
+      cfma(acc1, blk[l + 4], yy[l + 4]);
+      cfma(acc0, blk[l + 8], yy[l + 8]);
       cfma(acc1, blk[l + 12], yy[l + 12]);
     }
     CT acc = reduce4(mkc<CT>(acc0.x + acc1.x, acc0.y + acc1.y));
@@ -1514,14 +1521,21 @@ __device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __res
   for (int I = NB - 1; I >= 0; --I) {
     const int e4 = min((fdiv(I * LA_BLK + r0 + 7, L.fd_K) + L.reach + 1) * K - 1, NPAD - 1) >> 2;   // last group of rows
     CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
-    for (int J = I + 1; J <= (e4 >> 2); ++J) {
+    const int Jf = (e4 + 1) >> 2, k1 = (e4 + 1) & 3;   // the first block not taken whole, its groups
+    for (int J = I + 1; J < Jf; ++J) {
       const CT* blk = F + (size_t)(J * (J + 1) / 2 + I) * 256;
       const CT* xx = rhs + J * LA_BLK;
-      const int k1 = e4 - 4 * J;
       cfma_conj(acc0, blk[l * LA_BLK + r], xx[l]);
-      if (k1 >= 1) cfma_conj(acc1, blk[(l + 4) * LA_BLK + r], xx[l + 4]);
-      if (k1 >= 2) cfma_conj(acc0, blk[(l + 8) * LA_BLK + r], xx[l + 8]);
-      if (k1 >= 3) cfma_conj(acc1, blk[(l + 12) * LA_BLK + r], xx[l + 12]);
+      cfma_conj(acc1, blk[(l + 4) * LA_BLK + r], xx[l + 4]);
+      cfma_conj(acc0, blk[(l + 8) * LA_BLK + r], xx[l + 8]);
+      cfma_conj(acc1, blk[(l + 12) * LA_BLK + r], xx[l + 12]);
+    }
+    if (k1 && Jf > I) {
+      const CT* blk = F + (size_t)(Jf * (Jf + 1) / 2 + I) * 256;
+      const CT* xx = rhs + Jf * LA_BLK;
+      cfma_conj(acc0, blk[l * LA_BLK + r], xx[l]);
+      if (k1 >= 2) cfma_conj(acc1, blk[(l + 4) * LA_BLK + r], xx[l + 4]);
+      if (k1 >= 3) cfma_conj(acc0, blk[(l + 8) * LA_BLK + r], xx[l + 8]);
     }
     CT acc = reduce4(mkc<CT>(acc0.x + acc1.x, acc0.y + acc1.y));
     if (l == 0) tvec[r] = mkc<CT>(y[I * LA_BLK + r].x - acc.x, y[I * LA_BLK + r].y - acc.y);
@@ -1566,6 +1580,8 @@ __device__ __forceinline__ CPair<double2> load_colpair<double2>(const double2* b
   return p;
 }
 
+constexpr unsigned kPipeBoundCtas = 304;
+
 template <typename CT>
 __device__ __forceinline__ CT reduce_xor(CT v, int m) {
   v.x += __shfl_xor_sync(0xffffffffu, v.x, m);
@@ -1595,7 +1611,9 @@ __device__ __forceinline__ void load_fwd_band(CPair<CT>& p, const CT* a, bool in
   else p.load_zero();
 }
 
-template <typename CT, int NPAD>
+// SKIP leaves the products of zero blocks out: worth it where the FP64 pipe is the bound; its branches keep loads from
+// being issued ahead, which costs more where a few CTAs wait on latency.
+template <typename CT, int NPAD, bool SKIP>
 __device__ __forceinline__ void subvol_solve_wide(const CT* __restrict__ F, int band, CT* rhs, CT* y, CT* tvec,
                                                   CT* part) {
   constexpr int NB = NPAD / LA_BLK;
@@ -1623,7 +1641,7 @@ __device__ __forceinline__ void subvol_solve_wide(const CT* __restrict__ F, int 
       CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
 #pragma unroll
       for (int J = 0; J < I; ++J) {
-        if (J < I - band) continue;   // zero blocks: their products would still take the pipe
+        if (SKIP && J < I - band) continue;   // zero blocks: their products would still take the pipe
         cfma(acc0, cur[J].a(), y[J * LA_BLK + 2 * q]);
         cfma(acc1, cur[J].b(), y[J * LA_BLK + 2 * q + 1]);
       }
@@ -1672,7 +1690,7 @@ __device__ __forceinline__ void subvol_solve_wide(const CT* __restrict__ F, int 
       CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
 #pragma unroll
       for (int J = I + 1; J < NB; ++J) {
-        if (J > I + band) continue;
+        if (SKIP && J > I + band) continue;
         cfma_conj(acc0, cur[J].a(), rhs[J * LA_BLK + 2 * q]);
         cfma_conj(acc1, cur[J].b(), rhs[J * LA_BLK + 2 * q + 1]);
       }
@@ -2149,9 +2167,14 @@ k_sweep_fine(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const typen
     sRhs[t] = out;
   }
   __syncthreads();
-  if (use_wide_solve<R, NPAD>())
-    subvol_solve_wide<CT, NPAD>(factors + (size_t)b * L.fsize, L.band, sRhs, sY, sT, sRed);
-  else
+  // FP64 from about two CTAs per SM on is bound by its pipe (4x4x4 x 4, a colour of 512 subvolumes: 488 us with every
+  // product, 445 us without; of 12: 149 and 171 us)
+  if (use_wide_solve<R, NPAD>()) {
+    if (sizeof(R) == 8 && gridDim.x > kPipeBoundCtas)
+      subvol_solve_wide<CT, NPAD, true>(factors + (size_t)b * L.fsize, L.band, sRhs, sY, sT, sRed);
+    else
+      subvol_solve_wide<CT, NPAD, false>(factors + (size_t)b * L.fsize, L.band, sRhs, sY, sT, sRed);
+  } else
     subvol_solve<CT, NPAD>(L, factors + (size_t)b * L.fsize, sRhs, sY, sT);
   __syncthreads();
   for (int t = tid; t < npts * K; t += kSweepThreads) {
@@ -2980,7 +3003,7 @@ cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeM
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  return launch_overlapped(L.overlap, kern, nblocks, kSweepThreads, smem, s, L, g, tm, f, yx, c, factors, colour);
+  return launch_overlapped(L.overlap && sizeof(R) == 4, kern, nblocks, kSweepThreads, smem, s, L, g, tm, f, yx, c, factors, colour);
   }
 }
 template <typename R, int NPAD>
@@ -2998,7 +3021,7 @@ cudaError_t launch_sweep_coarse_n(const LevelGeom& L, const R* sigma, const Time
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  return launch_overlapped(L.overlap, kern, nblocks, kSweepThreads, smem, s, L, sigma, tm, gvec, e, factors, colour, status);
+  return launch_overlapped(L.overlap && sizeof(R) == 4, kern, nblocks, kSweepThreads, smem, s, L, sigma, tm, gvec, e, factors, colour, status);
 }
 
 template <typename R>
@@ -3014,7 +3037,7 @@ cudaError_t launch_gresid_tiles_r(const LevelGeom& L, const R* sigma, const Time
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  return launch_overlapped(L.overlap, kern, L.nsub, kSweepThreads, smem, s, L, sigma, tm, gvec, e, out, L.npad);
+  return launch_overlapped(L.overlap && sizeof(R) == 4, kern, L.nsub, kSweepThreads, smem, s, L, sigma, tm, gvec, e, out, L.npad);
 }
 
 // finest-level sweeps and factorisations also take the wide sizes

@@ -458,9 +458,11 @@ cudaError_t launch_sweep_coarse(const LevelGeom& L, const R* sigma, const TimeMa
 // visible (at once for an ordinary launch).  Whatever a predecessor of the running chain may write - the level
 // vectors, right-hand sides, residuals - is read or written after overlap_wait only; factors, stencils, time
 // matrices and the potential are final before a chain begins.  It hides the launch latency and the constant
-// loads of the many short kernels of a V-cycle.  Launches of more than kOverlapMax CTAs, about two per SM, go
-// out in the ordinary way: they are not bound by their launch, and early successors only took their issue
-// slots (256^2 FP64, sweeps of 1024 CTAs: 43.2 ms without, 48.3 ms with overlap).
+// loads of the many short kernels of a complex64 V-cycle.  Launches of more than kOverlapMax CTAs, about two per
+// SM, go out in the ordinary way: they are not bound by their launch, and early successors only took their
+// issue slots (3D 128^3 mixed: 124.2 ms without, 127.5 ms with every launch overlapped).  So do FP64 launches, which
+// the early successors' FP64 conversions slow down (22x12x32 points, 4x4x4 x 4: 20.3 ms without, 25.2 ms with;
+// 256^2 with every sweep: 43.2 and 48.3 ms).
 constexpr unsigned kOverlapMax = 304;
 __device__ __forceinline__ void overlap_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void overlap_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
