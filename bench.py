@@ -42,12 +42,12 @@ METRIC = "spacetime unknowns relaxed/s"
 # (set to None when a kernel changes):
 # - 2D 256x256 FP64: the finest k_factor launch (4096 subvolumes) and one full k_sweep_fine sweep (four
 #   colour launches), profiles/dram_2d_softcore_256x256_fp64.md
-# - 3D 128^3 complex64: one k_factor_wide launch (32768 subvolumes of 256 unknowns) and one full wide
+# - 3D 128^3 complex64: one k_factor_band launch (32768 subvolumes of 256 unknowns) and one full k_sweep_super
 #   sweep (eight colour launches of 4096), profiles/dram_3d_hydrogen_128x128x128_mixed.md
 NCU_BYTES_PER_SUBVOLUME = {("factor", 0): (867072 + 287257600) / 4096,
                            ("sweep", 0): (390778880 + 216064) / 4096,
-                           ("factor_wide", 1): (33378560 + 9068625920) / 32768,
-                           ("sweep_wide", 1): (10943546368 + 56069376) / 32768}
+                           ("factor_wide", 1): (19604992 + 7257668864) / 32768,
+                           ("sweep_wide", 1): (9965988608 + 61851392) / 32768}
 FP64_PEAK_TFLOPS = 152 * 4 * 2070e6 / 1e12   # 152 SMs x 4 FP64 flop/clk/SM x 2070 MHz (derived)
 FP32_PEAK_TFLOPS = 152 * 256 * 2070e6 / 1e12  # 152 SMs x 128 FP32 lanes x 2 flop (FMA) x 2070 MHz (derived)
 L2_BYTES = 129 * 2 ** 20
@@ -256,11 +256,14 @@ def dominant_roofline(prof, w, precision, ms_total, traffic_ok, peaks=None):
     swp_ms_full = prof["ms_sweep"] / max(prof["n_sweep"], 1)   # one event pair per full sweep
     nsub, fbytes = finest_factor_store(w, precision)
     wide = fbytes // (16 if precision == 0 else 8) > 136 * 128   # more than 128 unknowns: global-memory factor
-    fac_name = "k_factor_wide" if wide else ("k_factor" if precision == 0 else "k_factor_blk")
+    # complex64 with more than 128 unknowns: the register-window variants (band of at most 8 blocks)
+    fac_name = (("k_factor_wide" if precision == 0 else "k_factor_wide: k_factor_band") if wide
+                else ("k_factor" if precision == 0 else "k_factor_blk"))
     if prof["ms_factor"] >= prof["ms_sweep"]:
         dom, flops, dms, cls = f"{fac_name} (finest level)", prof["flops_factor"], fac_ms, "factor"
     else:
-        dom, flops, dms, cls = "k_sweep_fine (one sweep, all colours)", prof["flops_sweep"], swp_ms_full, "sweep"
+        swp_name = "k_sweep_fine: k_sweep_super" if wide and precision == 1 else "k_sweep_fine"
+        dom, flops, dms, cls = f"{swp_name} (one sweep, all colours)", prof["flops_sweep"], swp_ms_full, "sweep"
     bps = NCU_BYTES_PER_SUBVOLUME.get((cls + ("_wide" if wide else ""), precision)) if traffic_ok else None
     traffic = round(bps * nsub) if bps else None
     kms = {"factor_per_launch": round(fac_ms, 4), "sweep_full": round(swp_ms_full, 4),
@@ -306,7 +309,7 @@ def stencil_roofline(prof, precision, c64=False):
     peak, note = hbm_peak()
     gbs = prof[by] / (prof[ms] * 1e-3) / 1e9
     return {"bound": "hbm", "kernel": ("k_stencil_tma / k_mresid complex64 (V-cycle residual)" if c64 else
-                                       "k_mresid FP64 (action residual, S1)"),
+                                       "k_residual FP64 (action residual, S1)"),
             "achieved": round(gbs, 1), "peak": peak, "unit": "GB/s", "frac": round(gbs / peak, 4), "peak_note": note,
             "launches": prof[n], "us_per_launch": round(1e3 * prof[ms] / prof[n], 2),
             "note": ("bound by the FP64 pipe, not by HBM" if not c64 else
