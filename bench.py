@@ -40,10 +40,11 @@ METRIC = "spacetime unknowns relaxed/s"
 # (kernel class, precision) -> DRAM bytes (read + write) per finest-level subvolume of the current kernels,
 # from one-pass ncu captures of full-size launches, scaled to a launch by the subvolumes it processes
 # (set to None when a kernel changes):
-# - 2D 256x256 FP64: one full k_sweep_fine sweep (four colour launches), profiles/dram_2d_softcore_256x256_fp64.md
+# - 2D 256x256 FP64: the finest k_factor launch (4096 subvolumes) and one full k_sweep_fine sweep (four
+#   colour launches), profiles/dram_2d_softcore_256x256_fp64.md
 # - 3D 128^3 complex64: one k_factor_band launch (32768 subvolumes of 256 unknowns) and one full k_sweep_super
 #   sweep (eight colour launches of 4096), profiles/dram_3d_hydrogen_128x128x128_mixed.md
-NCU_BYTES_PER_SUBVOLUME = {("factor", 0): None,
+NCU_BYTES_PER_SUBVOLUME = {("factor", 0): (772608 + 286944000) / 4096,
                            ("sweep", 0): (330939648 + 530432) / 4096,
                            ("factor_wide", 1): (19604992 + 7257668864) / 32768,
                            ("sweep_wide", 1): (9965988608 + 61851392) / 32768}
