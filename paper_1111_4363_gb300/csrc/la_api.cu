@@ -19,6 +19,7 @@ using namespace la;
 struct la_ctx {
   la_config cfg;
   cudaStream_t stream = 0;
+  int device = 0;           // the device that holds the context's memory and runs its kernels
   std::string err;
   int K = 0, L = 0, dim = 0, np0 = 0;
   long long nunk0 = 0;
@@ -422,11 +423,12 @@ extern "C" la_status la_init(const la_config* cfg, void* stream, la_ctx** out) {
     c->have_map_e32 = encode_stencil_map(c->fine, c->K, c->d_e32, &c->map_e32);
     c->have_map_z32 = encode_stencil_map(c->fine, c->K, c->d_z32, &c->map_z32);
   }
-  if (cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess ||
+  if (cudaGetDevice(&c->device) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess ||
       cudaMallocHost(&c->h_N, sizeof(double) * 2) != cudaSuccess) {
-    g_init_error = "stream, event or pinned-buffer creation failed";
+    g_init_error = "device query, stream, event or pinned-buffer creation failed";
     la_finalize(c);
     return LA_ECUDA;
   }
@@ -1435,8 +1437,16 @@ extern "C" la_status la_residual(la_ctx* c, const void* psi0, double t0, const v
   if (!c || !psi0 || !cin) return c ? fail(c, LA_EINVAL, "invalid argument") : LA_EINVAL;
   if (!c->have_ham) return fail(c, LA_ESTATE, "la_set_hamiltonian must be called first");
   LA_TRY(load_any(c, c->d_psi, psi0, sizeof(double2) * (size_t)c->np0));
-  // coefficients and residual that live on the device, aligned as the kernel reads them, are used in place
-  const auto in_place = [](const void* p) { return is_device_ptr(p) && (reinterpret_cast<uintptr_t>(p) & 31) == 0; };
+  // coefficients and residual that live on the context's device, aligned as the kernel reads them, are used in
+  // place; all others (host or managed memory, another GPU's) are copied
+  const auto in_place = [c](const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return usable_in_place(a, c->device, p);
+  };
   const size_t cb = sizeof(double2) * (size_t)c->nunk0;
   const double2* cd = (const double2*)cin;
   const unsigned char *c0 = (const unsigned char*)cin, *r0 = (const unsigned char*)r_out;

@@ -348,6 +348,13 @@ __host__ inline int matrix_reach(int dim, const int sub[3], int man, int box) {
   return reach;
 }
 
+// Whether the kernels of a context on `device` may read or write caller memory p in place: memory of that
+// device (another GPU's is reachable from a kernel only with peer access enabled, which a caller need not have
+// done, while a copy always works) on the 32-byte boundary of the FP64 records' widest access.
+__host__ inline bool usable_in_place(const cudaPointerAttributes& a, int device, const void* p) {
+  return a.type == cudaMemoryTypeDevice && a.device == device && (reinterpret_cast<uintptr_t>(p) & 31) == 0;
+}
+
 template <typename R> struct C2;
 template <> struct C2<double> { typedef double2 T; };
 template <> struct C2<float> { typedef float2 T; };
