@@ -868,8 +868,7 @@ __global__ void k_restrict(LevelGeom F, LevelGeom C, const CT* __restrict__ sf, 
 // 4 x 4 (x 4) children there, in the same order and with the same weights as k_restrict.
 constexpr int kRx = 8, kRy = 4, kRz = 2;
 template <typename CT, int K>
-__global__ void __launch_bounds__(256) k_restrict_tile(LevelGeom F, LevelGeom C, const CT* __restrict__ sf,
-                                                       CT* __restrict__ gc, CT* __restrict__ ec) {
+__global__ void __launch_bounds__(256) k_restrict_tile(LevelGeom F, LevelGeom C, const CT* sf, CT* gc, CT* ec) {
   typedef typename CR<CT>::R RR;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   overlap_trigger();
@@ -922,7 +921,7 @@ __global__ void __launch_bounds__(256) k_restrict_tile(LevelGeom F, LevelGeom C,
 }
 
 template <typename CT, int K>
-__global__ void k_prolong_add(LevelGeom F, LevelGeom C, const CT* __restrict__ ec, CT* __restrict__ ef) {
+__global__ void k_prolong_add(LevelGeom F, LevelGeom C, const CT* ec, CT* ef) {
   typedef typename CR<CT>::R RR;
   overlap_trigger();
   overlap_wait();

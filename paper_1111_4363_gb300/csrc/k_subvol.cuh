@@ -1961,9 +1961,9 @@ __host__ __device__ constexpr bool use_wide_solve() {
 // z = Wt r, right-hand side (M~^dagger z)_U, solve, c_U += delta.
 template <typename R, int NPAD>
 __global__ void __launch_bounds__(kSweepThreads)
-k_sweep_fine(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const typename C2<R>::T* __restrict__ f,
-             const typename C2<R>::T* __restrict__ yx, typename C2<R>::T* __restrict__ c,
-             const typename C2<R>::T* __restrict__ factors, int colour) {
+k_sweep_fine(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const typename C2<R>::T* f,
+             const typename C2<R>::T* yx, typename C2<R>::T* c, const typename C2<R>::T* __restrict__ factors,
+             int colour) {
   typedef typename C2<R>::T CT;
   extern __shared__ __align__(16) unsigned char smem[];
   overlap_trigger();
@@ -2296,8 +2296,7 @@ __device__ __forceinline__ void load_time_f32(const TimeMats* __restrict__ tm, f
 template <int K, bool WARP>
 __device__ __forceinline__ void sweep_rhs(const LevelGeom& L, const FineOp& g, const SweepBox& B, int tid, int NT,
                                           int npad, const float* sM, float* sV, float2* sC, float2* sZ, float2* sRhs,
-                                          const float2* __restrict__ f, const float2* __restrict__ yx,
-                                          const float2* __restrict__ c) {
+                                          const float2* f, const float2* yx, const float2* c) {
   constexpr int KK = K * K;
   auto sync = [] {
     if (WARP) __syncwarp();
@@ -2447,7 +2446,7 @@ __device__ __forceinline__ void sweep_rhs(const LevelGeom& L, const FineOp& g, c
 // c of unknown t of U plus delta, with c_U still in sC.
 template <int K>
 __device__ __forceinline__ void sweep_update(const LevelGeom& L, const FineOp& g, const SweepBox& B, int t, float2 d,
-                                             const float2* sC, float2* __restrict__ c) {
+                                             const float2* sC, float2* c) {
   const int i = t / K, m = t - i * K;
   int lx, ly, lz;
   SweepBox::coords(i, B.du0, B.du1, lx, ly, lz);
@@ -2464,9 +2463,8 @@ __device__ __forceinline__ void sweep_update(const LevelGeom& L, const FineOp& g
 // (116 us); an L2 prefetch of the band at the start of the CTA costs 7 us.
 template <int NPAD, int K>
 __global__ void __launch_bounds__(kSuperThreads, K <= 4 ? 4 : 2)
-k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const float2* __restrict__ f,
-              const float2* __restrict__ yx, float2* __restrict__ c, const float2* __restrict__ factors, int colour,
-              FastDiv dn0, FastDiv dn1) {
+k_sweep_super(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const float2* f, const float2* yx, float2* c,
+              const float2* __restrict__ factors, int colour, FastDiv dn0, FastDiv dn1) {
   extern __shared__ __align__(16) unsigned char smem[];
   overlap_trigger();
   const int tid = threadIdx.x;
@@ -2508,9 +2506,8 @@ __host__ __device__ __forceinline__ SuperSmem small_smem(const LevelGeom& L, int
 }
 template <int NPAD, int K>
 __global__ void __launch_bounds__(32 * kSmallSweepWarps)
-k_sweep_small(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const float2* __restrict__ f,
-              const float2* __restrict__ yx, float2* __restrict__ c, const float2* __restrict__ factors, int colour,
-              FastDiv dn0, FastDiv dn1, int count) {
+k_sweep_small(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const float2* f, const float2* yx, float2* c,
+              const float2* __restrict__ factors, int colour, FastDiv dn0, FastDiv dn1, int count) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NB = NPAD / LA_BLK, NG = NPAD / 8;   // blocks per side; groups of eight rows
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, row = l >> 2, q = l & 3;
@@ -2653,8 +2650,8 @@ struct SubvolDiv {
 // Fills S.Rhs[0..npad) with (g - G e) on the subvolume with origin o and extent e (0 in padding).
 template <typename R>
 __device__ inline void coarse_rhs(const LevelGeom& L, const R* __restrict__ sigma,
-                                  const TimeMats* __restrict__ tm, const typename C2<R>::T* __restrict__ gvec,
-                                  const typename C2<R>::T* __restrict__ ev, const int o[3], const int e[3], int npad,
+                                  const TimeMats* __restrict__ tm, const typename C2<R>::T* gvec,
+                                  const typename C2<R>::T* ev, const int o[3], const int e[3], int npad,
                                   const CoarseSmem<R>& S) {
   typedef typename C2<R>::T CT;
   const int K = tm->K, KK = K * K;
@@ -2746,8 +2743,8 @@ __device__ inline void coarse_rhs(const LevelGeom& L, const R* __restrict__ sigm
 template <typename R, int NPAD>
 __global__ void __launch_bounds__(kSweepThreads)
 k_sweep_coarse(LevelGeom L, const R* __restrict__ sigma, const TimeMats* __restrict__ tm,
-               const typename C2<R>::T* __restrict__ gvec, typename C2<R>::T* __restrict__ ev,
-               const typename C2<R>::T* __restrict__ factors, int colour, int* __restrict__ status) {
+               const typename C2<R>::T* gvec, typename C2<R>::T* ev,
+               const typename C2<R>::T* __restrict__ factors, int colour, int* status) {
   typedef typename C2<R>::T CT;
   extern __shared__ __align__(16) unsigned char smem[];
   overlap_trigger();
@@ -2787,8 +2784,7 @@ k_sweep_coarse(LevelGeom L, const R* __restrict__ sigma, const TimeMats* __restr
 template <typename R>
 __global__ void __launch_bounds__(kSweepThreads)
 k_gresid_tiles(LevelGeom L, const R* __restrict__ sigma, const TimeMats* __restrict__ tm,
-               const typename C2<R>::T* __restrict__ gvec, const typename C2<R>::T* __restrict__ ev,
-               typename C2<R>::T* __restrict__ out, int npad) {
+               const typename C2<R>::T* gvec, const typename C2<R>::T* ev, typename C2<R>::T* out, int npad) {
   typedef typename C2<R>::T CT;
   extern __shared__ __align__(16) unsigned char smem[];
   overlap_trigger();

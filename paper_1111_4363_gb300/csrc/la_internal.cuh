@@ -464,7 +464,10 @@ cudaError_t launch_sweep_coarse(const LevelGeom& L, const R* sigma, const TimeMa
 // called overlap_trigger (or ended); overlap_wait returns when that kernel has finished and its writes are
 // visible (at once for an ordinary launch).  Whatever a predecessor of the running chain may write - the level
 // vectors, right-hand sides, residuals - is read or written after overlap_wait only; factors, stencils, time
-// matrices and the potential are final before a chain begins.  It hides the launch latency and the constant
+// matrices and the potential are final before a chain begins.  The pointers to what a predecessor writes carry no
+// __restrict__: with const it promises data that nothing changes while the kernel runs, which the compiler may turn
+// into non-coherent loads (ld.global.nc) that overlap_wait does not order; the coherent loads cost nothing measurable
+// here.  It hides the launch latency and the constant
 // loads of the many short kernels of a complex64 V-cycle.  Launches of more than kOverlapMax CTAs, about two per
 // SM, go out in the ordinary way: they are not bound by their launch, and early successors only took their
 // issue slots (3D 128^3 mixed: 124.2 ms without, 127.5 ms with every launch overlapped).  So do FP64 launches, which
