@@ -14,15 +14,22 @@ constexpr int kSmallManyMin = 1216;    // ... (8 per SM); with fewer, or factor_
 // of inv(L) for c < j, so that column j, once eliminated, holds inv(L)'s.  Rows are scaled by d^{-1/2} at the
 // end.  The registers rotate by one column per step (register c holds column (j + c) mod NP), which keeps the
 // loop rolled without a dynamic register index; u passes through shared memory, 16 bytes a load.
-// No barrier but the warp's: 7200 matrices of 32 unknowns (8 points x 4) take 94 us, half of the issue slots busy,
-// against 161 us for four matrices per 256-thread CTA with two barriers per column.
+// H and H^2 of a finest-level point pair are formed in FP64 and rounded once (D_i + D_j may cancel), as the larger
+// shared-memory factorisations do.  No barrier but the warp's: 7200 matrices of 32 unknowns (8 points x 4) take
+// 97 us (96 us with the pairs in FP32), half of the issue slots busy, against 161 us for four matrices per
+// 256-thread CTA with two barriers per column.
 template <int NP, int K, bool FINE>
 __global__ void __launch_bounds__(32 * kSmallWarps)
 k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const TimeMats* __restrict__ tm,
                float2* __restrict__ factors, int* __restrict__ status) {
   constexpr int KK = K * K, JMAX = NP / K;   // points of a full subvolume of this size class, at most
   __shared__ float sP[LA_NPAIR * KK], sPd[2 * KK];
-  __shared__ float sD[kSmallWarps][32], sX[kSmallWarps][32], sN[kSmallWarps][32];
+  // FINE: D = dsum + V0 and the in-grid neighbours' weights of H^2's diagonal per point, and (H, H^2) of the point pairs
+  // i >= j of each matrix
+  constexpr int NPAIR = JMAX * (JMAX + 1) / 2;
+  __shared__ double sD[kSmallWarps][FINE ? 32 : 1], sN[kSmallWarps][FINE ? 32 : 1];
+  __shared__ float2 sHH[kSmallWarps][FINE ? (32 / NP) * NPAIR : 1];
+  __shared__ float sX[kSmallWarps][32];
   __shared__ int sXYZ[kSmallWarps][32];
   __shared__ __align__(16) float2 sBuf[kSmallWarps][2][32];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, r = lane & (NP - 1), half = lane / NP;
@@ -34,7 +41,7 @@ k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const Tim
     subvol_box(L, b, o, e);
     npts = e[0] * e[1] * e[2];
   }
-  const float wx = (float)(0.5 * g.ih2[0]), wy = (float)(0.5 * g.ih2[1]), wz = (float)(0.5 * g.ih2[2]);
+  const double wx = 0.5 * g.ih2[0], wy = 0.5 * g.ih2[1], wz = 0.5 * g.ih2[2];
   const int s0 = half * NP;
   if (r < npts) {
     int lx, ly, lz;
@@ -42,17 +49,30 @@ k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const Tim
     sXYZ[w][s0 + r] = lx | (ly << 8) | (lz << 16);
     if (FINE) {
       const int px = o[0] + lx, py = o[1] + ly, pz = o[2] + lz;
-      sD[w][s0 + r] = (float)(g.dsum + g.V0[(pz * g.n[1] + py) * g.n[0] + px]);
+      sD[w][s0 + r] = g.dsum + g.V0[(pz * g.n[1] + py) * g.n[0] + px];
       sX[w][s0 + r] = (float)fine_x(g, px, py, pz);
       const int cx = (px > 0 ? 1 : 0) + (px + 1 < g.n[0] ? 1 : 0), cy = (py > 0 ? 1 : 0) + (py + 1 < g.n[1] ? 1 : 0),
                 cz = (pz > 0 ? 1 : 0) + (pz + 1 < g.n[2] ? 1 : 0);
-      sN[w][s0 + r] = wx * wx * (float)cx + wy * wy * (float)cy + wz * wz * (float)cz;
+      sN[w][s0 + r] = wx * wx * cx + wy * wy * cy + wz * wz * cz;
     }
   }
   __syncthreads();
   for (int i = tid; i < KK; i += blockDim.x) {
     sPd[i] = sP[KK + i] - sP[3 * KK + i];
     sPd[KK + i] = sP[2 * KK + i] - sP[6 * KK + i];
+  }
+  if (FINE) {
+    // once per pair over the matrix's lanes: the FP64 pipe takes a warp's instruction 16 cycles, whoever of it is active
+    for (int p = r; p < npts * (npts + 1) / 2; p += NP) {
+      int a = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
+      while (a * (a + 1) / 2 > p) --a;
+      while ((a + 1) * (a + 2) / 2 <= p) ++a;
+      const int q = p - a * (a + 1) / 2, xa = sXYZ[w][s0 + a], xq = sXYZ[w][s0 + q];
+      double H, H2;
+      wide_h_h2<double>((xq & 255) - (xa & 255), ((xq >> 8) & 255) - ((xa >> 8) & 255), (xq >> 16) - (xa >> 16),
+                        sD[w][s0 + a], sD[w][s0 + q], sN[w][s0 + a], wx, wy, wz, H, H2);
+      sHH[w][half * NPAIR + p] = make_float2((float)H, (float)H2);
+    }
   }
   __syncthreads();
   // row r = (point i, time function m)
@@ -64,13 +84,11 @@ k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const Tim
   if (row_in) {
     const int xi = sXYZ[w][s0 + i];
     const int ix = xi & 255, iy = (xi >> 8) & 255, iz = xi >> 16;
-    float Di = 0.f, Xi = 0.f, Ni = 0.f;
+    float Xi = 0.f;
     const float* sg = nullptr;
     const int nbox = box5_count(L.dim);
     if (FINE) {
-      Di = sD[w][s0 + i];
       Xi = sX[w][s0 + i];
-      Ni = sN[w][s0 + i];
     } else {
       sg = sigma + sigma_offset(((o[2] + iz) * L.n[1] + (o[1] + iy)) * L.n[0] + (o[0] + ix), 0, 0, nbox);
     }
@@ -80,9 +98,8 @@ k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const Tim
       const int xj = sXYZ[w][s0 + j];
       const int dx = (xj & 255) - ix, dy = ((xj >> 8) & 255) - iy, dz = (xj >> 16) - iz;
       if (FINE) {
-        float H, H2;
-        wide_h_h2<float>(dx, dy, dz, Di, sD[w][s0 + j], Ni, wx, wy, wz, H, H2);
-        const float Xj = sX[w][s0 + j];
+        const float2 hh = sHH[w][half * NPAIR + i * (i + 1) / 2 + j];
+        const float H = hh.x, H2 = hh.y, Xj = sX[w][s0 + j];
 #pragma unroll
         for (int n = 0; n < K; ++n) {
           const int mn = m * K + n;
