@@ -21,6 +21,7 @@ from __future__ import annotations
 
 import argparse
 import dataclasses
+import itertools
 import json
 import os
 import statistics
@@ -299,6 +300,53 @@ def dominant_roofline(prof, w, precision, ms_total, traffic_ok, peaks=None):
             "algorithmic_flops": flops, "traffic_note": tnote, "peak_note": peak_note, "kernel_ms": kms}
 
 
+def factor_reach(w):
+    """Largest distance, in a subvolume's x-fastest point order, of two points that its local matrix couples: edge
+    neighbours in the square form, points at most two grid steps apart in the least-squares one."""
+    steps = 1 if getattr(w, "local_form", "lsq") == "square" else 2
+    span = [min(w.sub[a] - 1, steps) if a < w.dim else 0 for a in range(3)]
+    return max(dx + w.sub[0] * dy + w.sub[0] * w.sub[1] * dz
+               for dz in range(-span[2], span[2] + 1) for dy in range(-span[1], span[1] + 1)
+               for dx in range(-span[0], span[0] + 1) if abs(dx) + abs(dy) + abs(dz) <= steps)
+
+
+def envelope_flops(n, K, reach, square):
+    """Real flops (8 per complex multiply-add) of one factorisation of an n-unknown subvolume and of its two triangular
+    solves, counted inside the factor's envelope: an entry of column j is at most `reach` points below point
+    j // K.  Dense local algebra (4/3 n^3, LU 8/3 n^3, 8 n^2) up to lower orders where the reach covers the
+    subvolume.  The solves of the square form run over the whole LU."""
+    def last(i):
+        return min(n - 1, (i // K + reach + 1) * K - 1)
+
+    below = [last(j) - j for j in range(n)]
+    if square:   # the pivot row, one of the rows down to last(j), reaches the last column such a row couples to
+        return sum(8.0 * m * (last(last(j)) - j + 1) for j, m in enumerate(below)), 8.0 * n * n
+    return sum(4.0 * m * (m + 1) for m in below), sum(16.0 * m + 8.0 for m in below)
+
+
+def envelope_roofline(roofline, w, precision):
+    """A dominant_roofline whose rate counts the flops inside the envelope of the FP64 factors of at most 128 unknowns.
+    The library's counters hold dense local algebra there, while the kernels leave out the exact zeros outside
+    the envelope, so a rate formed from the counters is not one of the pipe (wider factors: the counters hold
+    the blocks of the band)."""
+    pts = int(np.prod([w.sub[a] for a in range(w.dim)]))
+    if roofline["bound"] != "alu" or precision != 0 or pts * w.nt > 128:
+        return roofline
+    square, reach, which = getattr(w, "local_form", "lsq") == "square", factor_reach(w), "sweep" in roofline["kernel"]
+    inside = dense = 0.0
+    for ext in itertools.product(*[[(min(w.sub[a], w.n[a]), w.n[a] // w.sub[a]), (w.n[a] % w.sub[a], 1)]
+                                   for a in range(w.dim)]):
+        n = int(np.prod([e for e, _ in ext])) * w.nt
+        count = int(np.prod([c for _, c in ext]))
+        if n and count:
+            inside += count * envelope_flops(n, w.nt, reach, square)[which]
+            dense += count * envelope_flops(n, w.nt, n, square)[which]
+    ratio = inside / dense
+    return dict(roofline, achieved=round(roofline["achieved"] * ratio, 4), frac=round(roofline["frac"] * ratio, 4),
+                algorithmic_flops=roofline["algorithmic_flops"] * ratio,
+                flops_note=f"inside the factor's envelope, {ratio:.3f} of dense local algebra")
+
+
 def stencil_roofline(prof, precision, c64=False):
     """Finest-level action-residual stencil against HBM: algorithmic bytes / event time.  c64: the
     complex64 V-cycle residual of the mixed path (TMA-staged kernel on 2D/3D grids); else the FP64
@@ -543,7 +591,8 @@ def run_ours(args):
     e2e_value = nunk * e2e_sweeps / e2e_s * (ws if ws > 1 else 1)
     ctx.close()
 
-    roofline = dominant_roofline(prof, w, precision, ms, traffic_ok=args.workload in ("2d", "3d"), peaks=peaks)
+    roofline = envelope_roofline(dominant_roofline(prof, w, precision, ms, traffic_ok=args.workload in ("2d", "3d"),
+                                                   peaks=peaks), w, precision)
     if getattr(w, "local_form", "lsq") == "square":
         roofline["kernel"] = roofline["kernel"].replace("k_factor", "k_factor_square").replace("k_sweep_fine",
                                                                                                "k_sweep_square")
@@ -799,7 +848,8 @@ def run_3d_adjoint(args):
                       "l2": l2_note(w, precision)},
            "cycles_per_step": sum(s_[0] for s_ in stats) / args.steps,
            "backward_ms_per_step": 1e3 * el_b / args.steps, "set_hamiltonian_s": setup_s,
-           "roofline": dominant_roofline(prof, w, precision, 1e3 * el_f, traffic_ok=False),
+           "roofline": envelope_roofline(dominant_roofline(prof, w, precision, 1e3 * el_f, traffic_ok=False), w,
+                                         precision),
            "stencil_roofline": stencil_roofline(prof, precision),
            "stencil_roofline_c64": stencil_roofline(prof, precision, c64=True),
            "dipole_T": float(hd * (x * psi.abs() ** 2).sum()), "grad_norm": float(np.linalg.norm(grad)),

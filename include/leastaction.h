@@ -207,7 +207,10 @@ la_status la_time_matrices(la_ctx* ctx, double t0, double* out);
    (the two triangular solves; the residual stencil is not counted).  Where the finest-level factor
    has 16 x 16 blocks that vanish identically (subvolumes of more than 128 unknowns: G_UU couples only
    points at most two grid steps apart, and the factor keeps that envelope), both counts cover only the
-   blocks of the band: the block-banded Cholesky and the solves over the band's blocks.  Algorithmic
+   blocks of the band: the block-banded Cholesky and the solves over the band's blocks.  For at most 128
+   unknowns they are the dense counts above also where the kernels leave out the entries outside the
+   envelope (FP64, and the square form's LU, 8/3 n^3): a rate formed from them is one of dense local
+   algebra, not of the arithmetic pipe.  Algorithmic
    bytes of the residual stencil: c in, r out, f in where present (K complex each per point) and V0 in. */
 typedef struct {
   long long launches;     /* kernels launched by the library since enabling */
