@@ -1105,15 +1105,6 @@ __global__ void k_c128_to_c64(long long n, const double2* __restrict__ x, float2
 void launch_axpy_c64_to_c128(long long n, const float2* x, double2* y, cudaStream_t s) {
   k_axpy_c64_to_c128<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, x, y);
 }
-__global__ void k_scale_c128(long long n, double a, const double2* __restrict__ x, double2* __restrict__ y) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double2 v = x[i];
-  y[i] = make_double2(a * v.x, a * v.y);
-}
-void launch_scale_c128(long long n, double a, const double2* x, double2* y, cudaStream_t s) {
-  k_scale_c128<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, a, x, y);
-}
 // Trial coefficients c = a0 h0 + a1 h1 + a2 h2 (h1, h2 nullable), the extrapolation of the last
 // converged coefficient vectors h0 (newest), h1, h2 of a propagation.
 __global__ void k_trial(long long n, double a0, double a1, double a2, const double2* __restrict__ h0,

@@ -2744,7 +2744,7 @@ template <typename R, int NPAD>
 __global__ void __launch_bounds__(kSweepThreads)
 k_sweep_coarse(LevelGeom L, const R* __restrict__ sigma, const TimeMats* __restrict__ tm,
                const typename C2<R>::T* gvec, typename C2<R>::T* ev,
-               const typename C2<R>::T* __restrict__ factors, int colour, int* status) {
+               const typename C2<R>::T* __restrict__ factors, int colour) {
   typedef typename C2<R>::T CT;
   extern __shared__ __align__(16) unsigned char smem[];
   overlap_trigger();
@@ -3005,7 +3005,7 @@ cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeM
 template <typename R, int NPAD>
 cudaError_t launch_sweep_coarse_n(const LevelGeom& L, const R* sigma, const TimeMats* tm, int K,
                                   const typename C2<R>::T* gvec, typename C2<R>::T* e,
-                                  const typename C2<R>::T* factors, int colour, int* status, cudaStream_t s) {
+                                  const typename C2<R>::T* factors, int colour, cudaStream_t s) {
   const int nblocks = colour_count(L, colour);
   if (nblocks == 0) return cudaSuccess;
   const size_t smem = sweep_coarse_smem(L, K, sizeof(R), sizeof(typename C2<R>::T));
@@ -3017,7 +3017,8 @@ cudaError_t launch_sweep_coarse_n(const LevelGeom& L, const R* sigma, const Time
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  return launch_overlapped(L.overlap && sizeof(R) == 4, kern, nblocks, kSweepThreads, smem, s, L, sigma, tm, gvec, e, factors, colour, status);
+  return launch_overlapped(L.overlap && sizeof(R) == 4, kern, nblocks, kSweepThreads, smem, s, L, sigma, tm, gvec, e,
+                           factors, colour);
 }
 
 template <typename R>

@@ -34,8 +34,8 @@ cudaError_t launch_sweep_fine<float>(const LevelGeom& L, const FineOp& g, const 
 template <>
 cudaError_t launch_sweep_coarse<float>(const LevelGeom& L, const float* sigma, const TimeMats* tm, int K,
                                         const float2* gvec, float2* e, const float2* factors, int colour,
-                                        int* status, cudaStream_t s) {
-#define LA_CALL(N) launch_sweep_coarse_n<float, N>(L, sigma, tm, K, gvec, e, factors, colour, status, s)
+                                        cudaStream_t s) {
+#define LA_CALL(N) launch_sweep_coarse_n<float, N>(L, sigma, tm, K, gvec, e, factors, colour, s)
   LA_NPAD_DISPATCH(L.npad, LA_CALL)
 #undef LA_CALL
 }

@@ -24,8 +24,8 @@ cudaError_t launch_sweep_fine<double>(const LevelGeom& L, const FineOp& g, const
 template <>
 cudaError_t launch_sweep_coarse<double>(const LevelGeom& L, const double* sigma, const TimeMats* tm, int K,
                                         const double2* gvec, double2* e, const double2* factors, int colour,
-                                        int* status, cudaStream_t s) {
-#define LA_CALL(N) launch_sweep_coarse_n<double, N>(L, sigma, tm, K, gvec, e, factors, colour, status, s)
+                                        cudaStream_t s) {
+#define LA_CALL(N) launch_sweep_coarse_n<double, N>(L, sigma, tm, K, gvec, e, factors, colour, s)
   LA_NPAD_DISPATCH(L.npad, LA_CALL)
 #undef LA_CALL
 }

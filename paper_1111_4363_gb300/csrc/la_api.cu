@@ -692,7 +692,7 @@ static la_status sweep_level(la_ctx* c, int l, int nsweeps) {
                                  c->stream);
       else
         e = launch_sweep_coarse<R>(c->geo[l], sigma_of<R>(c, l), c->d_tm, c->K, (const CT*)c->d_g[l], (CT*)c->d_e[l],
-                                   (const CT*)c->d_fac[l], col, c->d_status, c->stream);
+                                   (const CT*)c->d_fac[l], col, c->stream);
       if (e != cudaSuccess) return fail(c, LA_ECUDA, "sweep level %d colour %d: %s", l, col, cudaGetErrorString(e));
     }
     // inside a capture the records are graph nodes (external), not capture-internal joins

@@ -405,7 +405,6 @@ void launch_advance(int np, const TimeMats* tm, const double2* c, double2* psi, 
 void launch_axpy_c64_to_c128(long long n, const float2* x, double2* y, cudaStream_t s);
 void launch_c128_to_c64(long long n, const double2* x, float2* y, cudaStream_t s);
 void launch_f64_to_f32(long long n, const double* x, float* y, cudaStream_t s);
-void launch_scale_c128(long long n, double a, const double2* x, double2* y, cudaStream_t s);
 void launch_trial(long long n, const double* a, const double2* h0, const double2* h1, const double2* h2, double2* c,
                   cudaStream_t s);
 // device-side relaxation loop of one context (la_step_batch): state and per-step record
@@ -456,7 +455,7 @@ cudaError_t launch_sweep_square(const LevelGeom& L, const FineOp& g, const TimeM
 template <typename R>
 cudaError_t launch_sweep_coarse(const LevelGeom& L, const R* sigma, const TimeMats* tm, int K,
                                 const typename C2<R>::T* gvec, typename C2<R>::T* e,
-                                const typename C2<R>::T* factors, int colour, int* status, cudaStream_t s);
+                                const typename C2<R>::T* factors, int colour, cudaStream_t s);
 
 
 // ------------------------------------------------------------------ overlapped launches
