@@ -965,7 +965,8 @@ void launch_restrict(const LevelGeom& F, const LevelGeom& C, int K, const typena
       cudaFuncSetAttribute(k_restrict_tile<CT, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); \
       attr = true;                                                                                         \
     }                                                                                                      \
-    launch_overlapped(F.overlap && sizeof(R) == 4, k_restrict_tile<CT, KK>, grid, 256, smem, s, F, C, sf, gc, ec); \
+    launch_overlapped(F.overlap && sizeof(R) == 4, kOverlapMax, k_restrict_tile<CT, KK>, grid, 256, smem, s, F, C, sf, gc, \
+                      ec);                                                                                 \
   } while (0)
     switch (K) {
       case 1: LA_CALL(1); break;
@@ -988,8 +989,8 @@ template <typename R>
 void launch_prolong_add(const LevelGeom& F, const LevelGeom& C, int K, const typename C2<R>::T* ec,
                         typename C2<R>::T* ef, cudaStream_t s) {
 #define LA_CALL(KK) \
-  launch_overlapped(F.overlap && sizeof(R) == 4, k_prolong_add<typename C2<R>::T, KK>, (F.np + 127) / 128, 128, 0, s, F, C, \
-                    ec, ef)
+  launch_overlapped(F.overlap && sizeof(R) == 4, kOverlapMax, k_prolong_add<typename C2<R>::T, KK>,       \
+                    (F.np + 127) / 128, 128, 0, s, F, C, ec, ef)
   LA_K_DISPATCH(K, LA_CALL)
 #undef LA_CALL
 }

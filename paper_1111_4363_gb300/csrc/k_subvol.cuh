@@ -2946,7 +2946,8 @@ cudaError_t launch_sweep_super(const LevelGeom& L, const FineOp& g, const TimeMa
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   const FastDiv dn0 = make_fastdiv((L.nb[0] - (colour & 1) + 1) / 2),
                 dn1 = make_fastdiv((L.nb[1] - ((colour >> 1) & 1) + 1) / 2);
-  return launch_overlapped(L.overlap, kern, nblocks, kSuperThreads, smem, s, L, g, tm, f, yx, c, factors, colour, dn0, dn1);
+  return launch_overlapped(L.overlap, kOverlapSweep, kern, nblocks, kSuperThreads, smem, s, L, g, tm, f, yx, c, factors,
+                           colour, dn0, dn1);
 }
 template <int NPAD, int K>
 cudaError_t launch_sweep_small(const LevelGeom& L, const FineOp& g, const TimeMats* tm, const float2* f,
@@ -2963,8 +2964,8 @@ cudaError_t launch_sweep_small(const LevelGeom& L, const FineOp& g, const TimeMa
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   const FastDiv dn0 = make_fastdiv((L.nb[0] - (colour & 1) + 1) / 2),
                 dn1 = make_fastdiv((L.nb[1] - ((colour >> 1) & 1) + 1) / 2);
-  return launch_overlapped(L.overlap, kern, (nblocks + kSmallSweepWarps - 1) / kSmallSweepWarps, 32 * kSmallSweepWarps,
-                           smem, s, L, g, tm, f, yx, c, factors, colour, dn0, dn1, nblocks);
+  return launch_overlapped(L.overlap, kOverlapMax, kern, (nblocks + kSmallSweepWarps - 1) / kSmallSweepWarps,
+                           32 * kSmallSweepWarps, smem, s, L, g, tm, f, yx, c, factors, colour, dn0, dn1, nblocks);
 }
 template <typename R, int NPAD>
 cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeMats* tm, int K,
@@ -2999,7 +3000,8 @@ cudaError_t launch_sweep_fine_n(const LevelGeom& L, const FineOp& g, const TimeM
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  return launch_overlapped(L.overlap && sizeof(R) == 4, kern, nblocks, kSweepThreads, smem, s, L, g, tm, f, yx, c, factors, colour);
+  return launch_overlapped(L.overlap && sizeof(R) == 4, kOverlapSweep, kern, nblocks, kSweepThreads, smem, s, L, g, tm, f,
+                           yx, c, factors, colour);
   }
 }
 template <typename R, int NPAD>
@@ -3017,8 +3019,8 @@ cudaError_t launch_sweep_coarse_n(const LevelGeom& L, const R* sigma, const Time
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  return launch_overlapped(L.overlap && sizeof(R) == 4, kern, nblocks, kSweepThreads, smem, s, L, sigma, tm, gvec, e,
-                           factors, colour);
+  return launch_overlapped(L.overlap && sizeof(R) == 4, kOverlapMax, kern, nblocks, kSweepThreads, smem, s, L, sigma, tm,
+                           gvec, e, factors, colour);
 }
 
 template <typename R>
@@ -3034,7 +3036,8 @@ cudaError_t launch_gresid_tiles_r(const LevelGeom& L, const R* sigma, const Time
     attr_set = true;
   }
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  return launch_overlapped(L.overlap && sizeof(R) == 4, kern, L.nsub, kSweepThreads, smem, s, L, sigma, tm, gvec, e, out, L.npad);
+  return launch_overlapped(L.overlap && sizeof(R) == 4, kOverlapMax, kern, L.nsub, kSweepThreads, smem, s, L, sigma, tm,
+                           gvec, e, out, L.npad);
 }
 
 // finest-level sweeps and factorisations also take the wide sizes

@@ -33,6 +33,8 @@
 
 namespace la {
 
+constexpr int kSms = 152;  // multiprocessors of a GB300: unit of the launch rules that depend on the CTAs per SM
+
 // Per-context time-basis data, in device global memory.  Static parts are written by the
 // host at init; Eb, Eb0 and Theta are rewritten by k_time_matrices for every step.
 struct TimeMats {
@@ -466,18 +468,25 @@ cudaError_t launch_sweep_coarse(const LevelGeom& L, const R* sigma, const TimeMa
 // matrices and the potential are final before a chain begins.  The pointers to what a predecessor writes carry no
 // __restrict__: with const it promises data that nothing changes while the kernel runs, which the compiler may turn
 // into non-coherent loads (ld.global.nc) that overlap_wait does not order; the coherent loads cost nothing measurable
-// here.  It hides the launch latency and the constant
-// loads of the many short kernels of a complex64 V-cycle.  Launches of more than kOverlapMax CTAs, about two per
-// SM, go out in the ordinary way: they are not bound by their launch, and early successors only took their
-// issue slots (3D 128^3 mixed: 124.2 ms without, 127.5 ms with every launch overlapped).  So do FP64 launches, which
-// the early successors' FP64 conversions slow down (22x12x32 points, 4x4x4 x 4: 20.3 ms without, 25.2 ms with;
-// 256^2 with every sweep: 43.2 and 48.3 ms).
-constexpr unsigned kOverlapMax = 304;
+// here.  It hides the launch latency and the constant loads of the many short kernels of a complex64 V-cycle.
+// A launch of more than `max_ctas` CTAs goes out in the ordinary way: it is not bound by its latency, and early
+// successors take its issue slots (3D 128^3 mixed: 124.2 ms with these lines, 127.5 ms with every launch overlapped).
+// Where the lines lie, one step of 3 cycles in mixed precision, K = 4 unless given, plain / overlapped:
+// - kOverlapSweep, one CTA per SM, for finest sweeps of more than 32 unknowns, whose CTAs work longest.  3D 4x4x4 on
+//   32^3 (64 CTAs a colour) 2.76 / 2.55 ms, 40^3 (125) 3.26 / 3.19 ms, 48^3 (216) 3.83 / 4.13 ms; 4x4x2 on 36^3
+//   (144 to 225) 2.58 / 2.73 ms, 40^3 (250) 2.88 / 3.11 ms; 2D 8x8 on 256^2 (256) 1.53 / 1.60 ms.
+// - kOverlapMax, two per SM, for the other kernels.  Coarse sweeps: 2D 4x4 on 128^2 (256 CTAs) 753 / 724 us, 192^2 (576)
+//   930 / 907 us, but with the 576 of the residual of 4x4 x 6 on 96^2 755 / 790 us.  Small finest sweeps: 2D 2x2 on
+//   128^2 (256 CTAs) 402 / 388 us, 3D 2x2x2 on 40^3 (250) 1.55 / 1.62 ms.
+// FP64 launches are all plain: the early successors' FP64 conversions slow them down (22x12x32 points, 4x4x4 x 4:
+// 20.3 ms plain, 25.2 ms overlapped; 256^2 with every sweep: 43.2 and 48.3 ms).
+constexpr unsigned kOverlapSweep = kSms;
+constexpr unsigned kOverlapMax = 2 * kSms;
 __device__ __forceinline__ void overlap_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void overlap_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename... P, typename... A>
-inline cudaError_t launch_overlapped(bool overlap, void (*kern)(P...), dim3 grid, int threads, size_t smem,
-                                     cudaStream_t s, A... args) {
+inline cudaError_t launch_overlapped(bool overlap, unsigned max_ctas, void (*kern)(P...), dim3 grid, int threads,
+                                     size_t smem, cudaStream_t s, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
@@ -487,7 +496,7 @@ inline cudaError_t launch_overlapped(bool overlap, void (*kern)(P...), dim3 grid
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
-  cfg.numAttrs = overlap && grid.x * grid.y * grid.z <= kOverlapMax ? 1 : 0;
+  cfg.numAttrs = overlap && grid.x * grid.y * grid.z <= max_ctas ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
