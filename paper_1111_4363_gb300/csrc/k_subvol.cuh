@@ -1580,8 +1580,6 @@ __device__ __forceinline__ CPair<double2> load_colpair<double2>(const double2* b
   return p;
 }
 
-constexpr unsigned kPipeBoundCtas = 304;
-
 template <typename CT>
 __device__ __forceinline__ CT reduce_xor(CT v, int m) {
   v.x += __shfl_xor_sync(0xffffffffu, v.x, m);
@@ -1611,8 +1609,17 @@ __device__ __forceinline__ void load_fwd_band(CPair<CT>& p, const CT* a, bool in
   else p.load_zero();
 }
 
-// SKIP leaves the products of zero blocks out: worth it where the FP64 pipe is the bound; its branches keep loads from
-// being issued ahead, which costs more where a few CTAs wait on latency.
+// Whether an FP64 solve leaves the products of zero blocks out (SKIP).  Worth it where the FP64 pipe is the bound and
+// enough products go; its branches keep loads from being issued ahead, which costs more where a CTA has an SM for
+// itself, and is all there is to it in a wide band.  One colour, every product / without the zero blocks':
+//   band 8 of 16 (4x4x4 x 4): 150 CTAs 147 / 168 us, 160 215 / 204 us, 294 220 / 217 us, 343 318 / 280 us, 512 467 / 449 us;
+//   band 4 (8x8 x 4): 160 CTAs 199 / 142 us, 400 295 / 197 us (100: 128 / 114 us, but 16x4 x 4 131 / 147 us);
+//   band 7 of 12 (4x4x4 x 3): 160 CTAs 136 / 135 us, 294 140 / 142 us, 343 200 / 186 us;
+//   band 11 of 16 (4x4x3 x 5): 160 CTAs 221 / 232 us, 343 414 / 456 us; band 15 (8x4x2 x 4): 343 CTAs 409 / 471 us.
+template <int NB>
+__device__ __forceinline__ bool skip_zero_blocks(int band, unsigned ctas) {
+  return 2 * band <= NB ? ctas > kSms : 3 * band <= 2 * NB && ctas > 2 * kSms;
+}
 template <typename CT, int NPAD, bool SKIP>
 __device__ __forceinline__ void subvol_solve_wide(const CT* __restrict__ F, int band, CT* rhs, CT* y, CT* tvec,
                                                   CT* part) {
@@ -2167,10 +2174,8 @@ k_sweep_fine(LevelGeom L, FineOp g, const TimeMats* __restrict__ tm, const typen
     sRhs[t] = out;
   }
   __syncthreads();
-  // FP64 from about two CTAs per SM on is bound by its pipe (4x4x4 x 4, a colour of 512 subvolumes: 488 us with every
-  // product, 445 us without; of 12: 149 and 171 us)
   if (use_wide_solve<R, NPAD>()) {
-    if (sizeof(R) == 8 && gridDim.x > kPipeBoundCtas)
+    if (sizeof(R) == 8 && skip_zero_blocks<NPAD / LA_BLK>(L.band, gridDim.x))
       subvol_solve_wide<CT, NPAD, true>(factors + (size_t)b * L.fsize, L.band, sRhs, sY, sT, sRed);
     else
       subvol_solve_wide<CT, NPAD, false>(factors + (size_t)b * L.fsize, L.band, sRhs, sY, sT, sRed);
