@@ -1470,13 +1470,13 @@ __device__ __forceinline__ CT reduce4(CT v) {
   return v;
 }
 
-template <typename CT, int NPAD>
-__device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __restrict__ F, CT* rhs, CT* y, CT* tvec) {
+template <typename CT, int NPAD, bool ENV>
+__device__ __forceinline__ void subvol_solve_t(const LevelGeom& L, const CT* __restrict__ F, CT* rhs, CT* y, CT* tvec) {
   constexpr int NB = NPAD / LA_BLK;
   const int tid = threadIdx.x;
   if (tid >= 64) return;
   const int r = tid >> 2, l = tid & 3, r0 = r & 8;   // r0: the warp's first row of a block
-  // A factor has no entry further than L.reach points from its diagonal: a warp's eight rows start at the first
+  // ENV: a factor has no entry further than L.reach points from its diagonal: a warp's eight rows start at the first
   // column its first row couples to and (backward) its eight columns end at the last row its last column
   // couples to, in steps of the four columns that the lanes of a row take together.  Predicated lanes would
   // still occupy the FP64 pipe, so the bounds are the warp's.  The block that a bound cuts stands outside the loop
@@ -1485,9 +1485,9 @@ __device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __res
   // forward: y_I = inv(L_II) (rhs_I - sum_{J<I} L_IJ y_J)
   for (int I = 0; I < NB; ++I) {
     const CT* rowblk = F + (size_t)(I * (I + 1) / 2) * 256;
-    const int c0 = max((fdiv(I * LA_BLK + r0, L.fd_K) - L.reach) * K, 0) >> 2;   // first group of four columns
+    const int c0 = ENV ? max((fdiv(I * LA_BLK + r0, L.fd_K) - L.reach) * K, 0) >> 2 : 0;   // first group of four columns
     CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
-    if ((c0 & 3) && (c0 >> 2) < I) {
+    if (ENV && (c0 & 3) && (c0 >> 2) < I) {
       const CT* blk = rowblk + (c0 >> 2) * 256 + r * LA_BLK;
       const CT* yy = y + (c0 >> 2) * LA_BLK;
       if ((c0 & 3) <= 1) cfma(acc1, blk[l + 4], yy[l + 4]);
@@ -1510,7 +1510,7 @@ __device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __res
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int c = l + 4 * k;
-      if (4 * k > r0 + 7) break;
+      if (ENV && 4 * k > r0 + 7) break;
       if (c <= r) cfma(acc0, dblk[c], tvec[c]);
     }
     acc = reduce4(acc0);
@@ -1519,7 +1519,8 @@ __device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __res
   }
   // backward: x_I = inv(L_II)^dagger (y_I - sum_{J>I} L_JI^dagger x_J), x stored in rhs
   for (int I = NB - 1; I >= 0; --I) {
-    const int e4 = min((fdiv(I * LA_BLK + r0 + 7, L.fd_K) + L.reach + 1) * K - 1, NPAD - 1) >> 2;   // last group of rows
+    const int e4 =   // last group of rows
+        (ENV ? min((fdiv(I * LA_BLK + r0 + 7, L.fd_K) + L.reach + 1) * K - 1, NPAD - 1) : NPAD - 1) >> 2;
     CT acc0 = mkc<CT>(0, 0), acc1 = mkc<CT>(0, 0);
     const int Jf = (e4 + 1) >> 2, k1 = (e4 + 1) & 3;   // the first block not taken whole, its groups
     for (int J = I + 1; J < Jf; ++J) {
@@ -1530,7 +1531,7 @@ __device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __res
       cfma_conj(acc0, blk[(l + 8) * LA_BLK + r], xx[l + 8]);
       cfma_conj(acc1, blk[(l + 12) * LA_BLK + r], xx[l + 12]);
     }
-    if (k1 && Jf > I) {
+    if (ENV && k1 && Jf > I) {
       const CT* blk = F + (size_t)(Jf * (Jf + 1) / 2 + I) * 256;
       const CT* xx = rhs + Jf * LA_BLK;
       cfma_conj(acc0, blk[l * LA_BLK + r], xx[l]);
@@ -1545,13 +1546,20 @@ __device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __res
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int cc = l + 4 * k;
-      if (4 * k + 3 < r0) continue;
+      if (ENV && 4 * k + 3 < r0) continue;
       if (cc >= r) cfma_conj(acc0, dblk[cc * LA_BLK + r], tvec[cc]);
     }
     acc = reduce4(acc0);
     if (l == 0) rhs[I * LA_BLK + r] = acc;
     solve_bar();
   }
+}
+
+template <typename CT, int NPAD>
+__device__ __forceinline__ void subvol_solve(const LevelGeom& L, const CT* __restrict__ F, CT* rhs, CT* y, CT* tvec) {
+  if (solve_inside_envelope(L.reach, L.sub[0] * L.sub[1] * L.sub[2], NPAD / LA_BLK, gridDim.x, sizeof(CT) == 16))
+    subvol_solve_t<CT, NPAD, true>(L, F, rhs, y, tvec);
+  else subvol_solve_t<CT, NPAD, false>(L, F, rhs, y, tvec);
 }
 
 // Triangular solves with a wide factor (more than eight block rows) by all 128 threads of the

@@ -357,6 +357,23 @@ __host__ inline bool usable_in_place(const cudaPointerAttributes& a, int device,
   return a.type == cudaMemoryTypeDevice && a.device == device && (reinterpret_cast<uintptr_t>(p) & 31) == 0;
 }
 
+// Whether the two-warp triangular solves stay inside the envelope (subvol_solve, at most 128 unknowns): subvolumes of
+// npts points, factors of nb block rows, `ctas` subvolumes of a colour.  The same sums either way; the bounds cost
+// instructions in every step of the chain, and a warp's products go in groups of four columns.
+// - FP64 on up to three CTAs per SM waits on the chain: worth it where the envelope leaves out two block columns' worth
+//   of a full row.  Time with the bounds over time without, a colour of about 12 CTAs: 5x5 x 3 (reach 10 of 24, 6 block
+//   rows) 0.86, 4x4 x 6 (8 of 15, 6) 1.00, 8x4 x 2 (16 of 31, 4) 1.00, 4x4 x 2 (2 rows) 1.09; of 275: 2x2x2 x 3 (6 of 7) 1.06.
+// - FP64 on more CTAs is bound by its pipe: worth it up to three quarters of the points.  500 CTAs: 4x4 x 6 0.94, 4x2 x 4
+//   (5 of 7) 0.99, 3x3 x 2 (6 of 8) 0.97; 1000: 4x2x2 x 8 (12 of 15) 1.04.  One block row: 1.01 to 1.02.
+// - complex64 (Galerkin levels) always waits on the chain.  Whole steps: 1D 16 x 8 (reach 2 of 15) 0.81, 8 x 8 (2 of 7)
+//   0.99; 2D 8x4 x 4 (18 of 31) 1.14, 4x4 x 4, 6, 8 (10 of 15) 1.05, 1.15, 1.17; 3D 4x2x2 x 4, 8 (14 of 15) 1.02, 1.16.
+__host__ __device__ inline bool solve_inside_envelope(int reach, int npts, int nb, unsigned ctas, bool fp64) {
+  const int all = npts - 1;   // the reach that covers the subvolume
+  if (nb < 2) return false;
+  if (!fp64) return 3 * reach <= all;
+  return ctas > 3 * kSms ? 4 * reach <= 3 * all : (all - reach) * nb >= 2 * all;
+}
+
 template <typename R> struct C2;
 template <> struct C2<double> { typedef double2 T; };
 template <> struct C2<float> { typedef float2 T; };
