@@ -61,6 +61,12 @@ __device__ __forceinline__ double gal_fine_1d(const FineOp& g, int type, int ax,
   }
 }
 
+// Whether the finest 1D operator of a type has an entry at distance d.
+__device__ __forceinline__ bool gal_nonzero(int type, int d) {
+  if (type == kGalT || type == kGalTX) return d == 1 || d == -1;
+  return d == 0 || (type == kGalT2 && (d == 2 || d == -2));
+}
+
 // One thread per table entry; nf, nc the points per axis of the finer level and of this one.
 template <bool FROM_FINE>
 __global__ void k_gal_1d(FineOp g, int3 nf3, int3 nc3, const double* __restrict__ tf, double* __restrict__ tc) {
@@ -87,6 +93,8 @@ __global__ void k_gal_1d(FineOp g, int3 nf3, int3 nc3, const double* __restrict_
       for (int j = 0; j < 4; ++j) {
         const int b = 2 * K - 1 + j;
         if (b < 0 || b >= nfa || b - a > 2 || a - b > 2) continue;
+        // most of the pairs, which cost the most on a long 1D grid: 343 -> 217 us a call on 100,352 points, two levels
+        if (FROM_FINE && !gal_nonzero(type, b - a)) continue;
         s += gal_w(i) * gal_w(j) * (FROM_FINE ? gal_fine_1d(g, type, ax, a, b) : f[5LL * a + (b - a + 2)]);
       }
     }
@@ -132,8 +140,8 @@ __global__ void __launch_bounds__(128) k_gal_sep(int lax, LevelGeom C, const dou
 // z is contracted first, then y, for the fine x of the chunk all at once; the last step sums over x and
 // adds the products of the 1D tables: about 1000 + 125 x 40 FP64 operations per coarse point.  The
 // same sums taken per entry over the 4^3 points took 21.5 ms on 96^3, bound by FP64 issue with most lanes idle.
-constexpr int kGalChunk = 8, kGalThreads = 128;
-constexpr int kGalFx = 2 * kGalChunk + 4;   // fine x of a chunk
+// In 1D a point has 5 entries only, so a CTA takes 64 points: 343 us instead of 349 us a call on 100,352 points.
+constexpr int kGalChunk = 8, kGalChunk1D = 64, kGalThreads = 128;
 
 // W and G of coarse point J and offset o on one axis at fine point c (zero where c or J + o is outside).
 __device__ __forceinline__ void gal_wg(int J, int o, int c, int nf, int nc, double t, double& W, double& G) {
@@ -151,17 +159,18 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_first(FineOp g, LevelGeom C
   constexpr int OY = DIM > 1 ? 5 : 1, OZ = DIM > 2 ? 5 : 1, NBOX = 5 * OY * OZ;
   constexpr int RY = DIM > 1 ? 6 : 1, RZ = DIM > 2 ? 6 : 1;   // fine rows per axis
   constexpr int CY = DIM > 1 ? 2 : 0, CZ = DIM > 2 ? 2 : 0;   // index of offset 0
-  __shared__ double F[3][kGalFx][RZ][RY];        // D, D^2, D x
-  __shared__ double ZW[3][kGalFx][RY][OZ];       // contracted over z with W
-  __shared__ double ZG[kGalFx][RY][OZ];          // D contracted with G
-  __shared__ double YW[3][kGalFx][OZ][OY];       // then over y with W
-  __shared__ double YG[kGalFx][OZ][OY];          // G W + W G of D
-  __shared__ double wx[kGalChunk][5][6], gx[kGalChunk][5][6], wy[OY][RY], gy[OY][RY], wz[OZ][RZ], gz[OZ][RZ];
+  constexpr int NJ = DIM > 1 ? kGalChunk : kGalChunk1D, NX = 2 * NJ + 4;   // coarse points and fine x of a chunk
+  __shared__ double F[3][NX][RZ][RY];        // D, D^2, D x
+  __shared__ double ZW[3][NX][RY][OZ];       // contracted over z with W
+  __shared__ double ZG[NX][RY][OZ];          // D contracted with G
+  __shared__ double YW[3][NX][OZ][OY];       // then over y with W
+  __shared__ double YG[NX][OZ][OY];          // G W + W G of D
+  __shared__ double wx[NJ][5][6], gx[NJ][5][6], wy[OY][RY], gy[OY][RY], wz[OZ][RZ], gz[OZ][RZ];
   const int tid = threadIdx.x;
-  const int nchunk = (C.n[0] + kGalChunk - 1) / kGalChunk;
+  const int nchunk = (C.n[0] + NJ - 1) / NJ;
   const int ch = blockIdx.x % nchunk, row = blockIdx.x / nchunk;
   const int jy = row % C.n[1], jz = row / C.n[1];
-  const int J0 = ch * kGalChunk, nj = min(kGalChunk, C.n[0] - J0);
+  const int J0 = ch * NJ, nj = min(NJ, C.n[0] - J0);
   const int fx0 = 2 * J0 - 2, fy0 = DIM > 1 ? 2 * jy - 2 : 0, fz0 = DIM > 2 ? 2 * jz - 2 : 0;
   for (int t = tid; t < nj * 30; t += kGalThreads) {
     const int j = t / 30, o = (t / 6) % 5, i = t % 6;
@@ -181,8 +190,8 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_first(FineOp g, LevelGeom C
     wz[0][0] = 1.0;
     gz[0][0] = 0.0;
   }
-  for (int t = tid; t < RZ * RY * kGalFx; t += kGalThreads) {
-    const int lx = t % kGalFx, ly = (t / kGalFx) % RY, lz = t / (kGalFx * RY);
+  for (int t = tid; t < RZ * RY * NX; t += kGalThreads) {
+    const int lx = t % NX, ly = (t / NX) % RY, lz = t / (NX * RY);
     const int x = fx0 + lx, y = fy0 + ly, z = fz0 + lz;
     double d = 0.0, xl = 0.0;
     if (fine_in(g, x, y, z)) {
@@ -194,7 +203,7 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_first(FineOp g, LevelGeom C
     F[2][lx][lz][ly] = d * xl;
   }
   __syncthreads();
-  for (int t = tid; t < kGalFx * RY * OZ; t += kGalThreads) {
+  for (int t = tid; t < NX * RY * OZ; t += kGalThreads) {
     const int oz = t % OZ, ly = (t / OZ) % RY, lx = t / (OZ * RY);
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, ag = 0.0;
 #pragma unroll
@@ -211,7 +220,7 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_first(FineOp g, LevelGeom C
     ZG[lx][ly][oz] = ag;
   }
   __syncthreads();
-  for (int t = tid; t < kGalFx * OZ * OY; t += kGalThreads) {
+  for (int t = tid; t < NX * OZ * OY; t += kGalThreads) {
     const int oy = t % OY, oz = (t / OY) % OZ, lx = t / (OY * OZ);
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, ag = 0.0;
 #pragma unroll
@@ -282,7 +291,7 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_first(FineOp g, LevelGeom C
   }
 }
 
-// Further levels, the factors (0,1), (1,1), (1,2) (and their copies (1,0) and (2,1)): one CTA per chunk of
+// Further levels in 2D and 3D, the factors (0,1), (1,1), (1,2) (and their copies (1,0) and (2,1)): one CTA per chunk of
 // kGalChunk coarse points along x of one row (Jy, Jz) and one factor.  It walks the fine points of the row;
 // the stencils of the 4 x 4 fine rows at one fine x are staged in shared memory (the next ones in flight),
 // contracted over z and y (both the rows and the offsets), and every second fine x completes a coarse
@@ -291,8 +300,8 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_first(FineOp g, LevelGeom C
 template <int DIM>
 __global__ void __launch_bounds__(kGalThreads) k_gal_contract(LevelGeom F, const double* __restrict__ sf, LevelGeom C,
                                                               double* __restrict__ sc) {
-  constexpr int OX = 5, OY = DIM > 1 ? 5 : 1, OZ = DIM > 2 ? 5 : 1, NBOX = OX * OY * OZ;
-  constexpr int AY = DIM > 1 ? 4 : 1, AZ = DIM > 2 ? 4 : 1, NROW = AY * AZ;
+  constexpr int OX = 5, OY = 5, OZ = DIM > 2 ? 5 : 1, NBOX = OX * OY * OZ;
+  constexpr int AY = 4, AZ = DIM > 2 ? 4 : 1, NROW = AY * AZ;
   __shared__ double S[2][NROW * NBOX];
   __shared__ double Z[AY * NBOX];       // [ay][oz'][oy][ox]
   __shared__ double Y[4][NBOX];         // contracted over z and y, ring over the fine x
@@ -302,7 +311,7 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_contract(LevelGeom F, const
   const int pair = blockIdx.y == 0 ? 1 : (blockIdx.y == 1 ? 4 : 5);
   const int jy = row % C.n[1], jz = row / C.n[1];
   const int J0 = ch * kGalChunk, J1 = min(J0 + kGalChunk, C.n[0]);
-  auto fine_y = [&](int i) { return DIM > 1 ? 2 * jy - 1 + i : jy; };
+  auto fine_y = [&](int i) { return 2 * jy - 1 + i; };
   auto fine_z = [&](int i) { return DIM > 2 ? 2 * jz - 1 + i : jz; };
   auto stage = [&](int ax, double* dst) {
     if (ax >= 0 && ax < F.n[0])
@@ -356,22 +365,18 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_contract(LevelGeom F, const
     if (in) {
       // y: contracted over the fine y rows
       for (int e = tid; e < NBOX; e += kGalThreads) {
-        const int ox = e % OX, oyc = (e / OX) % OY - (DIM > 1 ? 2 : 0), oz = e / (OX * OY);
+        const int ox = e % OX, oyc = (e / OX) % OY - 2, oz = e / (OX * OY);
         double v = 0.0;
-        if (DIM > 1) {
-          const int ky = jy + oyc;
-          if (ky >= 0 && ky < C.n[1])
+        const int ky = jy + oyc;
+        if (ky >= 0 && ky < C.n[1])
 #pragma unroll
-            for (int i = 0; i < AY; ++i)
+          for (int i = 0; i < AY; ++i)
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const int d = 2 * oyc + j - i, b = 2 * ky - 1 + j;
-                if (d >= -2 && d <= 2 && b >= 0 && b < F.n[1])
-                  v = fma(gal_w(i) * gal_w(j), Z[i * NBOX + (oz * OY + (d + 2)) * OX + ox], v);
-              }
-        } else {
-          v = Z[e];
-        }
+            for (int j = 0; j < 4; ++j) {
+              const int d = 2 * oyc + j - i, b = 2 * ky - 1 + j;
+              if (d >= -2 && d <= 2 && b >= 0 && b < F.n[1])
+                v = fma(gal_w(i) * gal_w(j), Z[i * NBOX + (oz * OY + (d + 2)) * OX + ox], v);
+            }
         Y[ax & 3][e] = v;
       }
     }
@@ -381,7 +386,7 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_contract(LevelGeom F, const
       const int jx = (ax - 2) >> 1;
       for (int e = tid; e < NBOX; e += kGalThreads) {
         const int ox = e % OX - 2, oyi = (e / OX) % OY, ozi = e / (OX * OY);
-        const int kx = jx + ox, ky = jy + (DIM > 1 ? oyi - 2 : 0), kz = jz + (DIM > 2 ? ozi - 2 : 0);
+        const int kx = jx + ox, ky = jy + oyi - 2, kz = jz + (DIM > 2 ? ozi - 2 : 0);
         const bool kin = kx >= 0 && kx < C.n[0] && ky >= 0 && ky < C.n[1] && kz >= 0 && kz < C.n[2];
         double v = 0.0;
         if (kin)
@@ -404,6 +409,30 @@ __global__ void __launch_bounds__(kGalThreads) k_gal_contract(LevelGeom F, const
   }
 }
 
+// The same in 1D, one thread per entry: 16 products at most, so nothing is gained by contracting (a level of 25,088
+// points adds 48 us to a call, 118 us with the walk along x).
+__global__ void __launch_bounds__(128) k_gal_line(LevelGeom F, const double* __restrict__ sf, LevelGeom C,
+                                                  double* __restrict__ sc) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 5 * C.np) return;
+  const int pair = blockIdx.y == 0 ? 1 : (blockIdx.y == 1 ? 4 : 5);
+  const int J = t / 5, e = t - 5 * J, K = J + e - 2;
+  const bool kin = K >= 0 && K < C.np;
+  double v = 0.0;
+  if (kin)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int a = 2 * J - 1 + i, b = 2 * K - 1 + j, d = b - a;
+        if (d >= -2 && d <= 2 && a >= 0 && a < F.np && b >= 0 && b < F.np)
+          v = fma(gal_w(i) * gal_w(j), sf[sigma_offset(a, pair, d + 2, 5)], v);
+      }
+  sc[sigma_offset(J, pair, e, 5)] = v;
+  if (pair == 1) sc[sigma_offset(J, 3, e, 5)] = v;
+  if (pair == 5) sc[kin ? sigma_offset(K, 7, 4 - e, 5) : sigma_offset(J, 7, e, 5)] = v;
+}
+
 void launch_galerkin(const FineOp& g, const LevelGeom* geo, int levels, double* const* sigma, double* tab0,
                      double* tab1, cudaStream_t s) {
   double* tab[2] = {tab0, tab1};
@@ -414,7 +443,8 @@ void launch_galerkin(const FineOp& g, const LevelGeom* geo, int levels, double* 
     const unsigned tb = (unsigned)((nt + 127) / 128), eb = (unsigned)((ne + 127) / 128);
     if (l == 1) {
       k_gal_1d<true><<<tb, 128, 0, s>>>(g, nf, nc, nullptr, tab[1]);
-      const unsigned grid = (unsigned)(((C.n[0] + kGalChunk - 1) / kGalChunk) * C.n[1] * C.n[2]);
+      const int nj = C.dim == 1 ? kGalChunk1D : kGalChunk;
+      const unsigned grid = (unsigned)(((C.n[0] + nj - 1) / nj) * C.n[1] * C.n[2]);
       if (C.dim == 1) k_gal_first<1><<<grid, kGalThreads, 0, s>>>(g, C, tab[1], sigma[1]);
       else if (C.dim == 2) k_gal_first<2><<<grid, kGalThreads, 0, s>>>(g, C, tab[1], sigma[1]);
       else k_gal_first<3><<<grid, kGalThreads, 0, s>>>(g, C, tab[1], sigma[1]);
@@ -422,7 +452,7 @@ void launch_galerkin(const FineOp& g, const LevelGeom* geo, int levels, double* 
       k_gal_1d<false><<<tb, 128, 0, s>>>(g, nf, nc, tab[(l - 1) & 1], tab[l & 1]);
       k_gal_sep<<<eb, 128, 0, s>>>(g.lax, C, tab[l & 1], sigma[l]);
       const dim3 grid((unsigned)(((C.n[0] + kGalChunk - 1) / kGalChunk) * C.n[1] * C.n[2]), 3);
-      if (C.dim == 1) k_gal_contract<1><<<grid, kGalThreads, 0, s>>>(F, sigma[l - 1], C, sigma[l]);
+      if (C.dim == 1) k_gal_line<<<dim3((unsigned)((5LL * C.np + 127) / 128), 3), 128, 0, s>>>(F, sigma[l - 1], C, sigma[l]);
       else if (C.dim == 2) k_gal_contract<2><<<grid, kGalThreads, 0, s>>>(F, sigma[l - 1], C, sigma[l]);
       else k_gal_contract<3><<<grid, kGalThreads, 0, s>>>(F, sigma[l - 1], C, sigma[l]);
     }
