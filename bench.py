@@ -257,14 +257,11 @@ def dominant_roofline(prof, w, precision, ms_total, traffic_ok, peaks=None):
     swp_ms_full = prof["ms_sweep"] / max(prof["n_sweep"], 1)   # one event pair per full sweep
     nsub, fbytes = finest_factor_store(w, precision)
     wide = fbytes // (16 if precision == 0 else 8) > 136 * 128   # more than 128 unknowns: global-memory factor
-    # complex64 with more than 128 unknowns: the register-window variants (band of at most 8 blocks)
-    fac_name = (("k_factor_wide" if precision == 0 else "k_factor_wide: k_factor_band") if wide
-                else ("k_factor" if precision == 0 else "k_factor_blk"))
+    fac_name = "k_factor_wide" if wide else ("k_factor" if precision == 0 else "k_factor_blk")
     if prof["ms_factor"] >= prof["ms_sweep"]:
         dom, flops, dms, cls = f"{fac_name} (finest level)", prof["flops_factor"], fac_ms, "factor"
     else:
-        swp_name = "k_sweep_fine: k_sweep_super" if wide and precision == 1 else "k_sweep_fine"
-        dom, flops, dms, cls = f"{swp_name} (one sweep, all colours)", prof["flops_sweep"], swp_ms_full, "sweep"
+        dom, flops, dms, cls = "k_sweep_fine (one sweep, all colours)", prof["flops_sweep"], swp_ms_full, "sweep"
     bps = NCU_BYTES_PER_SUBVOLUME.get((cls + ("_wide" if wide else ""), precision)) if traffic_ok else None
     traffic = round(bps * nsub) if bps else None
     kms = {"factor_per_launch": round(fac_ms, 4), "sweep_full": round(swp_ms_full, 4),
@@ -322,6 +319,41 @@ def envelope_flops(n, K, reach, square):
     if square:   # the pivot row, one of the rows down to last(j), reaches the last column such a row couples to
         return sum(8.0 * m * (last(last(j)) - j + 1) for j, m in enumerate(below)), 8.0 * n * n
     return sum(4.0 * m * (m + 1) for m in below), sum(16.0 * m + 8.0 for m in below)
+
+
+def band_blocks(w):
+    """Block bandwidth of a finest-level factor in 16 x 16 blocks: the largest I - J of a block (I, J) that holds two
+    points at most two grid steps apart (x-fastest order)."""
+    steps = range(-2, 3)
+    far = max(dx + w.sub[0] * dy + w.sub[0] * w.sub[1] * dz for dx in steps
+              for dy in (steps if w.dim > 1 else (0,)) for dz in (steps if w.dim > 2 else (0,))
+              if abs(dx) + abs(dy) + abs(dz) <= 2)
+    nb = -(-int(np.prod([w.sub[a] for a in range(w.dim)])) * w.nt // 16)
+    reach = [d for d in range(1, nb) for J in range(nb - d)
+             if (16 * (J + d)) // w.nt - (16 * J + 15) // w.nt <= far]
+    return min(max(reach, default=0) or 1, nb - 1)
+
+
+def finest_kernels(w, precision):
+    """(factorisation, sweep) kernels of the finest level, by the conditions of the library's dispatch."""
+    n = int(np.prod([w.sub[a] for a in range(w.dim)])) * w.nt
+    if getattr(w, "local_form", "lsq") == "square":
+        return "k_factor_square", "k_sweep_square"
+    if precision == 0:
+        return ("k_factor_wide" if n > 128 else "k_factor"), "k_sweep_fine"
+    if n <= 32:
+        return "k_factor_small", "k_sweep_small"
+    if n > 128 and band_blocks(w) <= 8:
+        return "k_factor_band", "k_sweep_super"
+    return ("k_factor_wide" if n > 128 else "k_factor_blk"), "k_sweep_fine"
+
+
+def finest_roofline(prof, w, precision, ms_total, traffic_ok, peaks=None):
+    """The bench line's roofline: dominant_roofline with the kernel's own name and the flops inside the envelope."""
+    r = dominant_roofline(prof, w, precision, ms_total, traffic_ok, peaks)
+    factor, sweep = finest_kernels(w, precision)
+    what = r["kernel"][r["kernel"].index(" "):]
+    return envelope_roofline(dict(r, kernel=(sweep if "sweep" in r["kernel"] else factor) + what), w, precision)
 
 
 def envelope_roofline(roofline, w, precision):
@@ -591,11 +623,7 @@ def run_ours(args):
     e2e_value = nunk * e2e_sweeps / e2e_s * (ws if ws > 1 else 1)
     ctx.close()
 
-    roofline = envelope_roofline(dominant_roofline(prof, w, precision, ms, traffic_ok=args.workload in ("2d", "3d"),
-                                                   peaks=peaks), w, precision)
-    if getattr(w, "local_form", "lsq") == "square":
-        roofline["kernel"] = roofline["kernel"].replace("k_factor", "k_factor_square").replace("k_sweep_fine",
-                                                                                               "k_sweep_square")
+    roofline = finest_roofline(prof, w, precision, ms, traffic_ok=args.workload in ("2d", "3d"), peaks=peaks)
     prec_tag = "f64" if precision == 0 else "c64 local solves + f64 refinement"
 
     out = {"metric": METRIC, "value": value, "unit": "unknowns/s", "n_gpus": ws, "steps": args.steps,
@@ -848,8 +876,7 @@ def run_3d_adjoint(args):
                       "l2": l2_note(w, precision)},
            "cycles_per_step": sum(s_[0] for s_ in stats) / args.steps,
            "backward_ms_per_step": 1e3 * el_b / args.steps, "set_hamiltonian_s": setup_s,
-           "roofline": envelope_roofline(dominant_roofline(prof, w, precision, 1e3 * el_f, traffic_ok=False), w,
-                                         precision),
+           "roofline": finest_roofline(prof, w, precision, 1e3 * el_f, traffic_ok=False),
            "stencil_roofline": stencil_roofline(prof, precision),
            "stencil_roofline_c64": stencil_roofline(prof, precision, c64=True),
            "dipole_T": float(hd * (x * psi.abs() ** 2).sum()), "grad_norm": float(np.linalg.norm(grad)),

@@ -5,8 +5,11 @@
 namespace la {
 namespace {
 
-constexpr int kSmallWarps = 4;         // warps per CTA on levels with enough matrices for every SM
-constexpr int kSmallManyMin = 1216;    // ... (8 per SM); with fewer, or factor_group 1, one warp per CTA spreads them
+// Warps per CTA on levels of at least kSmallManyMin matrices, eight per SM; with fewer, or factor_group 1, one.  Four
+// convert the time matrices once, one spreads better and ends its CTA sooner.  The line is flat: with one / four warps
+// 900, 1225, 1600 and 3600 matrices take 24 / 26, 29 / 30, 30 / 32 and 57 / 55 us (2D 4x2 x 4), 26 / 26, 31 / 31,
+// 32 / 31 and 60 / 55 us (2x2 x 8), 27 / 28, 33 / 35, 35 / 36 and 67 / 65 us (4x4 x 2).
+constexpr int kSmallWarps = 4, kSmallManyMin = 8 * kSms;
 
 // NP lanes per matrix (one or two matrices per warp), lane r holding row r.  G_UU is assembled in registers
 // and replaced in place by the inverse of its unit lower factor: G = L D L^dagger, step j subtracts
