@@ -46,9 +46,9 @@ METRIC = "spacetime unknowns relaxed/s"
 # - 3D 128^3 complex64: one k_factor_band launch (32768 subvolumes of 256 unknowns) and one full k_sweep_super
 #   sweep (eight colour launches of 4096), profiles/dram_3d_hydrogen_128x128x128_mixed.md
 NCU_BYTES_PER_SUBVOLUME = {("factor", 0): (772608 + 286944000) / 4096,
-                           ("sweep", 0): (330939648 + 530432) / 4096,
+                           ("sweep", 0): (330927104 + 286720) / 4096,
                            ("factor_wide", 1): (19604992 + 7257668864) / 32768,
-                           ("sweep_wide", 1): (9965988608 + 61851392) / 32768}
+                           ("sweep_wide", 1): (9973023232 + 62259712) / 32768}
 FP64_PEAK_TFLOPS = 152 * 4 * 2070e6 / 1e12   # 152 SMs x 4 FP64 flop/clk/SM x 2070 MHz (derived)
 FP32_PEAK_TFLOPS = 152 * 256 * 2070e6 / 1e12  # 152 SMs x 128 FP32 lanes x 2 flop (FMA) x 2070 MHz (derived)
 L2_BYTES = 129 * 2 ** 20

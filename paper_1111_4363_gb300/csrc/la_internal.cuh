@@ -189,7 +189,7 @@ struct LevelGeom {
   // x and y extents of U + 2 (c box), U + 1 (footprint) and U (1 on unused axes)
   FastDiv fd_K, fd_c[2], fd_f[2], fd_u[2];
   FastDiv fd_pair;   // Galerkin levels: stencil values per point, 9 pairs x the radius-2 box
-  // launch this level's sweeps, residuals and transfers so that a kernel may start before the one it follows has
+  // launch this level's sweeps, residuals and restrictions so that a kernel may start before the one it follows has
   // finished (programmatic dependent launch); off inside conditional graph bodies
   int overlap;
   int one_per_cta;   // factorise one subvolume matrix per CTA (no packing of small matrices)
@@ -487,7 +487,8 @@ cudaError_t launch_sweep_coarse(const LevelGeom& L, const R* sigma, const TimeMa
 // into non-coherent loads (ld.global.nc) that overlap_wait does not order; the coherent loads cost nothing measurable
 // here.  It hides the launch latency and the constant loads of the many short kernels of a complex64 V-cycle.
 // A launch of more than `max_ctas` CTAs goes out in the ordinary way: it is not bound by its latency, and early
-// successors take its issue slots (3D 128^3 mixed: 124.2 ms with these lines, 127.5 ms with every launch overlapped).
+// successors take its issue slots (3D 128^3 mixed, three steps: 123.9 ms with these lines, 127.5 ms with every launch
+// overlapped).
 // Where the lines lie, one step of 3 cycles in mixed precision, K = 4 unless given, plain / overlapped:
 // - kOverlapSweep, one CTA per SM, for finest sweeps of more than 32 unknowns, whose CTAs work longest.  3D 4x4x4 on
 //   32^3 (64 CTAs a colour) 2.76 / 2.55 ms, 40^3 (125) 3.26 / 3.19 ms, 48^3 (216) 3.83 / 4.13 ms; 4x4x2 on 36^3
