@@ -11,6 +11,27 @@ namespace {
 // 32 / 31 and 60 / 55 us (2x2 x 8), 27 / 28, 33 / 35, 35 / 36 and 67 / 65 us (4x4 x 2).
 constexpr int kSmallWarps = 4, kSmallManyMin = 8 * kSms;
 
+// The entries of H and H^2 that only the spacings enter, w_a = 1 / (2 h_a^2): w_a, w_a^2 and 2 sum w_a^2 (a point's
+// neighbours away from the walls) in FP64, and rounded once w_a, w_a^2 and 2 w_x w_y, 2 w_x w_z, 2 w_y w_z.
+struct SpacingWeights {
+  double w[3], w2[3], inner;
+  float f[3], f2[3], fxy, fxz, fyz;
+};
+inline SpacingWeights spacing_weights(const FineOp& g) {
+  SpacingWeights s;
+  for (int a = 0; a < 3; ++a) {
+    s.w[a] = 0.5 * g.ih2[a];
+    s.w2[a] = s.w[a] * s.w[a];
+    s.f[a] = (float)s.w[a];
+    s.f2[a] = (float)s.w2[a];
+  }
+  s.inner = 2.0 * (s.w2[0] + s.w2[1] + s.w2[2]);
+  s.fxy = (float)(2.0 * s.w[0] * s.w[1]);
+  s.fxz = (float)(2.0 * s.w[0] * s.w[2]);
+  s.fyz = (float)(2.0 * s.w[1] * s.w[2]);
+  return s;
+}
+
 // NP lanes per matrix (one or two matrices per warp), lane r holding row r.  G_UU is assembled in registers
 // and replaced in place by the inverse of its unit lower factor: G = L D L^dagger, step j subtracts
 // (a_rj / d_j) u from the rows r > j, where u_c = conj(a_cj) for the columns c > j still to eliminate and u_c = row j
@@ -19,20 +40,24 @@ constexpr int kSmallWarps = 4, kSmallManyMin = 8 * kSms;
 // loop rolled without a dynamic register index; u passes through shared memory, 16 bytes a load.
 // H and H^2 of a finest-level point pair are formed in FP64 and rounded once (D_i + D_j may cancel), as the larger
 // shared-memory factorisations do.  No barrier but the warp's: 7200 matrices of 32 unknowns (8 points x 4) take
-// 97 us (96 us with the pairs in FP32), half of the issue slots busy, against 161 us for four matrices per
+// 96 us (the same with the pairs in FP32), half of the issue slots busy, against 161 us for four matrices per
 // 256-thread CTA with two barriers per column.
 template <int NP, int K, bool FINE>
 __global__ void __launch_bounds__(32 * kSmallWarps)
-k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const TimeMats* __restrict__ tm,
-               float2* __restrict__ factors, int* __restrict__ status) {
+k_factor_small(LevelGeom L, FineOp g, SpacingWeights sw, const float* __restrict__ sigma,
+               const TimeMats* __restrict__ tm, float2* __restrict__ factors, int* __restrict__ status) {
   constexpr int KK = K * K, JMAX = NP / K;   // points of a full subvolume of this size class, at most
   __shared__ float sP[LA_NPAIR * KK], sPd[2 * KK];
-  // FINE: D = dsum + V0 and the in-grid neighbours' weights of H^2's diagonal per point, and (H, H^2) of the point pairs
-  // i >= j of each matrix
+  // FINE, per point: D = dsum + V0; the entries that D enters, rounded from FP64: H and H^2 on the diagonal, H^2 of the
+  // links to the lower neighbours in the subvolume along x, y, z
+  __shared__ double sD[kSmallWarps][FINE ? 32 : 1];
+  __shared__ float sE[kSmallWarps][5][FINE ? 32 : 1], sX[kSmallWarps][32];
+  // (H, H^2) of the point pairs i >= j, which K rows each look up: a table from K = 4 on, below that formed where they
+  // are used (4000 matrices, K = 4 with 8 points: 59 us, 67 us without a table; 576, K = 3 with 8 points: 21.7 us,
+  // 23.1 us with one; 4000, K = 1 with 32 points: 72 us, 86 us with one)
+  constexpr bool kTable = FINE && K >= 4;
   constexpr int NPAIR = JMAX * (JMAX + 1) / 2;
-  __shared__ double sD[kSmallWarps][FINE ? 32 : 1], sN[kSmallWarps][FINE ? 32 : 1];
-  __shared__ float2 sHH[kSmallWarps][FINE ? (32 / NP) * NPAIR : 1];
-  __shared__ float sX[kSmallWarps][32];
+  __shared__ float2 sHH[kSmallWarps][kTable ? (32 / NP) * NPAIR : 1];
   __shared__ int sXYZ[kSmallWarps][32];
   __shared__ __align__(16) float2 sBuf[kSmallWarps][2][32];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, r = lane & (NP - 1), half = lane / NP;
@@ -44,7 +69,6 @@ k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const Tim
     subvol_box(L, b, o, e);
     npts = e[0] * e[1] * e[2];
   }
-  const double wx = 0.5 * g.ih2[0], wy = 0.5 * g.ih2[1], wz = 0.5 * g.ih2[2];
   const int s0 = half * NP;
   if (r < npts) {
     int lx, ly, lz;
@@ -54,9 +78,6 @@ k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const Tim
       const int px = o[0] + lx, py = o[1] + ly, pz = o[2] + lz;
       sD[w][s0 + r] = g.dsum + g.V0[(pz * g.n[1] + py) * g.n[0] + px];
       sX[w][s0 + r] = (float)fine_x(g, px, py, pz);
-      const int cx = (px > 0 ? 1 : 0) + (px + 1 < g.n[0] ? 1 : 0), cy = (py > 0 ? 1 : 0) + (py + 1 < g.n[1] ? 1 : 0),
-                cz = (pz > 0 ? 1 : 0) + (pz + 1 < g.n[2] ? 1 : 0);
-      sN[w][s0 + r] = wx * wx * cx + wy * wy * cy + wz * wz * cz;
     }
   }
   __syncthreads();
@@ -64,20 +85,46 @@ k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const Tim
     sPd[i] = sP[KK + i] - sP[3 * KK + i];
     sPd[KK + i] = sP[2 * KK + i] - sP[6 * KK + i];
   }
-  if (FINE) {
-    // once per pair over the matrix's lanes: the FP64 pipe takes a warp's instruction 16 cycles, whoever of it is active
+  if (FINE && r < npts) {   // one point per lane: the FP64 pipe takes a warp's instruction 16 cycles, whoever is active
+    const int x = sXYZ[w][s0 + r], l3[3] = {x & 255, (x >> 8) & 255, x >> 16}, below[3] = {1, e[0], e[0] * e[1]};
+    const double D = sD[w][s0 + r];
+    double d2 = fma(D, D, sw.inner);   // less w_a^2 for each neighbour beyond a Dirichlet wall; unused axes have w = 0
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int p = o[a] + l3[a];
+      if (a < g.dim && p == 0) d2 -= sw.w2[a];
+      if (a < g.dim && p + 1 == g.n[a]) d2 -= sw.w2[a];
+      if (l3[a] > 0) sE[w][2 + a][s0 + r] = (float)(-sw.w[a] * (D + sD[w][s0 + r - below[a]]));
+    }
+    sE[w][0][s0 + r] = (float)D;
+    sE[w][1][s0 + r] = (float)d2;
+  }
+  __syncthreads();
+  // (H, H^2) of points i and j <= i, (dx, dy, dz) apart: in x-fastest order a neighbour j is i's lower one on its axis
+  auto h_h2 = [&](int i, int dx, int dy, int dz) {
+    const int ax = abs(dx), ay = abs(dy), az = abs(dz), a1 = ax + ay + az;
+    if (a1 == 0) return make_float2(sE[w][0][s0 + i], sE[w][1][s0 + i]);
+    if (a1 == 1) return make_float2(ax ? -sw.f[0] : (ay ? -sw.f[1] : -sw.f[2]), sE[w][ax ? 2 : (ay ? 3 : 4)][s0 + i]);
+    float H2 = 0.f;
+    if (a1 == 2) {
+      H2 = ax ? (ay ? sw.fxy : sw.fxz) : sw.fyz;
+      if (ax == 2) H2 = sw.f2[0];
+      if (ay == 2) H2 = sw.f2[1];
+      if (az == 2) H2 = sw.f2[2];
+    }
+    return make_float2(0.f, H2);
+  };
+  if constexpr (kTable) {
     for (int p = r; p < npts * (npts + 1) / 2; p += NP) {
       int a = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
       while (a * (a + 1) / 2 > p) --a;
       while ((a + 1) * (a + 2) / 2 <= p) ++a;
-      const int q = p - a * (a + 1) / 2, xa = sXYZ[w][s0 + a], xq = sXYZ[w][s0 + q];
-      double H, H2;
-      wide_h_h2<double>((xq & 255) - (xa & 255), ((xq >> 8) & 255) - ((xa >> 8) & 255), (xq >> 16) - (xa >> 16),
-                        sD[w][s0 + a], sD[w][s0 + q], sN[w][s0 + a], wx, wy, wz, H, H2);
-      sHH[w][half * NPAIR + p] = make_float2((float)H, (float)H2);
+      const int xa = sXYZ[w][s0 + a], xq = sXYZ[w][s0 + p - a * (a + 1) / 2];
+      sHH[w][half * NPAIR + p] =
+          h_h2(a, (xq & 255) - (xa & 255), ((xq >> 8) & 255) - ((xa >> 8) & 255), (xq >> 16) - (xa >> 16));
     }
+    __syncwarp();
   }
-  __syncthreads();
   // row r = (point i, time function m)
   const int i = r / K, m = r - i * K;
   const bool row_in = i < npts;
@@ -101,8 +148,9 @@ k_factor_small(LevelGeom L, FineOp g, const float* __restrict__ sigma, const Tim
       const int xj = sXYZ[w][s0 + j];
       const int dx = (xj & 255) - ix, dy = ((xj >> 8) & 255) - iy, dz = (xj >> 16) - iz;
       if (FINE) {
-        const float2 hh = sHH[w][half * NPAIR + i * (i + 1) / 2 + j];
-        const float H = hh.x, H2 = hh.y, Xj = sX[w][s0 + j];
+        const float2 hh = kTable ? sHH[w][kTable ? half * NPAIR + i * (i + 1) / 2 + j : 0] : h_h2(i, dx, dy, dz);
+        const float H = hh.x, H2 = hh.y;
+        const float Xj = sX[w][s0 + j];
 #pragma unroll
         for (int n = 0; n < K; ++n) {
           const int mn = m * K + n;
@@ -182,8 +230,12 @@ cudaError_t launch_k(const LevelGeom& L, const FineOp* fine, const float* sigma,
                      int* status, cudaStream_t s) {
   const int warps = L.nsub >= kSmallManyMin && !L.one_per_cta ? kSmallWarps : 1, per = warps * (32 / NP);
   const int grid = (L.nsub + per - 1) / per;
-  if (fine) k_factor_small<NP, K, true><<<grid, 32 * warps, 0, s>>>(L, *fine, sigma, tm, factors, status);
-  else k_factor_small<NP, K, false><<<grid, 32 * warps, 0, s>>>(L, FineOp{}, sigma, tm, factors, status);
+  if (fine) {
+    k_factor_small<NP, K, true><<<grid, 32 * warps, 0, s>>>(L, *fine, spacing_weights(*fine), sigma, tm, factors,
+                                                            status);
+  } else {
+    k_factor_small<NP, K, false><<<grid, 32 * warps, 0, s>>>(L, FineOp{}, SpacingWeights{}, sigma, tm, factors, status);
+  }
   return cudaGetLastError();
 }
 }  // namespace
