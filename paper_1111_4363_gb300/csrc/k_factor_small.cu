@@ -54,7 +54,7 @@ k_factor_small(LevelGeom L, FineOp g, SpacingWeights sw, const float* __restrict
   __shared__ float sE[kSmallWarps][5][FINE ? 32 : 1], sX[kSmallWarps][32];
   // (H, H^2) of the point pairs i >= j, which K rows each look up: a table from K = 4 on, below that formed where they
   // are used (4000 matrices, K = 4 with 8 points: 59 us, 67 us without a table; 576, K = 3 with 8 points: 21.7 us,
-  // 23.1 us with one; 4000, K = 1 with 32 points: 72 us, 86 us with one)
+  // 23.1 us with one; 4000, K = 1 with 32 points: 72 us, 86 us with a table of entries formed in FP64 pair by pair)
   constexpr bool kTable = FINE && K >= 4;
   constexpr int NPAIR = JMAX * (JMAX + 1) / 2;
   __shared__ float2 sHH[kSmallWarps][kTable ? (32 / NP) * NPAIR : 1];
